@@ -333,15 +333,17 @@ int aenet_neighbor_stats(aenet_ctx *ctx, int64_t out[3]);
  * forces run as one fused kernel (the FP32 form with hidden widths <= 32),
  * whose time is then all reported under "forces" (descriptor and network read
  * ~0), and AENET_PATH_PIPELINED when that kernel ran in its pipelined form
- * (AENET_OPT_PIPELINE), and AENET_PATH_LIST when the step built the exact
- * neighbour list in every step (AENET_OPT_MD_LIST; the list build is then
- * reported under "cell sort" and the list-driven potential kernel under
- * "forces"). Any output pointer except ms may be NULL. Returns
+ * (AENET_OPT_PIPELINE), AENET_PATH_LIST when the step takes the list form of
+ * AENET_OPT_MD_LIST, and AENET_PATH_ROWS when the step built exact neighbour
+ * lists and ran the list-driven potential kernel over them, as aenet_compute
+ * does (the list build is then reported under "cell sort" and the potential
+ * kernel under "forces"). Any output pointer except ms may be NULL. Returns
  * AENET_E_STATE if no timed step has run. Synchronises.
  */
 #define AENET_PATH_FUSED 1
 #define AENET_PATH_PIPELINED 2
 #define AENET_PATH_LIST 4
+#define AENET_PATH_ROWS 8
 int aenet_md_stage_times(aenet_ctx *ctx, float ms[6], int *kernels_per_step, int *path_flags);
 
 /*
@@ -421,13 +423,12 @@ int aenet_descriptors_noalloc(int n_atoms, const double *pos, const int32_t *typ
  * atom itself at zero shift excluded) are found in every step either by the
  * fused potential kernel itself from the staged cells (OFF) or by a list
  * kernel that writes each atom's exact list after the binning, which the
- * list-driven potential kernel then reads (ON; the Verlet-list machinery with
- * no skin and no rebuild test). The same pairs enter the same arithmetic, so
- * the two agree to FP32 rounding order. AUTO takes ON for every basis except
- * angular order 6 with radial order 20 (its spherical-harmonic angular sum
- * runs faster in the fused kernel). Other evaluations (aenet_compute and the
- * batch calls) always use the fused kernel. A change re-captures the MD step.
- * Other values give AENET_E_ARG.
+ * list-driven potential kernel then reads (ON). The same pairs enter the same
+ * sums, so the two agree to FP32 rounding order. AUTO takes ON for every basis
+ * except angular order 6 with radial order 20, whose steps evaluate as
+ * aenet_compute does: over lists as well (AENET_PATH_ROWS). aenet_compute
+ * builds its lists in every call, whatever this option says. A change
+ * re-captures the MD step. Other values give AENET_E_ARG.
  */
 #define AENET_OPT_MD_LIST 4
 #define AENET_MD_LIST_AUTO 0

@@ -163,6 +163,8 @@ struct Context {
     bool own_stream = false;
     int precision = AENET_FP32;
     bool fuse_network = true;      // BF16 forms: tensor-core network inside the fused kernel
+    bool batch_call = false;       // set during the batch entry points
+    bool cell_search = false;      // set while an MD step with AENET_MD_LIST_OFF is enqueued
     bool pipeline = false;         // FP32 fused form: the pipelined kernel (one CTA of 16 warps per SM)
     Basis basis{};
     Net net{};
@@ -243,7 +245,8 @@ struct Context {
     // MD steps without a skin: AENET_MD_LIST_AUTO (0), _OFF (1: the fused kernel searches the cells
     // itself) or _ON (2: the exact list is built in every step and the list kernel evaluates it)
     int md_list = 0;
-    bool last_list = false;            // the captured MD step builds the exact list in every step
+    bool last_list = false;            // the captured MD step takes the list form of AENET_OPT_MD_LIST
+    bool last_rows = false;            // ... or builds lists in every step as aenet_compute does
     // tilt factors xy, xz, yz of the restricted triclinic cell of single-structure
     // calls (zero: orthorhombic)
     double tilt[3] = {0.0, 0.0, 0.0};
@@ -255,8 +258,17 @@ struct Context {
     double *d_vl_ref = nullptr;        // [atoms * 3] positions at the last build (input order)
     unsigned *d_vl_flag = nullptr;     // [2]: rebuild flag, last-CTA counter
     unsigned long long *d_vl_builds = nullptr;  // list builds so far
-    double *d_vl_epart = nullptr;      // [4 * SMs] energy partials of the list-mode kernel
-    double *d_vl_vpart = nullptr;      // [4 * SMs * 9] virial partials
+    // neighbour lists built for every evaluation (direct rows: displacement, index and species)
+    float4 *d_rows = nullptr;          // [atoms of a slice * caps.nb]
+    size_t cap_rows = 0;
+    int *d_list_count = nullptr;       // [atoms]
+    int cap_list = 0;
+    float *d_pnet = nullptr;           // network parameters packed in the list kernel's layout
+    float *d_vir_atom = nullptr;       // [atoms * 6] virial of every atom (batches)
+    int cap_vir_atom = 0;
+    int cap_parts = 0;
+    double *d_vl_epart = nullptr;      // [SMs * slices] energy partials of the list kernel
+    double *d_vl_vpart = nullptr;      // [SMs * slices * 9] virial partials
     bool vl_valid = false;             // list, origins and cell maps describe the MD state
     cudaStream_t aux_stream = nullptr; // captures the body of the rebuild conditional
     int maps_n = -1;                   // atoms of the evaluation that last wrote the cell maps
@@ -424,6 +436,10 @@ bool tc_fused_supported(const Context &c);
 cudaError_t launch_fused_tc(Context &c, const Grid &g, int n);
 // Either fused form: descriptor, networks and forces in one kernel.
 inline bool fused_path(const Context &c) { return fused_supported(c) || tc_fused_supported(c); }
+// Whether evaluations take that form: the FP32 fused form of one structure,
+// except for the pipelined kernel and MD steps asked to search the cells in the
+// fused kernel.
+inline bool rows_form(const Context &c) { return fused_supported(c) && !c.pipeline && !c.cell_search && !c.batch_call; }
 int ann_blocks(int n);
 
 // Forces to input order (FP64) only.
@@ -455,13 +471,27 @@ cudaError_t launch_md_vl_kick_drift(Context &c, int n, double dt, double *pos, d
 // Rebuild, part 1: bin the current positions, record each atom's origin and
 // reference position (then launch_sort and launch_vl_build).
 cudaError_t launch_md_vl_bin(Context &c, const Grid &g, int n, const double *pos, const int32_t *types);
-// Rebuild, part 2: the Verlet list of every atom (k_potential, list-build mode).
+// Rebuild, part 2: the Verlet list of every atom (k_list_build, code rows).
 cudaError_t launch_vl_build(Context &c, const Grid &g, int n);
 // The fused potential over the Verlet list (persistent CTAs, atoms from a
 // counter); sets c.last_* to its partials.
 cudaError_t launch_potential_list(Context &c, const Grid &g, int n);
-// Largest CTA count of launch_potential_list (sizes its partial buffers).
+// Largest CTA count of a list-kernel launch (sizes its partial buffers).
 int potential_list_max_ctas(const Context &c);
+// Evaluation over lists built for it, for the sorted atoms [a_lo, a_hi) (slices
+// of list_slice(c, n) atoms): the list build (direct rows) and the list kernel.
+// The first build also clears the forces and statistics unless c.md_prezeroed;
+// the kernel appends its partial rows after *parts and sets c.last_*.
+int list_slice(const Context &c, int n);
+cudaError_t launch_rows_build(Context &c, const Grid &g, int n, int a_lo, int a_hi);
+// What the list kernel evaluates: everything, the G rows (c.d_G) only, or forces
+// and virial from given dE/dG rows (c.d_dEdG).
+enum class RowsMode { fused, descriptor, forces };
+cudaError_t launch_rows_potential(Context &c, const Grid &g, RowsMode mode, int a_lo, int a_hi, int *parts);
+// Network parameters into the list kernel's layout (c.d_pnet), on c.stream.
+cudaError_t pack_list_net(Context &c);
+// Dynamic shared memory of one list CTA of a single warp (what must fit).
+size_t list_smem_bytes(const Context &c);
 
 // Message reported by aenet_last_error(NULL) for calls made without a context.
 void set_context_free_error(const char *msg);

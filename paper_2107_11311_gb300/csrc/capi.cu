@@ -193,11 +193,43 @@ int ensure_stage(Context &c, int n) {
     return AENET_OK;
 }
 
+// Partial rows of `launches` launches of the list kernel.
+int ensure_parts(Context &c, int launches) {
+    const int P = potential_list_max_ctas(c) * std::max(1, launches);
+    if (P > c.cap_parts || !c.d_vl_epart) {
+        CK(grow(c.d_vl_epart, 0, (size_t)P), "cudaMalloc");
+        CK(grow(c.d_vl_vpart, 0, 9 * (size_t)P), "cudaMalloc");
+        c.cap_parts = P;
+        ++c.buf_gen;
+    }
+    return AENET_OK;
+}
+
+// Buffers of the evaluation over direct rows for n atoms with the capacities c.caps.
+int ensure_rows(Context &c, int n) {
+    const int slice = list_slice(c, n);
+    const size_t need = (size_t)slice * c.caps.nb;
+    if (need > c.cap_rows || !c.d_rows) {
+        c.cap_rows = 0;
+        CK(grow(c.d_rows, 0, need), "cudaMalloc");
+        c.cap_rows = need;
+        ++c.buf_gen;
+    }
+    if (n > c.cap_list || !c.d_list_count) {
+        CK(grow(c.d_list_count, 0, (size_t)std::max(n, 1)), "cudaMalloc");
+        c.cap_list = std::max(n, 1);
+        ++c.buf_gen;
+    }
+    return ensure_parts(c, (std::max(n, 1) + slice - 1) / slice);
+}
+
 int check_smem(Context &c, const Grid &g) {
     int dev = 0, optin = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    const size_t need = potential_smem_bytes(c, g) + 1024;  // + the kernel's static shared memory
+    // + the kernel's static shared memory
+    const bool rows = rows_form(c) || (!fused_path(c) && !c.batch_call);
+    const size_t need = rows ? list_smem_bytes(c) + 4096 : potential_smem_bytes(c, g) + 1024;
     if (optin > 0 && need > (size_t)optin)
         return fail(&c, AENET_E_CAPACITY, "neighbour lists need %zu B of shared memory (limit %d B)", need, optin);
     return AENET_OK;
@@ -211,11 +243,36 @@ cudaError_t mark(Context &c, int k) {
     return cudaEventRecordWithFlags(c.ev[k], c.stream, cudaEventRecordExternal);
 }
 
+// List build and list kernel over direct rows, with stage events 2, 3 and 4
+// between them when selected. The forces of the split path follow its
+// descriptors: with a single slice their rows are still in place.
+int enqueue_rows(Context &c, const Grid &g, int n, RowsMode mode) {
+    int rc = ensure_rows(c, n);
+    if (rc) return rc;
+    const int slice = list_slice(c, n);
+    int parts = 0;
+    for (int a0 = 0; a0 < std::max(n, 1); a0 += slice) {
+        const int a1 = std::min(n, a0 + slice);
+        if (mode != RowsMode::forces || slice < n) CK(launch_rows_build(c, g, n, a0, a1), "neighbour list");
+        if (a0 == 0 && mode == RowsMode::fused) {
+            CK(mark(c, 2), "event");
+            CK(mark(c, 3), "event");
+            CK(mark(c, 4), "event");
+        }
+        CK(launch_rows_potential(c, g, mode, a0, a1, &parts), "potential kernel (neighbour list)");
+    }
+    return AENET_OK;
+}
+
 // Descriptor, networks and forces after the cell list (fused kernel or the
 // three split kernels), with stage events 3, 4 (after descriptor, network) and
 // 5 (after forces) when selected. *n_eparts = number of energy partials written.
 int enqueue_potential(Context &c, const Grid &g, int n, int *n_eparts) {
-    if (fused_path(c)) {
+    if (rows_form(c)) {
+        const int rc = enqueue_rows(c, g, n, RowsMode::fused);
+        if (rc) return rc;
+        *n_eparts = c.pot_parts;
+    } else if (fused_path(c)) {
         // descriptor, network and forces in one kernel: their stage events coincide
         CK(mark(c, 3), "event");
         CK(mark(c, 4), "event");
@@ -229,7 +286,12 @@ int enqueue_potential(Context &c, const Grid &g, int n, int *n_eparts) {
         c.last_vpart = c.d_vir_part;
         c.last_vparts = c.pot_parts;
     } else {
-        CK(launch_fp_forward(c, g, n), "descriptor kernel");
+        const bool rows = !c.batch_call;
+        int rc = AENET_OK;
+        if (!rows)
+            CK(launch_fp_forward(c, g, n), "descriptor kernel");
+        else if ((rc = enqueue_rows(c, g, n, RowsMode::descriptor)))
+            return rc;
         CK(mark(c, 3), "event");
         if (c.precision == AENET_FP32) {
             CK(launch_ann(c, n), "network kernel");
@@ -239,11 +301,15 @@ int enqueue_potential(Context &c, const Grid &g, int n, int *n_eparts) {
             *n_eparts = tcgen05_eparts(c, n);
         }
         CK(mark(c, 4), "event");
-        CK(launch_fp_backward(c, g, n), "force kernel");
+        if (!rows) {
+            CK(launch_fp_backward(c, g, n), "force kernel");
+            c.last_vpart = c.d_vir_part;
+            c.last_vparts = c.pot_parts;
+        } else if ((rc = enqueue_rows(c, g, n, RowsMode::forces))) {
+            return rc;
+        }
         c.last_epart = c.d_e_part;
         c.last_eparts = *n_eparts;
-        c.last_vpart = c.d_vir_part;
-        c.last_vparts = c.pot_parts;
     }
     c.maps_n = n;          // the cell maps now describe this evaluation
     c.vl_valid = false;    // and no Verlet list matches them
@@ -423,6 +489,7 @@ extern "C" int aenet_setup(aenet_ctx **out, const aenet_model_desc *m, int preci
     if (precision != AENET_FP32) {
         if ((e = prepare_bf16_weights(c)) != cudaSuccess) return setup_fail(e, "BF16 weights");
     }
+    if (fused_supported(c) && (e = pack_list_net(c)) != cudaSuccess) return setup_fail(e, "network parameters");
     {
         const std::vector<int2> pairs = grad_pairs(c.net);
         if ((e = cudaMalloc(&c.d_wpairs, sizeof(int2) * pairs.size())) != cudaSuccess ||
@@ -473,7 +540,7 @@ static int compute_impl(Context &c, int n, const double *pos, const int32_t *typ
         if (G_out) {
             if ((rc = check_smem(c, g))) return rc;
             CK(launch_cells(c, g, n, dpos, dtypes), "cell list");
-            CK(launch_fp_forward(c, g, n), "descriptor kernel");
+            if ((rc = enqueue_rows(c, g, n, RowsMode::descriptor))) return rc;
         } else {
             if ((rc = enqueue_compute(c, g, n, dpos, dtypes, dF, dE))) return rc;
         }
@@ -554,6 +621,13 @@ extern "C" int aenet_compute_async(aenet_ctx *h, int n, const double *pos, const
 // global cell index space; one launch of each kernel over all cells.
 namespace aenet {
 namespace {
+
+// A batch call is in progress (rows_form).
+struct BatchCall {
+    Context &c;
+    explicit BatchCall(Context &ctx) : c(ctx) { c.batch_call = true; }
+    ~BatchCall() { c.batch_call = false; }
+};
 
 struct BatchLayout {
     std::vector<StructInfo> info;  // per structure
@@ -665,6 +739,7 @@ extern "C" int aenet_compute_batch(aenet_ctx *h, int n_struct, const int64_t *at
                                    double *virials) {
     if (!h) return fail(nullptr, AENET_E_ARG, "ctx is NULL");
     Context &c = h->c;
+    BatchCall in_batch(c);
     cudaGetLastError();
     BatchLayout L;
     int rc = batch_layout(c, n_struct, atom_offset, boxes, L);
@@ -782,6 +857,7 @@ extern "C" int aenet_batch_prepare(aenet_ctx *h, int n_struct, const int64_t *at
                                    double *virials, int flags) {
     if (!h) return fail(nullptr, AENET_E_ARG, "ctx is NULL");
     Context &c = h->c;
+    BatchCall in_batch(c);
     cudaGetLastError();
     c.plan.valid = false;
     if (c.batch_exec) cudaGraphExecDestroy(c.batch_exec);
@@ -899,6 +975,7 @@ extern "C" int aenet_batch_prepare(aenet_ctx *h, int n_struct, const int64_t *at
 extern "C" int aenet_batch_run(aenet_ctx *h) {
     if (!h) return fail(nullptr, AENET_E_ARG, "ctx is NULL");
     Context &c = h->c;
+    BatchCall in_batch(c);
     cudaGetLastError();
     if (!c.plan.valid || !c.batch_exec) return fail(&c, AENET_E_STATE, "no prepared batch");
     if (c.plan.gen != c.buf_gen || c.plan.stream != c.stream || c.plan.caps.nb != c.caps.nb ||
@@ -952,37 +1029,29 @@ static bool md_list_form(const Context &c) {
     return !(c.basis.Kr == 21 && c.basis.Ka == 7);
 }
 
-// One MD step on device buffers: kick + drift + binning, cell sort (and, in the
-// list form, the neighbour-list build), forces at the new positions, closing
-// kick with the FP64 reductions (and the record of (E_pot, E_kin) when rec !=
-// NULL). With timing, events bracket the 6 stages.
+// One MD step on device buffers: kick + drift + binning, cell sort, forces at the
+// new positions (rows: over lists built in the step, else the fused kernel's own
+// cell search), closing kick with the FP64 reductions (and the record of (E_pot,
+// E_kin) when rec != NULL). With timing, events bracket the 6 stages; the list
+// build is part of the cell sort's.
 static int enqueue_md_step(Context &c, const Grid &g, int n, double dt, double *pos, double *vel,
-                           const int32_t *types, double *rec, bool list_form) {
+                           const int32_t *types, double *rec, bool rows) {
+    c.cell_search = !rows;
     int rc = check_smem(c, g);
+    c.cell_search = false;
     if (rc) return rc;
     CK(mark(c, 0), "event");
     CK(launch_md_kick_drift_bin(c, g, n, dt, pos, vel, types), "kick + drift + binning + scan");
     CK(mark(c, 1), "event");
     CK(launch_scatter(c, n), "cell sort");
-    // list form: every image-atom within rc_max of each atom, from this step's
-    // cells, into the atom's list row (the list kernel of the Verlet path)
-    if (list_form) CK(launch_vl_build(c, g, n), "neighbour list");
-    CK(mark(c, 2), "event");
-    if (list_form) {
-        CK(mark(c, 3), "event");
-        CK(mark(c, 4), "event");
-        c.md_prezeroed = true;  // the kick + drift kernel cleared the forces and statistics
-        const cudaError_t pe = launch_potential_list(c, g, n);
-        c.md_prezeroed = false;
-        CK(pe, "potential kernel (neighbour list)");
-        CK(mark(c, 5), "event");
-    } else {
-        int n_eparts = 0;
-        c.md_prezeroed = true;
-        rc = enqueue_potential(c, g, n, &n_eparts);
-        c.md_prezeroed = false;
-        if (rc) return rc;
-    }
+    c.cell_search = !rows;
+    if (!rows_form(c)) CK(mark(c, 2), "event");
+    int n_eparts = 0;
+    c.md_prezeroed = true;  // the kick + drift kernel cleared the forces and statistics
+    rc = enqueue_potential(c, g, n, &n_eparts);
+    c.md_prezeroed = false;
+    c.cell_search = false;
+    if (rc) return rc;
     CK(launch_md_kick_finish(c, n, dt, vel, types, rec, rec ? rec + c.cap_rec : nullptr), "kick + reductions");
     CK(mark(c, 6), "event");
     return AENET_OK;
@@ -1074,16 +1143,13 @@ static int ensure_verlet(Context &c, int n, const Grid &g) {
         ++c.buf_gen;
     }
     if (!c.d_vl_flag) {
-        const size_t P = (size_t)potential_list_max_ctas(c);
         CK(grow(c.d_vl_flag, 0, 2), "cudaMalloc");
         CK(grow(c.d_vl_builds, 0, 1), "cudaMalloc");
-        CK(grow(c.d_vl_epart, 0, P + 1), "cudaMalloc");
-        CK(grow(c.d_vl_vpart, 0, 9 * P + 9), "cudaMalloc");
         CK(cudaMemsetAsync(c.d_vl_flag, 0, 2 * sizeof(unsigned), c.stream), "cudaMemsetAsync");
         CK(cudaMemsetAsync(c.d_vl_builds, 0, sizeof(unsigned long long), c.stream), "cudaMemsetAsync");
         ++c.buf_gen;
     }
-    return AENET_OK;
+    return ensure_parts(c, 1);
 }
 
 // n_steps MD steps in one fixed cell (edges box, tilts c.tilt).
@@ -1124,12 +1190,12 @@ static int md_fixed_cell(aenet_ctx *h, int n, double *pos, double *vel, const in
     if ((rc = validate_types_host(c, n, types))) return rc;
     if ((rc = ensure(c, n, g)) || (rc = ensure_stage(c, n))) return rc;
     if (c.caps.nb == 0) c.caps = estimate_caps(c, n, g);
-    if (verlet || list_form) {
-        // the list form keeps a relative margin of 1e-5 over rc_max: its list is then a
-        // superset of the pairs within rc_max, which the list kernel selects exactly
-        c.caps.rc_list = (float)(verlet ? c.basis.rc_max + c.skin : c.basis.rc_max * 1.00001);
+    if (verlet) {
+        c.caps.rc_list = (float)(c.basis.rc_max + c.skin);
         if ((rc = ensure_verlet(c, n, g))) return rc;
     }
+    const bool rows = fused_supported(c) && !c.pipeline && c.md_list != AENET_MD_LIST_OFF;
+    if (rows && !verlet && (rc = ensure_rows(c, n))) return rc;
     double *dpos = pos_dev ? pos : c.d_pos;
     double *dvel = vel_dev ? vel : c.d_vel;
     const int32_t *dtypes = typ_dev ? types : c.d_types;
@@ -1191,7 +1257,7 @@ static int md_fixed_cell(aenet_ctx *h, int n, double *pos, double *vel, const in
             CK(cudaStreamBeginCapture(c.stream, cudaStreamCaptureModeThreadLocal), "begin capture");
             c.ev_mask = ev_mask;
             int src = verlet ? enqueue_md_step_verlet(c, g, n, dt, dpos, dvel, dtypes, rec)
-                             : enqueue_md_step(c, g, n, dt, dpos, dvel, dtypes, rec, list_form);
+                             : enqueue_md_step(c, g, n, dt, dpos, dvel, dtypes, rec, rows);
             c.ev_mask = 0u;
             cudaError_t ce = cudaStreamEndCapture(c.stream, &graph);
             if (src) {
@@ -1232,6 +1298,7 @@ static int md_fixed_cell(aenet_ctx *h, int n, double *pos, double *vel, const in
             c.md_key.skin = c.skin;
             c.md_key.list_form = list_form;
             c.last_list = list_form;
+            c.last_rows = rows && !verlet;
             c.md_key.thermo_T0 = c.thermo_T0;
             c.md_key.thermo_tau = c.thermo_tau;
         }
@@ -1380,7 +1447,7 @@ extern "C" int aenet_md_stage_times(aenet_ctx *h, float *ms, int *kernels_per_st
     if (kernels_per_step) *kernels_per_step = c.md_kernels;
     if (path_flags)
         *path_flags = (fused_path(c) ? AENET_PATH_FUSED : 0) | (c.last_pipe ? AENET_PATH_PIPELINED : 0) |
-                      (c.last_list ? AENET_PATH_LIST : 0);
+                      (c.last_list ? AENET_PATH_LIST : 0) | (c.last_rows ? AENET_PATH_ROWS : 0);
     return AENET_OK;
 }
 
@@ -1460,6 +1527,7 @@ extern "C" int aenet_set_params(aenet_ctx *h, const double *params) {
         CK(cudaMemcpy(c.d_params, P.data(), sizeof(float) * NP, cudaMemcpyHostToDevice), "cudaMemcpy");
     }
     if (c.precision != AENET_FP32) CK(prepare_bf16_weights(c), "BF16 weights");
+    if (c.d_pnet) CK(pack_list_net(c), "network parameters");
     c.act_valid = false;
     return AENET_OK;
 }
@@ -1488,7 +1556,7 @@ extern "C" void aenet_destroy(aenet_ctx *h) {
                     c.d_sp_rank, c.d_sp_list, c.d_sinfo, c.d_bres, c.d_act,
                     c.d_wpart, c.d_wpairs, c.d_dEdW, c.d_work, c.d_order, c.d_psinfo, c.d_porder,
                     c.d_vl, c.d_vl_count, c.d_vl_origin, c.d_vl_ref, c.d_vl_flag, c.d_vl_builds,
-                    c.d_vl_epart, c.d_vl_vpart, c.d_lambda};
+                    c.d_vl_epart, c.d_vl_vpart, c.d_lambda, c.d_rows, c.d_list_count, c.d_pnet, c.d_vir_atom};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     for (int k = 0; k <= Context::kStages; ++k)

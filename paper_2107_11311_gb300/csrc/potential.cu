@@ -219,7 +219,7 @@ cudaError_t na_launch_fp(const Basis &B, const Grid &g, const Caps &caps, cudaSt
     kern<<<g.ncell, kPThreads, smem, st>>>(B, net, g, nullptr, 0, caps, pos4, cell_start, nullptr, nullptr, nullptr,
                                            nullptr,
                                            nullptr, Gs, nullptr, nullptr, nullptr, stats, err, nullptr, nullptr,
-                                           g.ncell, nullptr, nullptr, 1, 0, TcNet{});
+                                           g.ncell, 1, 0, TcNet{});
     return cudaGetLastError();
 }
 

@@ -1,8 +1,8 @@
-// Device code of the potential: the fused kernel k_potential (and its
-// descriptor-only, forces-only and list-building forms) and the Verlet-list
-// kernel k_potential_list, with their shared-memory layouts. Included by
-// potential.cu (cell-list evaluation) and potential_md.cu (MD with a Verlet
-// list), which are compiled in parallel; each instantiates the forms it launches.
+// Device code of the potential kernel that finds its neighbours in the staged
+// cells: k_potential (fused, descriptor-only and forces-only forms), with its
+// shared-memory layout, and the device functions that the list-driven kernel
+// (list_kernels.cuh) shares with it. Each including translation unit
+// instantiates the forms it launches.
 //
 // Fused potential kernel: neighbours, descriptor (Sec. II.B), network
 // (Sec. II.A) and chain rule to forces and virial in one pass per atom.
@@ -55,9 +55,8 @@ enum Mode : int {
     kFused = 0,       // descriptor -> FP32 network -> forces, energy and virial
     kDescriptor = 1,  // descriptor only: G rows (sorted order)
     kForces = 2,      // forces and virial from given dE/dG rows (sorted order)
-    kBuildList = 3,   // Verlet list: every image-atom within rc_max + skin (no potential)
-    kFusedTC = 4,     // descriptor -> BF16 tensor-core network -> forces (one geometry pass)
-    kFusedTCx3 = 5    // the same with split-BF16 operands (hi*hi + hi*lo + lo*hi)
+    kFusedTC = 3,     // descriptor -> BF16 tensor-core network -> forces (one geometry pass)
+    kFusedTCx3 = 4    // the same with split-BF16 operands (hi*hi + hi*lo + lo*hi)
 };
 
 __host__ __device__ constexpr bool is_tc_mode(int mode) { return mode == kFusedTC || mode == kFusedTCx3; }
@@ -344,123 +343,6 @@ __device__ __forceinline__ void complete_list(const Basis &B, const float *s_tw,
             }
         }
         nang += __popc(ma);
-    }
-}
-
-// Verlet-list build: append the staged image-atoms within rc_list of atom i
-// (their staged entries, index | image-offset code) to the atom's row of the
-// global list; entries past the capacity are counted but not stored.
-__device__ __forceinline__ void scan_tile_build(const float4 *s_pos, const int *s_idx, int len, float4 ui, int self,
-                                                float rc2, int *__restrict__ row, int cap, int lane, int &nnb) {
-    const unsigned lt_mask = (1u << lane) - 1u;
-    for (int base = 0; base < len; base += 32) {
-        const int q = base + lane;
-        bool in = false;
-        int e = 0;
-        if (q < len) {
-            const float4 p = s_pos[q];
-            e = s_idx[q];
-            const float dx = p.x - ui.x, dy = p.y - ui.y, dz = p.z - ui.z;
-            in = (dx * dx + dy * dy + dz * dz <= rc2) && (e != self);
-        }
-        const unsigned m = __ballot_sync(kFull, in);
-        if (in) {
-            const int slot = nnb + __popc(m & lt_mask);
-            if (slot < cap) row[slot] = e;
-        }
-        nnb += __popc(m);
-    }
-}
-
-// scan_tile_build for two atoms at once (u0 and u1; the second only if two):
-// each staged image-atom is loaded once and tested against both.
-__device__ __forceinline__ void scan_tile_build2(const float4 *s_pos, const int *s_idx, int len, float4 u0, float4 u1,
-                                                 int self0, int self1, bool two, float rc2, int *__restrict__ row0,
-                                                 int *__restrict__ row1, int cap, int lane, int &n0, int &n1) {
-    const unsigned lt_mask = (1u << lane) - 1u;
-    for (int base = 0; base < len; base += 32) {
-        const int q = base + lane;
-        bool in0 = false, in1 = false;
-        int e = 0;
-        if (q < len) {
-            const float4 p = s_pos[q];
-            e = s_idx[q];
-            const float dx0 = p.x - u0.x, dy0 = p.y - u0.y, dz0 = p.z - u0.z;
-            const float dx1 = p.x - u1.x, dy1 = p.y - u1.y, dz1 = p.z - u1.z;
-            in0 = (dx0 * dx0 + dy0 * dy0 + dz0 * dz0 <= rc2) && (e != self0);
-            in1 = two && (dx1 * dx1 + dy1 * dy1 + dz1 * dz1 <= rc2) && (e != self1);
-        }
-        const unsigned m0 = __ballot_sync(kFull, in0), m1 = __ballot_sync(kFull, in1);
-        if (in0) {
-            const int slot = n0 + __popc(m0 & lt_mask);
-            if (slot < cap) row0[slot] = e;
-        }
-        if (in1) {
-            const int slot = n1 + __popc(m1 & lt_mask);
-            if (slot < cap) row1[slot] = e;
-        }
-        n0 += __popc(m0);
-        n1 += __popc(m1);
-    }
-}
-
-__device__ __forceinline__ void store_list_count(int *vl_count, int i_s, int nnb, int cap, int lane, unsigned *err) {
-    if (lane == 0) {
-        vl_count[i_s] = nnb < cap ? nnb : cap;
-        if (nnb > cap) atomicOr(err, kErrNbCap);
-    }
-}
-
-// Phase 1 of the list build from the Verlet list: the entries of atom i that
-// now lie within the largest cutoff, with the displacement computed exactly as
-// from the staged tile, (u_j + offset) - u_i. The entries of kListRounds rounds
-// of 32 are loaded together, then their positions together, so that a list of
-// up to 32 kListRounds entries costs two dependent L2 round trips, not two per
-// round; the kept entries stay in list order.
-constexpr int kListRounds = 4;
-
-__device__ __forceinline__ void scan_list(const int *__restrict__ row, int cnt, const float4 *__restrict__ pos4,
-                                          const float4 *off_shift, float4 ui, int jbits, const Basis &B,
-                                          const Caps &caps, const WarpLists &W, int lane, int &nnb) {
-    const float rc2max = B.rc_max * B.rc_max;
-    const unsigned lt_mask = (1u << lane) - 1u;
-    const int jmask = (1 << jbits) - 1;
-    for (int base = 0; base < cnt; base += kListRounds * 32) {
-        int e[kListRounds];
-        float4 p[kListRounds];
-#pragma unroll
-        for (int r = 0; r < kListRounds; ++r) {
-            const int k = base + 32 * r + lane;
-            e[r] = k < cnt ? __ldg(row + k) : -1;  // entries are non-negative
-        }
-#pragma unroll
-        for (int r = 0; r < kListRounds; ++r)
-            p[r] = e[r] >= 0 ? pos4[e[r] & jmask] : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int r = 0; r < kListRounds; ++r) {
-            bool in = false;
-            float dx = 0.f, dy = 0.f, dz = 0.f, r2 = 0.f;
-            int j = 0, typ = 0;
-            if (e[r] >= 0) {
-                j = e[r] & jmask;
-                const float4 sh = off_shift[e[r] >> jbits];
-                dx = (p[r].x + sh.x) - ui.x;
-                dy = (p[r].y + sh.y) - ui.y;
-                dz = (p[r].z + sh.z) - ui.z;
-                r2 = dx * dx + dy * dy + dz * dz;
-                typ = __float_as_int(p[r].w);
-                in = r2 <= rc2max;
-            }
-            const unsigned m = __ballot_sync(kFull, in);
-            if (in) {
-                const int slot = nnb + __popc(m & lt_mask);
-                if (slot < caps.nb) {
-                    W.e_d[slot] = make_float4(dx, dy, dz, r2);
-                    W.e_j[slot] = j | (typ << 28);
-                }
-            }
-            nnb += __popc(m);
-        }
     }
 }
 
@@ -1373,16 +1255,15 @@ __device__ __noinline__ void tc_species_network(int t, const int *order, int cnt
 }
 
 template <int KRT, int KAT, bool EXACT, int MODE, bool BATCH, int HB, int NW = kPWarps>
-// (the list-build mode keeps no per-warp state: 32 registers give it eight CTAs per SM)
-__global__ void __launch_bounds__(NW * 32, MODE == kBuildList ? 8 : (NW == kPWarps ? 2 : 1))
+__global__ void __launch_bounds__(NW * 32, NW == kPWarps ? 2 : 1)
     k_potential(Basis B, FusedNet net, Grid g_one, const StructInfo *__restrict__ sinfo, int n_struct, Caps caps,
                 const float4 *__restrict__ pos4,
                 const int *__restrict__ cell_start, const float *__restrict__ params, const float *__restrict__ shift,
                 const float *__restrict__ scale, float4 *__restrict__ F4, float *__restrict__ eatom,
                 float *__restrict__ G_out, const float *__restrict__ dEdG_in, double *__restrict__ e_part,
                 double *__restrict__ vir_part, unsigned long long *__restrict__ stats, unsigned *__restrict__ err,
-                unsigned *__restrict__ work, const int *__restrict__ order, int n_items, int *__restrict__ vl_out,
-                int *__restrict__ vl_count, int split, int split_from, TcNet tc) {
+                unsigned *__restrict__ work, const int *__restrict__ order, int n_items, int split, int split_from,
+                TcNet tc) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ float s_tw[kMaxSpecies];
     __shared__ float s_sh[sh_angular<KRT, KAT, EXACT>() ? kShTab : 1];  // spherical-harmonic form's table
@@ -1401,10 +1282,7 @@ __global__ void __launch_bounds__(NW * 32, MODE == kBuildList ? 8 : (NW == kPWar
     const int tile = caps.tile;
     // one layout for every cell: sized for the largest image-offset table
     // (g_one.n_off is that maximum in a batch)
-    // (the list-build form keeps no per-warp lists: its CTAs are small)
-    constexpr bool kLists = MODE != kBuildList;
-    const PLayout L = make_playout(g_one.n_off, tile, kLists ? caps.nb : 0, kLists ? caps.ang : 0,
-                                   (MODE == kFused || kTC) ? B.n_species : 0, kTC ? kTcParStride : net.stride, NW,
+    const PLayout L = make_playout(g_one.n_off, tile, caps.nb, caps.ang, (MODE == kFused || kTC) ? B.n_species : 0, kTC ? kTcParStride : net.stride, NW,
                                    kTC);
     int *off_start = reinterpret_cast<int *>(smem + L.off_start);
     int *off_count = reinterpret_cast<int *>(smem + L.off_count);
@@ -1527,9 +1405,6 @@ __global__ void __launch_bounds__(NW * 32, MODE == kBuildList ? 8 : (NW == kPWar
     const int cnt = a_hi - a_lo;
     const int slot = order ? cell : item;  // row of this item's energy / virial partials (per cell in a batch)
     const int n_chunks = (total + tile - 1) / tile;
-    // list-build mode: the entry of the atom itself (zero image offset) is excluded
-    const int self_code = (g.m[0] + wx * (g.m[1] + wy * g.m[2])) << caps.vl_jbits;
-    const float rc2list = caps.rc_list * caps.rc_list;
     // Staging of chunk `chunk` of the item's neighbourhood into s_pos / s_idx;
     // the number of staged image-atoms is in s_kept after the next barrier.
     // In an orthorhombic cell the item's cell is the box [0, h) of the staged
@@ -1541,7 +1416,7 @@ __global__ void __launch_bounds__(NW * 32, MODE == kBuildList ? 8 : (NW == kPWar
     // the unfiltered enumeration.
     const bool filter = !kTC && !g.tri;
     // (a relative margin of 1e-5 keeps pairs at the cutoff to the last ulp)
-    const float rc2stage = (MODE == kBuildList ? rc2list : B.rc_max * B.rc_max) * 1.00001f;
+    const float rc2stage = B.rc_max * B.rc_max * 1.00001f;
     const unsigned lt_mask = (1u << lane) - 1u;
     auto stage = [&](int chunk) {
         const int base = chunk * tile;
@@ -1563,10 +1438,7 @@ __global__ void __launch_bounds__(NW * 32, MODE == kBuildList ? 8 : (NW == kPWar
                 const float4 p = pos4[j];
                 const float4 sh = off_shift[lo];
                 sp = make_float4(p.x + sh.x, p.y + sh.y, p.z + sh.z, p.w);
-                if constexpr (MODE == kBuildList)
-                    code = j | (lo << caps.vl_jbits);  // the Verlet-list entry: index and image offset
-                else
-                    code = j | (__float_as_int(sh.w) ? kShiftBit : 0);
+                code = j | (__float_as_int(sh.w) ? kShiftBit : 0);
                 keep = true;
                 if (filter) {
                     const float dx = fmaxf(fmaxf(-sp.x, sp.x - g.hf[0]), 0.f);
@@ -1805,35 +1677,18 @@ __global__ void __launch_bounds__(NW * 32, MODE == kBuildList ? 8 : (NW == kPWar
         if (total > 0) stage(0);
         __syncthreads();
         const int staged = s_kept;
-        if constexpr (MODE == kBuildList) {  // two atoms per warp: one pass over the tile serves both
-            for (;;) {
-                int a = 0;
-                if (lane == 0) a = atomicAdd(&s_next, 2);
-                a = __shfl_sync(kFull, a, 0);
-                if (a >= cnt) break;
-                const bool two = a + 1 < cnt;
-                const int i0 = c0 + a, i1 = two ? i0 + 1 : i0;
-                int n0 = 0, n1 = 0;
-                scan_tile_build2(s_pos, s_idx, staged, pos4[i0], pos4[i1], i0 | self_code, i1 | self_code, two,
-                                 rc2list, vl_out + (size_t)i0 * caps.vl_cap, vl_out + (size_t)i1 * caps.vl_cap,
-                                 caps.vl_cap, lane, n0, n1);
-                store_list_count(vl_count, i0, n0, caps.vl_cap, lane, err);
-                if (two) store_list_count(vl_count, i1, n1, caps.vl_cap, lane, err);
-            }
-        } else {
-            for (;;) {
-                int a = 0;
-                if (lane == 0) a = atomicAdd(&s_next, 1);
-                a = __shfl_sync(kFull, a, 0);
-                if (a >= cnt) break;
-                const int i_s = c0 + a;
-                const float4 ui = pos4[i_s];
-                int nnb = 0, nang = 0;
-                scan_tile(s_pos, s_idx, staged, ui, i_s, B, caps, W, lane, nnb);
-                finish_list(nnb, nang);
-                process_atom<KRT, KAT, EXACT, MODE, HB>(i_s, nnb, nang, B, net, s_par, s_tw, s_sh, W, lane, pos4, F4,
-                                                        eatom, G_out, dEdG_in, e_acc, vir);
-            }
+        for (;;) {
+            int a = 0;
+            if (lane == 0) a = atomicAdd(&s_next, 1);
+            a = __shfl_sync(kFull, a, 0);
+            if (a >= cnt) break;
+            const int i_s = c0 + a;
+            const float4 ui = pos4[i_s];
+            int nnb = 0, nang = 0;
+            scan_tile(s_pos, s_idx, staged, ui, i_s, B, caps, W, lane, nnb);
+            finish_list(nnb, nang);
+            process_atom<KRT, KAT, EXACT, MODE, HB>(i_s, nnb, nang, B, net, s_par, s_tw, s_sh, W, lane, pos4, F4,
+                                                    eatom, G_out, dEdG_in, e_acc, vir);
         }
     } else {
         const int n_rounds = (cnt + NW - 1) / NW;
@@ -1849,21 +1704,13 @@ __global__ void __launch_bounds__(NW * 32, MODE == kBuildList ? 8 : (NW == kPWar
                 __syncthreads();
                 if (active) {
                     const int len = s_kept;
-                    if constexpr (MODE == kBuildList)
-                        scan_tile_build(s_pos, s_idx, len, ui, i_s | self_code, rc2list,
-                                        vl_out + (size_t)i_s * caps.vl_cap, caps.vl_cap, lane, nnb);
-                    else
-                        scan_tile(s_pos, s_idx, len, ui, i_s, B, caps, W, lane, nnb);
+                    scan_tile(s_pos, s_idx, len, ui, i_s, B, caps, W, lane, nnb);
                 }
             }
             if (active) {
-                if constexpr (MODE == kBuildList) {
-                    store_list_count(vl_count, i_s, nnb, caps.vl_cap, lane, err);
-                } else {
-                    finish_list(nnb, nang);
-                    process_atom<KRT, KAT, EXACT, MODE, HB>(i_s, nnb, nang, B, net, s_par, s_tw, s_sh, W, lane, pos4, F4,
-                                                            eatom, G_out, dEdG_in, e_acc, vir);
-                }
+                finish_list(nnb, nang);
+                process_atom<KRT, KAT, EXACT, MODE, HB>(i_s, nnb, nang, B, net, s_par, s_tw, s_sh, W, lane, pos4, F4,
+                                                        eatom, G_out, dEdG_in, e_acc, vir);
             }
         }
     }
@@ -1895,112 +1742,6 @@ __global__ void __launch_bounds__(NW * 32, MODE == kBuildList ? 8 : (NW == kPWar
         atomicAdd(&stats[0], st_nb);
         atomicAdd(&stats[1], st_ang);
         atomicAdd(&stats[2], st_pairs);
-    }
-}
-
-// The fused potential over the Verlet list (MD steps between list builds).
-// Persistent CTAs (the network parameters are staged once per CTA); each warp
-// takes the next sorted atom from a global counter, forms its neighbour list
-// from its Verlet-list row (scan_list) and then runs the same descriptor,
-// network and chain rule as k_potential. Energy and virial partials per CTA.
-template <int KRT, int KAT, bool EXACT, int HB>
-__global__ void __launch_bounds__(kPThreads, 2)
-    k_potential_list(Basis B, FusedNet net, Grid g, Caps caps, int n, const float4 *__restrict__ pos4,
-                     const int *__restrict__ vl, const int *__restrict__ vl_count, const float *__restrict__ params,
-                     const float *__restrict__ shift, const float *__restrict__ scale, float4 *__restrict__ F4,
-                     float *__restrict__ eatom, double *__restrict__ e_part, double *__restrict__ vir_part,
-                     unsigned long long *__restrict__ stats, unsigned *__restrict__ err,
-                     unsigned *__restrict__ work) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ float s_tw[kMaxSpecies];
-    __shared__ float s_sh[sh_angular<KRT, KAT, EXACT>() ? kShTab : 1];  // spherical-harmonic form's table
-    __shared__ float s_vir[kPWarps][9];
-    __shared__ double s_e[kPWarps];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const PLayout L = make_playout(g.n_off, 0, caps.nb, caps.ang, B.n_species, net.stride);
-    float4 *off_shift = reinterpret_cast<float4 *>(smem + L.off_shift);
-    float *s_par = reinterpret_cast<float *>(smem + L.params);
-    unsigned char *wb = smem + L.warp_base + L.warp_bytes * warp;
-    WarpLists W;
-    W.e_d = reinterpret_cast<float4 *>(wb + L.e_d);
-    W.e_j = reinterpret_cast<int *>(wb + L.e_j);
-    W.e_fx = reinterpret_cast<float *>(wb + L.e_fx);
-    W.e_fy = reinterpret_cast<float *>(wb + L.e_fy);
-    W.e_fz = reinterpret_cast<float *>(wb + L.e_fz);
-    W.a_u = reinterpret_cast<float4 *>(wb + L.a_u);
-    W.a_x = reinterpret_cast<float4 *>(wb + L.a_x);
-    W.a_s = reinterpret_cast<float *>(wb + L.a_s);
-    W.coef = reinterpret_cast<float *>(wb + L.coef);
-#pragma unroll
-    for (int t = 0; t < kMaxSpecies; ++t)
-        if (tid == t) s_tw[t] = B.type_weight[t];
-    if constexpr (sh_angular<KRT, KAT, EXACT>()) load_sh_table(B.sh_b, s_sh, tid);
-    load_net_params<KRT, KAT, EXACT>(B, net, params, shift, scale, s_par, tid, kPThreads);
-    const int wx = 2 * g.m[0] + 1, wy = 2 * g.m[1] + 1;
-    for (int o = tid; o < g.n_off; o += kPThreads) {  // image offset of every list code
-        const int ox = o % wx - g.m[0], oy = (o / wx) % wy - g.m[1], oz = o / (wx * wy) - g.m[2];
-        off_shift[o] = make_float4(ox * g.hf[0] + oy * g.htf[0] + oz * g.htf[1], oy * g.hf[1] + oz * g.htf[2],
-                                   oz * g.hf[2], 0.f);
-    }
-    __syncthreads();
-
-    float vir[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) vir[k] = 0.f;
-    double e_acc = 0.0;
-    unsigned long long st_nb = 0, st_ang = 0, st_pairs = 0;
-    for (;;) {
-        int a = 0;
-        if (lane == 0) a = (int)atomicAdd(work, 1u);
-        a = __shfl_sync(kFull, a, 0);
-        if (a >= n) break;
-        const int i_s = a;
-        const float4 ui = pos4[i_s];
-        int nnb = 0, nang = 0;
-        scan_list(vl + (size_t)i_s * caps.vl_cap, vl_count[i_s], pos4, off_shift, ui, caps.vl_jbits, B, caps, W,
-                  lane, nnb);
-        if (nnb > caps.nb) {
-            if (lane == 0) atomicOr(err, kErrNbCap);
-            nnb = caps.nb;
-        }
-        __syncwarp();
-        complete_list(B, s_tw, caps, W, lane, nnb, nang, err);
-        if (nang > caps.ang) {
-            if (lane == 0) atomicOr(err, kErrAngCap);
-            nang = caps.ang;
-        }
-        st_nb += nnb;
-        st_ang += nang;
-        st_pairs += (unsigned long long)(nang * (nang - 1) / 2);
-        __syncwarp();
-        process_atom<KRT, KAT, EXACT, kFused, HB>(i_s, nnb, nang, B, net, s_par, s_tw, s_sh, W, lane, pos4, F4, eatom,
-                                                  nullptr, nullptr, e_acc, vir);
-    }
-    __syncthreads();  // every warp has left the loop
-    if (tid == 0) release_work_counter(work);
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        const float v = warp_sum(vir[k]);
-        if (lane == 0) s_vir[warp][k] = v;
-    }
-    if (lane == 0) s_e[warp] = e_acc;
-    if (lane == 0 && st_nb) {
-        atomicAdd(&stats[0], st_nb);
-        atomicAdd(&stats[1], st_ang);
-        atomicAdd(&stats[2], st_pairs);
-    }
-    __syncthreads();
-    if (tid < 9) {
-        float sv = 0.f;
-#pragma unroll
-        for (int w = 0; w < kPWarps; ++w) sv += s_vir[w][tid];
-        vir_part[(size_t)blockIdx.x * 9 + tid] = (double)sv;
-    }
-    if (warp == 0) {
-        double v = lane < kPWarps ? s_e[lane] : 0.0;
-#pragma unroll
-        for (int o = kPWarps / 2; o >= 1; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-        if (lane == 0) e_part[blockIdx.x] = v;
     }
 }
 

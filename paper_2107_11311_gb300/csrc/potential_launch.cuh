@@ -88,8 +88,8 @@ cudaError_t launch_mode(Context &c, const Grid &g, const FusedNet &net) {
                                               c.d_cell_start, c.d_params,
                                               c.d_shift, c.d_scale, c.d_F4, c.d_eatom, rows, c.d_dEdG,
                                               c.d_e_part, c.d_vir_part, c.d_stats, c.d_err, work,
-                                              (work && c.batch_sinfo) ? c.batch_order : nullptr, n_items, nullptr,
-                                              nullptr, split, split_from, tn);
+                                              (work && c.batch_sinfo) ? c.batch_order : nullptr, n_items, split,
+                                              split_from, tn);
     c.last_grid = grid;
     c.pot_parts = n_items;
     return cudaGetLastError();
