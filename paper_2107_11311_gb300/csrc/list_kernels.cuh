@@ -29,7 +29,7 @@ constexpr int kEntryIndex = 0x0fffffff;  // sorted index of a list entry; the bi
 // ------------------------------------------------------------------ the build
 
 constexpr int kBuildThreads = 128;
-constexpr int kBuildAtoms = 4;  // atoms a warp tests every staged image-atom against
+constexpr int kBuildAtoms = 2;  // atoms a warp tests every staged image-atom against
 
 struct BuildLayout {
     size_t off_start, off_prefix, off_shift, s_pos, total;
@@ -56,7 +56,7 @@ __host__ __device__ inline BuildLayout make_build_layout(int n_off, int tile) {
 //     memory; in an orthorhombic box only those within the cutoff of the cell
 //     itself (about 72% of a 27-cell neighbourhood). More than `tile` of them
 //     are taken in chunks.
-//  2. Each warp tests the staged atoms against four atoms at a time. With
+//  2. Each warp tests the staged atoms against two atoms at a time (four: 40 more registers, 3% slower). With
 //     t = |p|^2 - 2 p.u the test is t <= rc^2 - |u|^2, three FMAs per pair;
 //     its rounding is covered by a margin (the potential kernel applies the
 //     exact cutoff to the displacement). The atom itself passes the test and
@@ -64,7 +64,7 @@ __host__ __device__ inline BuildLayout make_build_layout(int n_off, int tile) {
 // It also clears the atoms' force accumulators and the neighbour statistics (F4
 // and stats, when given).
 template <bool BATCH, bool CODES>
-__global__ void __launch_bounds__(kBuildThreads, 8)
+__global__ void __launch_bounds__(kBuildThreads, 12)
     k_list_build(Grid g_one, const StructInfo *__restrict__ sinfo, int n_struct, float rc, int tile, int parts,
                  int a_lo, int a_hi, const float4 *__restrict__ pos4, const int *__restrict__ cell_start,
                  float4 *__restrict__ rows, int *__restrict__ codes, int cap, int jbits, int *__restrict__ count,
@@ -174,6 +174,8 @@ __global__ void __launch_bounds__(kBuildThreads, 8)
         if (tid == 0) s_next = 0;
         __syncthreads();
         const int len = s_kept;
+        if (warp == 0 && (len & 31) && lane >= (len & 31)) s_pos[(len & ~31) + lane] = make_float4(1e15f, 0.f, 0.f, 0.f);
+        __syncthreads();
         for (;;) {
             int a = 0;
             if (lane == 0) a = atomicAdd(&s_next, kBuildAtoms);
@@ -181,9 +183,11 @@ __global__ void __launch_bounds__(kBuildThreads, 8)
             if (a >= n) break;
             float mx[kBuildAtoms], my[kBuildAtoms], mz[kBuildAtoms], lim[kBuildAtoms];  // -2u; rc^2 - |u|^2
             int cnt[kBuildAtoms];
+            size_t row[kBuildAtoms];
 #pragma unroll
             for (int b = 0; b < kBuildAtoms; ++b) {
                 const int i = first + min(a + b, n - 1);
+                row[b] = (size_t)(i - (CODES ? 0 : a_lo)) * cap;
                 const float4 u = pos4[i];
                 const float u2 = u.x * u.x + u.y * u.y + u.z * u.z, ur = sqrtf(u2) + rc;
                 mx[b] = -2.f * u.x;
@@ -197,8 +201,8 @@ __global__ void __launch_bounds__(kBuildThreads, 8)
             __syncwarp();
             for (int base = 0; base < len; base += 32) {
                 const int k = base + lane;
-                float4 p = s_pos[min(k, len - 1)];
-                float pp = k < len ? p.x * p.x + p.y * p.y + p.z * p.z : 3e38f;
+                const float4 p = s_pos[k];  // (the tile is padded to whole rounds with atoms out of reach)
+                const float pp = p.x * p.x + p.y * p.y + p.z * p.z;
 #pragma unroll
                 for (int b = 0; b < kBuildAtoms; ++b) {
                     const float t = fmaf(p.x, mx[b], fmaf(p.y, my[b], fmaf(p.z, mz[b], pp)));
@@ -206,11 +210,10 @@ __global__ void __launch_bounds__(kBuildThreads, 8)
                     const unsigned m = __ballot_sync(kFull, in);
                     const int slot = cnt[b] + __popc(m & lt_mask);
                     if (in && slot < cap) {
-                        const size_t at = (size_t)(first + a + b - (CODES ? 0 : a_lo)) * cap + slot;
                         if constexpr (CODES)
-                            codes[at] = __float_as_int(p.w);
+                            codes[row[b] + slot] = __float_as_int(p.w);
                         else
-                            rows[at] = make_float4(fmaf(0.5f, mx[b], p.x), fmaf(0.5f, my[b], p.y),
+                            rows[row[b] + slot] = make_float4(fmaf(0.5f, mx[b], p.x), fmaf(0.5f, my[b], p.y),
                                                    fmaf(0.5f, mz[b], p.z), p.w);
                     }
                     cnt[b] += __popc(m);
@@ -232,11 +235,13 @@ __global__ void __launch_bounds__(kBuildThreads, 8)
 
 // -------------------------------------------------------------- the potential
 
-// Warps of a CTA (one CTA per SM). The pair form fits 80 registers, so 24
-// warps; the spherical-harmonic form's accumulators need up to 128 (16 warps).
+// Warps of a CTA (one CTA per SM): 20 at 96 registers for the pair form (water
+// 98,304 atoms, whole evaluation: 521 us; 24 warps at 80 registers spill, 534 us;
+// 16 at 128, 552 us), 16 at 128 for the spherical-harmonic form, whose
+// accumulators need them (solid 27,000: 273 us; 12 warps, 287 us).
 template <int KRT, int KAT, bool EXACT>
 __host__ __device__ constexpr int list_max_warps() {
-    return sh_angular<KRT, KAT, EXACT>() ? 16 : 24;
+    return sh_angular<KRT, KAT, EXACT>() ? 16 : 20;
 }
 
 // Descriptor slots in the list kernel: [radial | angular | radial_w | angular_w]
@@ -350,8 +355,8 @@ __host__ __device__ inline ListLayout make_list_layout(int n_off, int nb, int an
     L.red = q;  // reduction buffer; later dE/du sums of the angular entries (float4 each)
     const size_t red = sizeof(float) * 32 * kRedStride, grad = sizeof(float4) * ang;
     q = align16(q + (red > grad ? red : grad));
-    L.coef = q;  // network inputs (64 floats), then the coefficient quads (a, a, a_w, a_w) of every order
-    q = align16(q + sizeof(float4) * 32);
+    L.coef = q;  // network inputs, then the coefficient pairs (a, a_w) of every order (64 floats)
+    q = align16(q + sizeof(float2) * 32);
     L.sh = q;  // component sums and coefficients of the spherical-harmonic form
     if (sh) q = align16(q + sizeof(float) * kShScratch);
     L.warp_bytes = q;
@@ -370,15 +375,17 @@ struct ListWarp {
 
 // Entry k of round r of the main list: rounds 0 .. nra-1 hold the angular
 // entries (front), the later ones the others (back of the buffer, descending).
-__device__ __forceinline__ bool list_round(int r, int nra, int nang, int nrest, int nb, int lane, int &k) {
-    if (r < nra) {
-        k = 32 * r + lane;
-        return k < nang;
+struct Rounds {
+    int nra, nang, front, back, low;  // back - 32 r: index in a later round; low: the last of them
+    __device__ __forceinline__ Rounds(int nang_, int nrest, int nb, int lane)
+        : nra((nang_ + 31) >> 5), nang(nang_), front(lane), back(nb - 1 - lane + 32 * ((nang_ + 31) >> 5)),
+          low(nb - nrest) {}
+    __device__ __forceinline__ bool at(int r, int &k) const {
+        const bool ang = r < nra;  // (uniform)
+        k = ang ? front + 32 * r : back - 32 * r;
+        return ang ? k < nang : k >= low;
     }
-    const int q = 32 * (r - nra) + lane;
-    k = nb - 1 - q;
-    return q < nrest;
-}
+};
 
 // Warp totals of 8 pairs of partial sums (one pair per lane and order): lane l
 // returns the pair of order 2 (l & 3) + (l >> 4). Each lane leaves its 16 values
@@ -416,12 +423,30 @@ __device__ __forceinline__ float2 reduce8(const float2 (&v)[8], float *red, int 
 }
 __device__ __forceinline__ int reduce8_order(int lane) { return 2 * (lane & 3) + (lane >> 4); }
 
+// Two pairs (10 shuffles; the buffer would move 16): lane l returns the pair l >> 4.
+__device__ __forceinline__ float2 reduce2(float2 v0, float2 v1, int lane) {
+    const bool up = lane & 16;
+    float2 send = up ? v0 : v1, t = up ? v1 : v0;
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) {
+        t = __fadd2_rn(t, make_float2(__shfl_xor_sync(kFull, send.x, o), __shfl_xor_sync(kFull, send.y, o)));
+        send = t;
+    }
+    return t;
+}
+
 // The totals of orders [0, N) of v (a compile-time count), times scale, to
 // dst[2 (at + order)] and [.. + 1].
 template <int N>
 __device__ __forceinline__ void reduce_orders(const float2 *v, float *red, float *dst, int at, int lane) {
 #pragma unroll
     for (int b = 0; b < N; b += 8) {
+        if (N - b <= 2) {
+            const float2 t = reduce2(v[b], N - b == 2 ? v[b + 1 < N ? b + 1 : b] : dup2(0.f), lane);
+            const int o = b + (lane >> 4);
+            if ((lane & 15) == 0 && o < N) *reinterpret_cast<float2 *>(dst + 2 * (at + o)) = t;
+            continue;
+        }
         float2 w[8];
 #pragma unroll
         for (int q = 0; q < 8; ++q) w[q] = b + q < N ? v[b + q] : dup2(0.f);
@@ -441,21 +466,19 @@ __device__ __forceinline__ void reduce_orders(const float2 *v, float *red, float
 template <int KAT, bool EXACT>
 __device__ __forceinline__ void ring_forward(int n, int Ka, const ListWarp &W, int lane, float2 (&pp)[KAT],
                                              float2 (&pw)[KAT]) {
-    const int self = lane < n ? lane : 0, last = n >> 1;
+    const int self = lane < n ? lane : 0;
     float4 uj = W.a_u[self];
     const float sj = W.a_s[self];
     if (lane >= n) uj.w = 0.f;
     const float4 *pu = W.a_u + self + 1;
     const float *ps = W.a_s + self + 1;
-    for (int t = 1; t <= last; t += 2, pu += 2, ps += 2) {
+    const float2 fj = dup2(uj.w);
+    auto two = [&](float2 f) {  // two shifts; f: uj.w times the weight of each
         const float4 ua = pu[0], ub = pu[1];
-        const float sa = ps[0], sb = ps[1];
-        // weight 1/2 for the shift that meets every pair twice, 0 past the last one
-        const float fa = 2 * t == n ? 0.5f : 1.0f, fb = t + 1 > last ? 0.f : (2 * (t + 1) == n ? 0.5f : 1.0f);
         const float2 c = make_float2(uj.x * ua.x + uj.y * ua.y + uj.z * ua.z,
                                      uj.x * ub.x + uj.y * ub.y + uj.z * ub.z);
-        const float2 w = make_float2(uj.w * ua.w * fa, uj.w * ub.w * fb);
-        const float2 ww = make_float2(w.x * (sj * sa), w.y * (sj * sb));
+        const float2 w = make_float2(f.x * ua.w, f.y * ub.w);
+        const float2 ww = make_float2(w.x * (sj * ps[0]), w.y * (sj * ps[1]));
         const float2 x2 = __fadd2_rn(c, c);
         float2 tm = dup2(1.0f), tc = c;
         pp[0] = __fadd2_rn(pp[0], w);
@@ -470,35 +493,80 @@ __device__ __forceinline__ void ring_forward(int n, int Ka, const ListWarp &W, i
                 tc = tn;
             }
         }
-    }
+        pu += 2;
+        ps += 2;
+    };
+    if (n < 2) return;
+    const int full = (n - 1) >> 1;  // shifts that meet every pair once
+    for (int i = full >> 1; i > 0; --i) two(fj);
+    // what is left: a full shift (odd `full`), then the half-weighted one (even n)
+    if ((full & 1) || !(n & 1))
+        two((full & 1) ? make_float2(uj.w, (n & 1) ? 0.f : 0.5f * uj.w) : make_float2(0.5f * uj.w, 0.f));
 }
 
-// S = sum_q a_q T_q(x) and dS = sum_q a_q T_q'(x) of two arguments, a_q = a0_q +
-// w a1_q, the coefficient quads (a0, a0, a1, a1) read from shared memory
-// (clenshaw_d2 with the coefficients in memory instead of 4 K registers).
-template <int KT, bool EXACT>
-__device__ __forceinline__ void clenshaw_quads(float2 x, float2 w, const float4 *quad, int K, float2 &S, float2 &dS) {
-    // (a compiler barrier: hoisted out of the caller's loop the quads would hold
-    // 4 KT registers)
-    asm volatile("" ::: "memory");
-    const float2 m1 = dup2(-1.0f), x2 = __fadd2_rn(x, x);
-    float2 b1 = dup2(0.f), b2 = b1, D1 = b1, D2 = b1;
-#pragma unroll
-    for (int q = KT - 1; q >= 1; --q) {
-        if (EXACT || q < K) {
-            const float4 k = quad[q];
-            const float2 a = ffma2(w, make_float2(k.z, k.w), make_float2(k.x, k.y));
-            const float2 b = ffma2(x2, b1, ffma2(m1, b2, a));
-            const float2 D = ffma2(x2, D1, ffma2(m1, D2, b1));
-            b2 = b1;
-            b1 = b;
-            D2 = D1;
-            D1 = D;
-        }
+// One step of Clenshaw's recurrence for two arguments (clenshaw_d2): the
+// coefficient a0 + w a1 of each, then b and the halved derivative chain D. The
+// coefficients are scalars: two scalar FMAs take as long as one packed one, and
+// need no duplicated operand in registers or shared memory.
+struct Clenshaw2 {
+    float2 x2, b1, b2, D1, D2;
+    __device__ __forceinline__ explicit Clenshaw2(float2 x) : x2(__fadd2_rn(x, x)), b1(dup2(0.f)) { b2 = D1 = D2 = b1; }
+    __device__ __forceinline__ void step(float a0, float a1, float2 w) {
+        const float2 m1 = dup2(-1.0f), a = make_float2(fmaf(w.x, a1, a0), fmaf(w.y, a1, a0));
+        const float2 b = ffma2(x2, b1, ffma2(m1, b2, a));
+        const float2 D = ffma2(x2, D1, ffma2(m1, D2, b1));
+        b2 = b1;
+        b1 = b;
+        D2 = D1;
+        D1 = D;
     }
-    const float4 k = quad[0];
-    S = ffma2(x, b1, ffma2(m1, b2, ffma2(w, make_float2(k.z, k.w), make_float2(k.x, k.y))));
-    dS = ffma2(x2, D1, ffma2(dup2(-2.0f), D2, b1));
+    __device__ __forceinline__ void finish(float a0, float a1, float2 w, float2 x, float2 &S, float2 &dS) {
+        const float2 a = make_float2(fmaf(w.x, a1, a0), fmaf(w.y, a1, a0));
+        S = ffma2(x, b1, ffma2(dup2(-1.0f), b2, a));
+        dS = ffma2(x2, D1, ffma2(dup2(-2.0f), D2, b1));
+    }
+};
+
+// S = sum_q a_q T_q(x) and dS = sum_q a_q T_q'(x) of two arguments, a_q = a0_q +
+// w a1_q, the coefficient pairs (a0, a1) of orders 0 .. KT - 1 read from shared
+// memory, two orders per 128-bit load (KT registers each would not fit).
+template <int KT, bool EXACT>
+__device__ __forceinline__ void clenshaw_shared(float2 x, float2 w, const float2 *coef, int K, float2 &S, float2 &dS) {
+    // (a compiler barrier: the loads stay inside the caller's loop)
+    asm volatile("" ::: "memory");
+    Clenshaw2 c(x);
+    const float4 *two = reinterpret_cast<const float4 *>(coef);
+#pragma unroll
+    for (int h = (KT - 1) / 2; h >= 1; --h) {
+        const float4 k = two[h];
+        if (2 * h + 1 < KT && (EXACT || 2 * h + 1 < K)) c.step(k.z, k.w, w);
+        if (EXACT || 2 * h < K) c.step(k.x, k.y, w);
+    }
+    const float4 k = two[0];
+    if (KT > 1 && (EXACT || K > 1)) c.step(k.z, k.w, w);
+    c.finish(k.x, k.y, w, x, S, dS);
+}
+
+// The same with the coefficients in registers.
+template <int KT, bool EXACT>
+__device__ __forceinline__ void clenshaw_regs(float2 x, float2 w, const float (&a0)[KT], const float (&a1)[KT], int K,
+                                              float2 &S, float2 &dS) {
+    Clenshaw2 c(x);
+#pragma unroll
+    for (int q = KT - 1; q >= 1; --q)
+        if (EXACT || q < K) c.step(a0[q], a1[q], w);
+    c.finish(a0[0], a1[0], w, x, S, dS);
+}
+
+// Coefficient pairs of the KAT angular orders into registers.
+template <int KAT>
+__device__ __forceinline__ void load_coef(const float2 *coef, float (&a0)[KAT], float (&a1)[KAT]) {
+#pragma unroll
+    for (int q = 0; q < KAT; ++q) {
+        const float2 k = coef[q];
+        a0[q] = k.x;
+        a1[q] = k.y;
+    }
 }
 
 // Backward: with S_jk = sum_q a_q T_q(c), S'_jk its derivative and f the cutoff
@@ -509,42 +577,50 @@ __device__ __forceinline__ void clenshaw_quads(float2 x, float2 w, const float4 
 // the rest is done once per entry. Each lane adds its own side and takes S and
 // S' of the pair it is the partner of by two shuffles.
 template <int KAT, bool EXACT>
-__device__ __forceinline__ float4 ring_backward(int n, int Ka, const ListWarp &W, const float4 *quad, int lane) {
-    const int self = lane < n ? lane : 0, last = n >> 1;
+__device__ __forceinline__ float4 ring_backward(int n, int Ka, const ListWarp &W, const float2 *coef, int lane) {
+    float a0[KAT], a1[KAT];
+    load_coef(coef, a0, a1);
+    const int self = lane < n ? lane : 0;
     const float4 uj = W.a_u[self];
     const float sj = W.a_s[self];
     const float4 *pu = W.a_u + self + 1;
     const float *ps = W.a_s + self + 1;
     float4 V = make_float4(0.f, 0.f, 0.f, 0.f);  // V_j, B_j
-    for (int t = 1; t <= last; t += 2, pu += 2, ps += 2) {
+    int sa = lane == 0 ? n - 1 : lane - 1;       // lane (l - t) mod n
+    // two shifts: j: the second one is inside the range; ka, kb: their pairs are met
+    // once, so that the other side has to be added too
+    auto two = [&](bool j, bool ka, bool kb) {
         const float4 ua = pu[0], ub = pu[1];
         const float2 w = make_float2(sj * ps[0], sj * ps[1]);
         const float2 c = make_float2(uj.x * ua.x + uj.y * ua.y + uj.z * ua.z,
                                      uj.x * ub.x + uj.y * ub.y + uj.z * ub.z);
         float2 S, dS;
-        clenshaw_quads<KAT, EXACT>(c, w, quad, Ka, S, dS);
-        const bool two = t + 1 <= last;  // (uniform) the second shift is inside the range
-        const float fa = ua.w, fb = two ? ub.w : 0.f;
+        clenshaw_regs<KAT, EXACT>(c, w, a0, a1, Ka, S, dS);
+        const float fa = ua.w, fb = j ? ub.w : 0.f;
         const float ga = dS.x * fa, gb = dS.y * fb;
         V.x = fmaf(ga, ua.x, fmaf(gb, ub.x, V.x));
         V.y = fmaf(ga, ua.y, fmaf(gb, ub.y, V.y));
         V.z = fmaf(ga, ua.z, fmaf(gb, ub.z, V.z));
         V.w = fmaf(S.x, fa, fmaf(S.y, fb, V.w));
-        // the other side: this lane is the partner of lane (l - t) mod n; at t = n/2
-        // (n even) that pair has been added from both sides already
-        int sa = lane - t, sb = sa - 1;
-        if (sa < 0) sa += n;
-        if (sb < 0) sb += n;
+        // the other side: this lane is the partner of lane (l - t) mod n
+        const int sb = sa == 0 ? n - 1 : sa - 1;
         const float dSa = __shfl_sync(kFull, dS.x, sa), Sa = __shfl_sync(kFull, S.x, sa);
         const float dSb = __shfl_sync(kFull, dS.y, sb), Sb = __shfl_sync(kFull, S.y, sb);
         const float4 va = W.a_u[sa], vb = W.a_u[sb];
-        const float ha = 2 * t == n ? 0.f : va.w, hb = two && 2 * (t + 1) != n ? vb.w : 0.f;
-        const float ka = dSa * ha, kb = dSb * hb;
-        V.x = fmaf(ka, va.x, fmaf(kb, vb.x, V.x));
-        V.y = fmaf(ka, va.y, fmaf(kb, vb.y, V.y));
-        V.z = fmaf(ka, va.z, fmaf(kb, vb.z, V.z));
+        const float ha = ka ? va.w : 0.f, hb = kb ? vb.w : 0.f;
+        const float ma = dSa * ha, mb = dSb * hb;
+        V.x = fmaf(ma, va.x, fmaf(mb, vb.x, V.x));
+        V.y = fmaf(ma, va.y, fmaf(mb, vb.y, V.y));
+        V.z = fmaf(ma, va.z, fmaf(mb, vb.z, V.z));
         V.w = fmaf(Sa, ha, fmaf(Sb, hb, V.w));
-    }
+        sa = sb == 0 ? n - 1 : sb - 1;
+        pu += 2;
+        ps += 2;
+    };
+    if (n < 2) return V;
+    const int full = (n - 1) >> 1;
+    for (int i = full >> 1; i > 0; --i) two(true, true, true);
+    if ((full & 1) || !(n & 1)) two((full & 1) && !(n & 1), full & 1, false);
     return V;
 }
 
@@ -610,7 +686,9 @@ __device__ __forceinline__ void blocks_forward(int n, int Ka, const ListWarp &W,
 
 // (a_g: the sums (V, B) of every entry, zeroed and filled here)
 template <int KAT, bool EXACT>
-__device__ __forceinline__ void blocks_backward(int n, int Ka, const ListWarp &W, const float4 *quad, int lane) {
+__device__ __forceinline__ void blocks_backward(int n, int Ka, const ListWarp &W, const float2 *coef, int lane) {
+    float a0[KAT], a1[KAT];
+    load_coef(coef, a0, a1);
     const int nblk = (n + 31) >> 5, bs = (n + nblk - 1) / nblk;
     for (int k = lane; k < n; k += 32) W.a_g[k] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncwarp();
@@ -634,7 +712,7 @@ __device__ __forceinline__ void blocks_backward(int n, int Ka, const ListWarp &W
                 const float2 c = make_float2(uj.x * ua.x + uj.y * ua.y + uj.z * ua.z,
                                              uj.x * ub.x + uj.y * ub.y + uj.z * ub.z);
                 float2 S, dS;
-                clenshaw_quads<KAT, EXACT>(c, make_float2(sj * W.a_s[a.k], sj * W.a_s[b.k]), quad, Ka, S, dS);
+                clenshaw_regs<KAT, EXACT>(c, make_float2(sj * W.a_s[a.k], sj * W.a_s[b.k]), a0, a1, Ka, S, dS);
                 const float fa = a.v != 0.f ? ua.w : 0.f, fb = b.v != 0.f ? ub.w : 0.f;
                 const float ga = dS.x * fa, gb = dS.y * fb;
                 V.x = fmaf(ga, ua.x, fmaf(gb, ub.x, V.x));
@@ -760,14 +838,14 @@ __device__ __forceinline__ void sh_fingerprints(const float *sh, const float *ta
 // (A_c k_l, A'_c k'_l), k_l = sum_a g_a b_al, written over the component sums, V is
 // the contraction's gradient F and B = E - 2 w (sum_a g_a + s^2 sum_a g'_a).
 template <int KRT, int KAT>
-__device__ __forceinline__ void sh_gradients(int nang, const ListWarp &W, const float4 *quad, const float *tab,
+__device__ __forceinline__ void sh_gradients(int nang, const ListWarp &W, const float2 *coef, const float *tab,
                                              int lane) {
     float gsum = 0.f, gwsum = 0.f;
     float dv[2], dwv[2];
 #pragma unroll
     for (int a = 0; a < KAT; ++a) {
-        gsum += quad[KRT + a].x;
-        gwsum += quad[KRT + a].z;
+        gsum += coef[KRT + a].x;
+        gwsum += coef[KRT + a].y;
     }
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -779,8 +857,8 @@ __device__ __forceinline__ void sh_gradients(int nang, const ListWarp &W, const 
 #pragma unroll
             for (int a = 0; a < KAT; ++a) {
                 const float b = tab[kShTabB + a * (kShL + 1) + l];
-                kl = fmaf(quad[KRT + a].x, b, kl);
-                klw = fmaf(quad[KRT + a].z, b, klw);
+                kl = fmaf(coef[KRT + a].x, b, kl);
+                klw = fmaf(coef[KRT + a].y, b, klw);
             }
             const float n2 = 2.0f * tab[kShTabN + c];
             dv[h] = n2 * W.sh[2 * c] * kl;
@@ -835,7 +913,7 @@ __device__ __forceinline__ float list_network(const FusedNet &net, const float *
     {
         const float *wr = W1 + o * WS + h * NK1, *gx = xs + h * NK1;
         float2 za = dup2(0.f);
-#pragma unroll 2
+#pragma unroll 4
         for (int k = 0; k < NK1; k += 4) {
             const float4 gv = *reinterpret_cast<const float4 *>(gx + k);
             const float4 wv = *reinterpret_cast<const float4 *>(wr + k);
@@ -856,7 +934,7 @@ __device__ __forceinline__ float list_network(const FusedNet &net, const float *
             __syncwarp();
             const float *wr = Pt + net.offW[l] + o * HS + h * NKH, *xv = xs + h * NKH;
             float2 za = dup2(0.f);
-#pragma unroll 2
+#pragma unroll 4
             for (int k = 0; k < NKH; k += 4) {
                 const float4 gv = *reinterpret_cast<const float4 *>(xv + k);
                 const float4 wv = *reinterpret_cast<const float4 *>(wr + k);
@@ -901,23 +979,23 @@ __device__ __forceinline__ float list_network(const FusedNet &net, const float *
         }
     }
     // dE/dg of the lane's slot and its weighted copy: sums over even and odd neurons
+    // in the two halves of a packed accumulator
     __syncwarp();
-    if (lane < HB) *reinterpret_cast<float2 *>(xs + 2 * lane) = dup2(delta);
+    if (lane < HB) xs[lane] = delta;
     __syncwarp();
-    float2 dd = dup2(0.f), ee = dd;
+    float2 d0 = dup2(0.f), d1 = d0;
     const float *wq = W1 + s0;
 #pragma unroll 2
     for (int q = 0; q < HB; q += 4) {
-        const float4 d01 = *reinterpret_cast<const float4 *>(xs + 2 * q);
-        const float4 d23 = *reinterpret_cast<const float4 *>(xs + 2 * q + 4);
+        const float4 d = *reinterpret_cast<const float4 *>(xs + q);
         const float *w = wq + q * WS;
-        dd = ffma2(make_float2(w[0], w[P]), make_float2(d01.x, d01.y), dd);
-        ee = ffma2(make_float2(w[WS], w[WS + P]), make_float2(d01.z, d01.w), ee);
-        dd = ffma2(make_float2(w[2 * WS], w[2 * WS + P]), make_float2(d23.x, d23.y), dd);
-        ee = ffma2(make_float2(w[3 * WS], w[3 * WS + P]), make_float2(d23.z, d23.w), ee);
+        d0 = ffma2(make_float2(w[0], w[WS]), make_float2(d.x, d.y), d0);
+        d1 = ffma2(make_float2(w[P], w[WS + P]), make_float2(d.x, d.y), d1);
+        d0 = ffma2(make_float2(w[2 * WS], w[3 * WS]), make_float2(d.z, d.w), d0);
+        d1 = ffma2(make_float2(w[2 * WS + P], w[3 * WS + P]), make_float2(d.z, d.w), d1);
     }
-    c0 = (dd.x + ee.x) * sc0;
-    c1 = (dd.y + ee.y) * sc1;
+    c0 = (d0.x + d0.y) * sc0;
+    c1 = (d1.x + d1.y) * sc1;
     __syncwarp();  // every lane has read the deltas
     return E;
 }
@@ -974,7 +1052,7 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
     W.a_g = reinterpret_cast<float4 *>(wb + L.red);
     W.coef = reinterpret_cast<float *>(wb + L.coef);
     W.sh = reinterpret_cast<float *>(wb + L.sh);
-    const float4 *quad = reinterpret_cast<const float4 *>(W.coef);
+    const float2 *coef = reinterpret_cast<const float2 *>(W.coef);  // (a, a_w) of every order
 #pragma unroll
     for (int t = 0; t < kMaxSpecies; ++t)
         if (tid == t) s_tw[t] = B.type_weight[t];
@@ -999,15 +1077,37 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
     float vir[6];
 #pragma unroll
     for (int k = 0; k < 6; ++k) vir[k] = 0.f;
+    // The first two rounds of an atom's row, its length and its species are loaded
+    // while the atom before is in its last phase.
+    struct Ahead {
+        float4 e0, e1;
+        int c0, c1;  // code rows
+        int cnt, type;
+    } nx;
+    auto fetch = [&](int i) {
+        if (i >= a_hi) return;
+        nx.cnt = count[i];
+        nx.type = __float_as_int(pos4[i].w);
+        if constexpr (CODES) {
+            const int *row = codes + (size_t)i * caps.vl_cap;
+            nx.c0 = __ldg(row + lane);  // (rows hold at least 64 entries; those past the count are not used)
+            nx.c1 = __ldg(row + 32 + lane);
+        } else {
+            const float4 *row = rows + (size_t)(i - a_lo) * caps.vl_cap;
+            nx.e0 = __ldcs(row + lane);
+            nx.e1 = __ldcs(row + 32 + lane);
+        }
+    };
     const int n_static = nw * (int)gridDim.x;
     int a = a_lo + warp * (int)gridDim.x + (int)blockIdx.x;
+    fetch(a);
     while (a < a_hi) {
         int next = 0;  // the counter's reply is needed only at the end of the atom
         if (lane == 0) next = a_lo + n_static + (int)atomicAdd(work, 1u);
 
         // ---- 1. the list, and the radial sums of the descriptor as it is read (in
         // row order: sorted by distance the FP32 sums would be biased)
-        const int cnt = count[a];
+        const int cnt = nx.cnt, type = nx.type;
         int nang = 0, nrest = 0;
         bool over = false;
         constexpr bool kDesc = MODE != kForces;
@@ -1074,7 +1174,7 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
             const int *row = codes + (size_t)a * caps.vl_cap;
             auto code = [&](int base) { return base + lane < cnt ? __ldg(row + base + lane) : -1; };  // (entries >= 0)
             auto gather = [&](int e) { return e >= 0 ? pos4[e & jmask] : make_float4(0.f, 0.f, 0.f, 0.f); };
-            int e0 = code(0), e1 = code(32);
+            int e0 = lane < cnt ? nx.c0 : -1, e1 = 32 + lane < cnt ? nx.c1 : -1;
             float4 p0 = gather(e0);
             for (int base = 0; base < cnt; base += 32) {
                 const float4 p1 = gather(e1);
@@ -1088,11 +1188,10 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
             }
         } else {
             const float4 *row = rows + (size_t)(a - a_lo) * caps.vl_cap;
-            // (up to the row's capacity, so that the first loads do not wait for the count)
             auto load = [&](int base) {
-                return base + lane < caps.vl_cap ? __ldcs(row + base + lane) : make_float4(0.f, 0.f, 0.f, 0.f);
+                return base + lane < cnt ? __ldcs(row + base + lane) : make_float4(0.f, 0.f, 0.f, 0.f);
             };
-            float4 e0 = load(0), e1 = load(32);
+            float4 e0 = nx.e0, e1 = nx.e1;
             for (int base = 0; base < cnt; base += 32) {
                 const float4 e2 = load(base + 64);
                 append(base + lane < cnt, e0.x, e0.y, e0.z, __float_as_int(e0.w));
@@ -1104,7 +1203,7 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
         if (lane < 3)
             s_sum.st[warp][lane] += lane == 0 ? (unsigned long long)(nang + nrest)
                                    : lane == 1 ? (unsigned long long)nang
-                                               : (unsigned long long)nang * (unsigned)(nang - 1) / 2;
+                                               : (unsigned long long)((unsigned)nang * (unsigned)(nang - 1) / 2);
         if (nang > caps.ang) {
             if (lane == 0) atomicOr(err, kErrAngCap);
             nang = caps.ang;
@@ -1119,7 +1218,8 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
                 __syncwarp();
             }
         }
-        const int nra = (nang + 31) >> 5, nrounds = nra + ((nrest + 31) >> 5);
+        const Rounds rounds(nang, nrest, nb, lane);
+        const int nra = rounds.nra, nrounds = nra + ((nrest + 31) >> 5);
 
         // ---- 2. the descriptor
         float G0 = 0.f, G1 = 0.f;  // coefficient `lane` of [radial | angular], plain and weighted
@@ -1161,12 +1261,13 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
             const int k0 = lane_col<KRT, KAT>(lane, 0, Kr, Ka), k1 = lane_col<KRT, KAT>(lane, 1, Kr, Ka);
             if (k0 >= 0) G_out[(size_t)a * D + k0] = G0;
             if (k1 >= 0) G_out[(size_t)a * D + k1] = G1;
+            next = __shfl_sync(kFull, next, 0);
+            fetch(next);
         } else {
             // ---- 3. the network
             float c0, c1;
             if constexpr (MODE == kFused) {
-                const int t = __float_as_int(pos4[a].w);
-                const float E = list_network<KRT, KAT, HB>(net, s_par + t * net.stride, W.coef, lane, G0, G1,
+                const float E = list_network<KRT, KAT, HB>(net, s_par + type * net.stride, W.coef, lane, G0, G1,
                                                            G_out ? G_out + (size_t)a * net.rec_len : nullptr, Kr, Ka,
                                                            c0, c1);
                 if (lane == 0) {
@@ -1184,20 +1285,22 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
                 c0 *= 2.0f;
                 c1 *= 2.0f;
             }
-            if (lane < KRT + KAT) reinterpret_cast<float4 *>(W.coef)[lane] = make_float4(c0, c0, c1, c1);
+            if (lane < KRT + KAT) reinterpret_cast<float2 *>(W.coef)[lane] = make_float2(c0, c1);
             __syncwarp();
 
             // ---- 4. the chain rule: (V, B) of every angular entry
             if constexpr (kSh) {
-                sh_gradients<KRT, KAT>(nang, W, quad, s_sh, lane);
+                sh_gradients<KRT, KAT>(nang, W, coef, s_sh, lane);
             } else if (nang <= 32) {
-                const float4 V = ring_backward<KAT, EXACT>(nang, Ka, W, quad + KRT, lane);
+                const float4 V = ring_backward<KAT, EXACT>(nang, Ka, W, coef + KRT, lane);
                 __syncwarp();
                 if (lane < nang) W.a_g[lane] = V;
             } else {
-                blocks_backward<KAT, EXACT>(nang, Ka, W, quad + KRT, lane);
+                blocks_backward<KAT, EXACT>(nang, Ka, W, coef + KRT, lane);
             }
             __syncwarp();
+            next = __shfl_sync(kFull, next, 0);
+            fetch(next);
             // every entry: two rounds at a time, their Clenshaw sums packed
             float fix = 0.f, fiy = 0.f, fiz = 0.f;
             const float k2 = 2.0f * inv_rcr;
@@ -1207,8 +1310,7 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
             }
             for (int r = 0; r < nrounds; r += 2) {
                 int ka, kb;
-                const bool va = list_round(r, nra, nang, nrest, nb, lane, ka);
-                const bool vb = list_round(r + 1, nra, nang, nrest, nb, lane, kb) && r + 1 < nrounds;
+                const bool va = rounds.at(r, ka), vb = rounds.at(r + 1, kb);  // (none past the last round)
                 float4 ea = make_float4(1.f, 0.f, 0.f, 1.f), eb = ea;
                 int ja = 0, jb = 0;
                 if (va) {
@@ -1221,7 +1323,7 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
                 }
                 const float2 x = make_float2(2.0f * ea.w * inv_rcr - 1.0f, 2.0f * eb.w * inv_rcr - 1.0f);
                 float2 S, dS;
-                clenshaw_quads<KRT, EXACT>(x, make_float2(s_tw[ja >> 28], s_tw[jb >> 28]), quad, Kr, S, dS);
+                clenshaw_shared<KRT, EXACT>(x, make_float2(s_tw[ja >> 28], s_tw[jb >> 28]), coef, Kr, S, dS);
                 auto entry = [&](bool v, const float4 &e, int j, float S1, float dS1, int round, int k) {
                     float fc, dfc;
                     radial_cutoff(e.w, inv_rcr, fc, dfc);
@@ -1286,7 +1388,7 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
             }
         }
         __syncwarp();
-        a = __shfl_sync(kFull, next, 0);
+        a = next;
     }
 
     // ---- the CTA's partial sums

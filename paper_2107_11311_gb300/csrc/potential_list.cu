@@ -28,7 +28,7 @@ cudaError_t launch_build(Context &c, const Grid &g, int n, int a_lo, int a_hi, b
     // idle (a part restages the neighbourhood); a part has at least 4 atoms
     const double per_cell = (double)n / std::max(1, g.ncell);
     const int parts = std::max(1, std::min((4 * std::max(1, c.n_sm) + g.ncell - 1) / std::max(1, g.ncell),
-                                           (int)(per_cell / kBuildAtoms)));
+                                           (int)(per_cell / 4.0)));
     auto kern = c.batch_sinfo ? k_list_build<true, false> : codes ? k_list_build<false, true> : k_list_build<false, false>;
     cudaError_t e = allow_max_smem(kern);
     if (e != cudaSuccess) return e;
