@@ -386,16 +386,12 @@ cudaError_t launch_sort(Context &c, const Grid &g, int n);
 cudaError_t launch_cells_batch(Context &c, int n, int total_cells, const double *pos, const int32_t *types);
 // Per-structure energy (FP64 sum of E_i) and virial (FP64 sum of cell partials)
 // into c.d_bres rows, or (when given) straight into energies[S], virials[S*9].
-cudaError_t launch_batch_reduce(Context &c, double *energies = nullptr, double *virials = nullptr);
-
-// Descriptor of every atom into c.d_G (Sec. II.B; k_potential, descriptor mode).
-cudaError_t launch_fp_forward(Context &c, const Grid &g, int n);
+// The virials come from the cells' partial rows, or with atoms from every atom's
+// (c.d_vir_atom, the list kernel).
+cudaError_t launch_batch_reduce(Context &c, bool atoms, double *energies = nullptr, double *virials = nullptr);
 
 // Per-species networks: E_i and dE/dG_i (Sec. II.A, Eq. ANN-layer), energy block partials.
 cudaError_t launch_ann(Context &c, int n);
-
-// Forces and virial partials from c.d_dEdG (the chain rule; k_potential, forces mode).
-cudaError_t launch_fp_backward(Context &c, const Grid &g, int n);
 
 // Energy and virial reductions (E = sum_i E_i, Sec. II.A) over n_eparts energy partials and the
 // cells' virial partials, and outputs in input order.
@@ -436,10 +432,12 @@ bool tc_fused_supported(const Context &c);
 cudaError_t launch_fused_tc(Context &c, const Grid &g, int n);
 // Either fused form: descriptor, networks and forces in one kernel.
 inline bool fused_path(const Context &c) { return fused_supported(c) || tc_fused_supported(c); }
-// Whether evaluations take that form: the FP32 fused form of one structure,
-// except for the pipelined kernel and MD steps asked to search the cells in the
+// Whether evaluations take that form: the FP32 fused form, except (for one
+// structure) the pipelined kernel and MD steps asked to search the cells in the
 // fused kernel.
-inline bool rows_form(const Context &c) { return fused_supported(c) && !c.pipeline && !c.cell_search && !c.batch_call; }
+inline bool rows_form(const Context &c) {
+    return fused_supported(c) && (c.batch_call || (!c.pipeline && !c.cell_search));
+}
 int ann_blocks(int n);
 
 // Forces to input order (FP64) only.

@@ -220,6 +220,11 @@ int ensure_rows(Context &c, int n) {
         c.cap_list = std::max(n, 1);
         ++c.buf_gen;
     }
+    if (c.batch_call && (n > c.cap_vir_atom || !c.d_vir_atom)) {
+        CK(grow(c.d_vir_atom, 0, 6 * (size_t)std::max(n, 1)), "cudaMalloc");
+        c.cap_vir_atom = std::max(n, 1);
+        ++c.buf_gen;
+    }
     return ensure_parts(c, (std::max(n, 1) + slice - 1) / slice);
 }
 
@@ -228,7 +233,7 @@ int check_smem(Context &c, const Grid &g) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     // + the kernel's static shared memory
-    const bool rows = rows_form(c) || (!fused_path(c) && !c.batch_call);
+    const bool rows = rows_form(c) || !fused_path(c);
     const size_t need = rows ? list_smem_bytes(c) + 4096 : potential_smem_bytes(c, g) + 1024;
     if (optin > 0 && need > (size_t)optin)
         return fail(&c, AENET_E_CAPACITY, "neighbour lists need %zu B of shared memory (limit %d B)", need, optin);
@@ -286,12 +291,8 @@ int enqueue_potential(Context &c, const Grid &g, int n, int *n_eparts) {
         c.last_vpart = c.d_vir_part;
         c.last_vparts = c.pot_parts;
     } else {
-        const bool rows = !c.batch_call;
-        int rc = AENET_OK;
-        if (!rows)
-            CK(launch_fp_forward(c, g, n), "descriptor kernel");
-        else if ((rc = enqueue_rows(c, g, n, RowsMode::descriptor)))
-            return rc;
+        int rc = enqueue_rows(c, g, n, RowsMode::descriptor);
+        if (rc) return rc;
         CK(mark(c, 3), "event");
         if (c.precision == AENET_FP32) {
             CK(launch_ann(c, n), "network kernel");
@@ -301,13 +302,7 @@ int enqueue_potential(Context &c, const Grid &g, int n, int *n_eparts) {
             *n_eparts = tcgen05_eparts(c, n);
         }
         CK(mark(c, 4), "event");
-        if (!rows) {
-            CK(launch_fp_backward(c, g, n), "force kernel");
-            c.last_vpart = c.d_vir_part;
-            c.last_vparts = c.pot_parts;
-        } else if ((rc = enqueue_rows(c, g, n, RowsMode::forces))) {
-            return rc;
-        }
+        if ((rc = enqueue_rows(c, g, n, RowsMode::forces))) return rc;
         c.last_epart = c.d_e_part;
         c.last_eparts = *n_eparts;
     }
@@ -713,7 +708,7 @@ int batch_enqueue(Context &c, const BatchLayout &L, const StructInfo *sinfo, con
     cudaError_t e = launch_cells_batch(c, L.n, L.gall.ncell, dpos, dtypes);
     int n_eparts = 0;
     if (e == cudaSuccess) rc = enqueue_potential(c, L.gall, L.n, &n_eparts);
-    if (e == cudaSuccess && !rc) e = launch_batch_reduce(c, energies, virials);
+    if (e == cudaSuccess && !rc) e = launch_batch_reduce(c, rows_form(c) || !fused_path(c), energies, virials);
     if (e == cudaSuccess && !rc) e = launch_finalize_forces(c, L.n, dF);
     c.batch_sinfo = nullptr;
     c.batch_order = nullptr;
@@ -894,8 +889,9 @@ extern "C" int aenet_batch_prepare(aenet_ctx *h, int n_struct, const int64_t *at
     c.plan.forces = forces;
     c.plan.virials = virials;
 
-    // Candidate launches: one CTA per cell in index order, or persistent CTAs
-    // taking cells heaviest first; staging tiles of 256 ... 2048 image-atoms.
+    // Candidate launches: staging tiles of 256 ... 2048 image-atoms (of the list
+    // build, or of the fused kernel in the tensor-core forms), and for the latter
+    // one CTA per cell in index order or persistent CTAs taking cells heaviest first.
     struct Cand {
         bool persist;
         int tile;
@@ -904,7 +900,8 @@ extern "C" int aenet_batch_prepare(aenet_ctx *h, int n_struct, const int64_t *at
     std::vector<Cand> cands;
     const bool tune = (flags & AENET_BATCH_AUTOTUNE) != 0;
     if (tune) {
-        for (int p = 0; p < 2; ++p)
+        const bool lists = rows_form(c) || !fused_path(c);  // (its list kernel is persistent)
+        for (int p = lists ? 1 : 0; p < 2; ++p)
             for (int tile : {256, 512, 1024, 2048}) cands.push_back({p == 1, tile, 0.f});
     } else {
         cands.push_back({true, c.caps.tile, 0.f});

@@ -378,6 +378,46 @@ __global__ void k_batch_reduce(int n_struct, const StructInfo *__restrict__ sinf
     }
 }
 
+// The same from every atom's energy and virial (six sums, the list kernel): one
+// CTA per structure, a thread's atoms in FP64 and then a tree, in a fixed order.
+constexpr int kBatchThreads = 128;
+__global__ void __launch_bounds__(kBatchThreads)
+    k_batch_reduce_atoms(const StructInfo *__restrict__ sinfo, const int *__restrict__ cell_start,
+                         const float *__restrict__ eatom, const float *__restrict__ vir_atom,
+                         double *__restrict__ out, double *__restrict__ energies, double *__restrict__ virials) {
+    __shared__ double s_w[kBatchThreads / 32][7];
+    const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int c0 = sinfo[s].cell0, a0 = cell_start[c0], a1 = cell_start[c0 + sinfo[s].ncell];
+    double v[7] = {};
+    for (int k = a0 + tid; k < a1; k += kBatchThreads) {
+        v[0] += (double)eatom[k];
+        const float2 *w = reinterpret_cast<const float2 *>(vir_atom + (size_t)k * 6);
+        const float2 x = w[0], y = w[1], z = w[2];
+        v[1] += (double)x.x;
+        v[2] += (double)x.y;
+        v[3] += (double)y.x;
+        v[4] += (double)y.y;
+        v[5] += (double)z.x;
+        v[6] += (double)z.y;
+    }
+#pragma unroll
+    for (int q = 0; q < 7; ++q) {
+        v[q] = warp_sum_d(v[q]);
+        if (lane == 0) s_w[warp][q] = v[q];
+    }
+    __syncthreads();
+    if (tid < 10) {  // energy, then the symmetric virial (xx xy xz yy yz zz) as nine entries
+        const int q = tid - 1, lo = q < 0 ? 0 : min(q / 3, q % 3), hi = q < 0 ? 0 : max(q / 3, q % 3);
+        const int k = q < 0 ? 0 : 1 + (lo == 0 ? hi : lo == 1 ? 2 + hi : 5);
+        double t = 0.0;
+#pragma unroll
+        for (int w = 0; w < kBatchThreads / 32; ++w) t += s_w[w][k];
+        if (out) out[(size_t)s * 10 + tid] = t;
+        if (tid == 0 && energies) energies[s] = t;
+        if (tid > 0 && virials) virials[(size_t)s * 9 + q] = t;
+    }
+}
+
 bool thermostat_on(const Context &c) { return c.thermo_tau > 0.0 && c.d_lambda; }
 
 Thermostat thermostat(const Context &c, int n) {
@@ -429,9 +469,14 @@ cudaError_t launch_unsort_G(Context &c, int n, float *G) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_batch_reduce(Context &c, double *energies, double *virials) {
+cudaError_t launch_batch_reduce(Context &c, bool atoms, double *energies, double *virials) {
     const int per = kRedThreads / 32;
     double *rows = (energies || virials) ? nullptr : c.d_bres;
+    if (atoms) {
+        k_batch_reduce_atoms<<<c.batch_n, kBatchThreads, 0, c.stream>>>(c.batch_sinfo, c.d_cell_start, c.d_eatom,
+                                                                        c.d_vir_atom, rows, energies, virials);
+        return cudaGetLastError();
+    }
     k_batch_reduce<<<(c.batch_n + per - 1) / per, kRedThreads, 0, c.stream>>>(
         c.batch_n, c.batch_sinfo, c.d_cell_start, c.d_eatom, c.d_vir_part, rows, energies, virials);
     return cudaGetLastError();

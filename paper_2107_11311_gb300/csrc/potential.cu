@@ -1,6 +1,6 @@
-// Cell-list evaluation with the potential kernel: launch of its fused,
-// descriptor-only and forces-only forms (single structures and batches), and
-// the allocation-free descriptor entry point. The kernels themselves are in
+// Evaluation by the potential kernel that searches the cells itself: launch of
+// its fused and pipelined FP32 forms (one structure), and the allocation-free
+// descriptor entry point. The kernels themselves are in
 // potential_kernels.cuh.
 #include <stdio.h>
 
@@ -118,19 +118,6 @@ cudaError_t launch_fused_potential(Context &c, const Grid &g, int n) {
     return dispatch<kFused>(c, g);
 }
 
-cudaError_t launch_fp_forward(Context &c, const Grid &g, int n) {
-    (void)n;
-    cudaError_t e = cudaMemsetAsync(c.d_stats, 0, sizeof(unsigned long long) * 4, c.stream);
-    if (e != cudaSuccess) return e;
-    return dispatch<kDescriptor>(c, g);
-}
-
-cudaError_t launch_fp_backward(Context &c, const Grid &g, int n) {
-    cudaError_t e = cudaMemsetAsync(c.d_F4, 0, sizeof(float4) * (size_t)(n > 0 ? n : 1), c.stream);
-    if (e != cudaSuccess) return e;
-    return dispatch<kForces>(c, g);
-}
-
 }  // namespace aenet
 
 // ---------------------------------------------------------------------------
@@ -218,7 +205,7 @@ cudaError_t na_launch_fp(const Basis &B, const Grid &g, const Caps &caps, cudaSt
     if (e != cudaSuccess) return e;
     kern<<<g.ncell, kPThreads, smem, st>>>(B, net, g, nullptr, 0, caps, pos4, cell_start, nullptr, nullptr, nullptr,
                                            nullptr,
-                                           nullptr, Gs, nullptr, nullptr, nullptr, stats, err, nullptr, nullptr,
+                                           nullptr, Gs, nullptr, nullptr, stats, err, nullptr, nullptr,
                                            g.ncell, 1, 0, TcNet{});
     return cudaGetLastError();
 }

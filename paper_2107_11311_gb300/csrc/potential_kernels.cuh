@@ -26,9 +26,7 @@
 // need no division or transcendental call. Energy and virial leave as FP64
 // per-CTA partials, reduced in a fixed order by the reduction kernel.
 //
-// The same kernel in two other modes serves the split path (the BF16 network
-// forms, networks wider than 32, the descriptor-only API): kDescriptor writes
-// the G rows, kForces reads dE/dG rows and applies steps 1 and 4 only.
+// MODE kDescriptor writes the G rows only (the allocation-free entry point).
 #pragma once
 
 #include <stdio.h>
@@ -50,11 +48,11 @@ constexpr int kPWarps = 8;
 constexpr int kPThreads = kPWarps * 32;
 constexpr int kSlots = 64;
 
-// What one launch of k_potential computes.
+// What one launch of k_potential or k_potential_list computes.
 enum Mode : int {
     kFused = 0,       // descriptor -> FP32 network -> forces, energy and virial
     kDescriptor = 1,  // descriptor only: G rows (sorted order)
-    kForces = 2,      // forces and virial from given dE/dG rows (sorted order)
+    kForces = 2,      // forces and virial from given dE/dG rows (sorted order; list kernel)
     kFusedTC = 3,     // descriptor -> BF16 tensor-core network -> forces (one geometry pass)
     kFusedTCx3 = 4    // the same with split-BF16 operands (hi*hi + hi*lo + lo*hi)
 };
@@ -829,12 +827,11 @@ __device__ __forceinline__ void process_atom(int i_s, int nnb, int nang, const B
                                              const float *s_par, const float *s_tw, const float *s_sh,
                                              const WarpLists &W, int lane,
                                              const float4 *__restrict__ pos4, float4 *__restrict__ F4,
-                                             float *__restrict__ eatom, float *__restrict__ G_out,
-                                             const float *__restrict__ dEdG_in, double &e_acc, float (&vir)[9]) {
+                                             float *__restrict__ eatom, float *__restrict__ G_out, double &e_acc,
+                                             float (&vir)[9]) {
     const int Kr = EXACT ? KRT : B.Kr;
     const int Ka = EXACT ? KAT : B.Ka;
     const int s0 = 2 * lane, s1 = 2 * lane + 1;  // slots of the lane's dE/dG coefficients
-    if constexpr (MODE != kForces) {
     float G0, G1;  // descriptor slots g0, g1
     atom_descriptor<KRT, KAT, EXACT>(nnb, nang, B, s_tw, s_sh, W, lane, G0, G1);
     const int g0 = desc_slot0<KRT, KAT>(lane), g1 = desc_slot1<KRT, KAT>(lane);
@@ -974,20 +971,9 @@ __device__ __forceinline__ void process_atom(int i_s, int nnb, int nang, const B
         e_acc += (double)E;
         eatom[i_s] = E;
     }
-    }  // MODE == kFused
-    }  // MODE != kForces
-    if constexpr (MODE == kForces) {  // dE/dG given: scatter the row into the slot layout
-        const int D = 2 * (Kr + Ka);
-        const int c0 = slot_col<KRT, KAT>(s0, Kr, Ka), c1 = slot_col<KRT, KAT>(s1, Kr, Ka);
-        W.coef[s0] = c0 >= 0 ? dEdG_in[(size_t)i_s * D + c0] : 0.f;
-        W.coef[s1] = c1 >= 0 ? dEdG_in[(size_t)i_s * D + c1] : 0.f;
-        // the spherical-harmonic chain rule needs the atom's component sums,
-        // which no descriptor pass has left in this launch
-        if constexpr (sh_angular<KRT, KAT, EXACT>()) sh_component_sums(nang, W, lane);
-    }
     __syncwarp();
-
     atom_chain_rule<KRT, KAT, EXACT>(i_s, nnb, nang, B, s_tw, s_sh, W, W.coef, lane, F4, vir);
+    }  // MODE == kFused
 }
 
 // The network parameters of every species into the shared-memory layout of
@@ -1260,7 +1246,7 @@ __global__ void __launch_bounds__(NW * 32, NW == kPWarps ? 2 : 1)
                 const float4 *__restrict__ pos4,
                 const int *__restrict__ cell_start, const float *__restrict__ params, const float *__restrict__ shift,
                 const float *__restrict__ scale, float4 *__restrict__ F4, float *__restrict__ eatom,
-                float *__restrict__ G_out, const float *__restrict__ dEdG_in, double *__restrict__ e_part,
+                float *__restrict__ G_out, double *__restrict__ e_part,
                 double *__restrict__ vir_part, unsigned long long *__restrict__ stats, unsigned *__restrict__ err,
                 unsigned *__restrict__ work, const int *__restrict__ order, int n_items, int split, int split_from,
                 TcNet tc) {
@@ -1688,7 +1674,7 @@ __global__ void __launch_bounds__(NW * 32, NW == kPWarps ? 2 : 1)
             scan_tile(s_pos, s_idx, staged, ui, i_s, B, caps, W, lane, nnb);
             finish_list(nnb, nang);
             process_atom<KRT, KAT, EXACT, MODE, HB>(i_s, nnb, nang, B, net, s_par, s_tw, s_sh, W, lane, pos4, F4,
-                                                    eatom, G_out, dEdG_in, e_acc, vir);
+                                                    eatom, G_out, e_acc, vir);
         }
     } else {
         const int n_rounds = (cnt + NW - 1) / NW;
@@ -1710,13 +1696,13 @@ __global__ void __launch_bounds__(NW * 32, NW == kPWarps ? 2 : 1)
             if (active) {
                 finish_list(nnb, nang);
                 process_atom<KRT, KAT, EXACT, MODE, HB>(i_s, nnb, nang, B, net, s_par, s_tw, s_sh, W, lane, pos4, F4,
-                                                        eatom, G_out, dEdG_in, e_acc, vir);
+                                                        eatom, G_out, e_acc, vir);
             }
         }
     }
 
     // ---- cell partials: energy (FP64), virial (FP32 lanes -> FP64)
-    if constexpr (MODE == kFused || MODE == kForces || kTC) {
+    if constexpr (MODE == kFused || kTC) {
     #pragma unroll
         for (int k = 0; k < 9; ++k) {
             const float v = warp_sum(vir[k]);
@@ -1738,7 +1724,7 @@ __global__ void __launch_bounds__(NW * 32, NW == kPWarps ? 2 : 1)
     }
     }  // work items
     if (work && tid == 0) release_work_counter(work);  // every thread has left the loop
-    if (MODE != kForces && lane == 0 && st_nb) {  // statistics
+    if (lane == 0 && st_nb) {  // statistics
         atomicAdd(&stats[0], st_nb);
         atomicAdd(&stats[1], st_ang);
         atomicAdd(&stats[2], st_pairs);

@@ -1,7 +1,7 @@
-// Launch of the cell-list potential kernel in any of its modes (shared by the
-// translation units that instantiate them: potential.cu for the FP32 fused,
-// descriptor and force modes, potential_tc.cu for the tensor-core modes, so
-// that the two compile in parallel).
+// Launch of the cell-list potential kernel in its fused modes (shared by the
+// translation units that instantiate them: potential.cu for the FP32 network,
+// potential_tc.cu for the tensor-core networks, so that the two compile in
+// parallel).
 #pragma once
 
 #include <algorithm>
@@ -33,41 +33,40 @@ TcNet make_tc_net(const Context &c, const FusedNet &net) {
 template <int KRT, int KAT, bool EXACT, int MODE>
 cudaError_t launch_mode(Context &c, const Grid &g, const FusedNet &net) {
     constexpr bool tc = is_tc_mode(MODE);
-    const int n_sp = (MODE == kFused || tc) ? c.basis.n_species : 0;
+    const int n_sp = c.basis.n_species;
     size_t smem = make_playout(g.n_off, c.caps.tile, c.caps.nb, c.caps.ang, n_sp, tc ? kTcParStride : net.stride,
                                kPWarps, tc)
                       .total;
-    // the network's hidden-width bound is a template argument of the fused forms only
-    auto kern = c.batch_sinfo ? k_potential<KRT, KAT, EXACT, MODE, true, 32> : k_potential<KRT, KAT, EXACT, MODE, false, 32>;
+    // the network's hidden-width bound is a template argument; FP32 batches are
+    // evaluated over lists (potential_list.cu), so only the tensor-core modes have
+    // a batched form here
+    auto kern = k_potential<KRT, KAT, EXACT, MODE, false, 32>;
     int nw = kPWarps;
     if constexpr (tc) {
-        if (net.hb == 16)
-            kern = c.batch_sinfo ? k_potential<KRT, KAT, EXACT, MODE, true, 16>
-                                 : k_potential<KRT, KAT, EXACT, MODE, false, 16>;
-    }
-    if constexpr (MODE == kFused) {
-        if (net.hb == 16) {
-            kern = c.batch_sinfo ? k_potential<KRT, KAT, EXACT, MODE, true, 16>
-                                 : k_potential<KRT, KAT, EXACT, MODE, false, 16>;
-        } else if (smem > kTwoCtaSmem) {
-            // one CTA per SM anyway (wide networks of several species): give it
-            // 12 warps instead of 8 if their lists fit
-            int dev = 0, optin = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-            const size_t smem12 = make_playout(g.n_off, c.caps.tile, c.caps.nb, c.caps.ang, n_sp, net.stride, 12).total;
-            if (smem12 + 1024 <= (size_t)optin) {
-                nw = 12;
-                smem = smem12;
-                kern = c.batch_sinfo ? k_potential<KRT, KAT, EXACT, MODE, true, 32, 12>
-                                     : k_potential<KRT, KAT, EXACT, MODE, false, 32, 12>;
-            }
+        if (c.batch_sinfo)
+            kern = net.hb == 16 ? k_potential<KRT, KAT, EXACT, MODE, true, 16> : k_potential<KRT, KAT, EXACT, MODE, true, 32>;
+        else if (net.hb == 16)
+            kern = k_potential<KRT, KAT, EXACT, MODE, false, 16>;
+    } else if (c.batch_sinfo) {
+        return cudaErrorInvalidValue;
+    } else if (net.hb == 16) {
+        kern = k_potential<KRT, KAT, EXACT, MODE, false, 16>;
+    } else if (smem > kTwoCtaSmem) {
+        // one CTA per SM anyway (wide networks of several species): give it
+        // 12 warps instead of 8 if their lists fit
+        int dev = 0, optin = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        const size_t smem12 = make_playout(g.n_off, c.caps.tile, c.caps.nb, c.caps.ang, n_sp, net.stride, 12).total;
+        if (smem12 + 1024 <= (size_t)optin) {
+            nw = 12;
+            smem = smem12;
+            kern = k_potential<KRT, KAT, EXACT, MODE, false, 32, 12>;
         }
     }
     cudaError_t e = allow_max_smem(kern);
     if (e != cudaSuccess) return e;
-    // activation records (fused forms) / G rows
-    float *rows = (MODE == kFused || tc) ? (c.keep_act ? c.d_act : nullptr) : c.d_G;
+    float *rows = c.keep_act ? c.d_act : nullptr;  // activation records
     const TcNet tn = tc ? make_tc_net(c, net) : TcNet{};
     // one structure: (some) cells split into parts (persistent CTAs); batches: whole cells
     int split_from = 0;
@@ -86,8 +85,8 @@ cudaError_t launch_mode(Context &c, const Grid &g, const FusedNet &net) {
     }
     kern<<<grid, nw * 32, smem, c.stream>>>(c.basis, net, g, c.batch_sinfo, c.batch_n, c.caps, c.d_pos4,
                                               c.d_cell_start, c.d_params,
-                                              c.d_shift, c.d_scale, c.d_F4, c.d_eatom, rows, c.d_dEdG,
-                                              c.d_e_part, c.d_vir_part, c.d_stats, c.d_err, work,
+                                              c.d_shift, c.d_scale, c.d_F4, c.d_eatom, rows, c.d_e_part,
+                                              c.d_vir_part, c.d_stats, c.d_err, work,
                                               (work && c.batch_sinfo) ? c.batch_order : nullptr, n_items, split,
                                               split_from, tn);
     c.last_grid = grid;

@@ -22,13 +22,15 @@ int build_tile(const Context &c, const Grid &g, int n) {
 }
 
 cudaError_t launch_build(Context &c, const Grid &g, int n, int a_lo, int a_hi, bool codes, bool clear) {
-    const int tile = build_tile(c, g, n);
+    const int tile = c.batch_sinfo ? c.caps.tile : build_tile(c, g, n);  // (batches: the tuned tile)
     const size_t smem = make_build_layout(g.n_off, tile).total;
     // with few cells each is divided, so that the build does not leave most SMs
     // idle (a part restages the neighbourhood); a part has at least 4 atoms
     const double per_cell = (double)n / std::max(1, g.ncell);
-    const int parts = std::max(1, std::min((4 * std::max(1, c.n_sm) + g.ncell - 1) / std::max(1, g.ncell),
-                                           (int)(per_cell / 4.0)));
+    const int parts =
+        c.batch_sinfo ? 1
+                      : std::max(1, std::min((4 * std::max(1, c.n_sm) + g.ncell - 1) / std::max(1, g.ncell),
+                                             (int)(per_cell / 4.0)));
     auto kern = c.batch_sinfo ? k_list_build<true, false> : codes ? k_list_build<false, true> : k_list_build<false, false>;
     cudaError_t e = allow_max_smem(kern);
     if (e != cudaSuccess) return e;
@@ -79,11 +81,16 @@ cudaError_t launch_list(Context &c, const Grid &g, const ListLaunch &q, int *par
     const int n = q.a_hi - q.a_lo;
     const int nw = list_warps(c, L.warp_base, L.warp_bytes, n, most);
     if (nw <= 0) return cudaErrorInvalidConfiguration;
+    const bool batch = c.batch_sinfo != nullptr;
     auto kern = k_potential_list<KRT, KAT, EXACT, kFused, 32, false, false>;
     if (q.mode == kDescriptor)
         kern = k_potential_list<KRT, KAT, EXACT, kDescriptor, 32, false, false>;
     else if (q.mode == kForces)
-        kern = k_potential_list<KRT, KAT, EXACT, kForces, 32, false, false>;
+        kern = batch ? k_potential_list<KRT, KAT, EXACT, kForces, 32, false, true>
+                     : k_potential_list<KRT, KAT, EXACT, kForces, 32, false, false>;
+    else if (batch)
+        kern = net.hb == 32 ? k_potential_list<KRT, KAT, EXACT, kFused, 32, false, true>
+                            : k_potential_list<KRT, KAT, EXACT, kFused, 16, false, true>;
     else if (q.codes)
         kern = net.hb == 32 ? k_potential_list<KRT, KAT, EXACT, kFused, 32, true, false>
                             : k_potential_list<KRT, KAT, EXACT, kFused, 16, true, false>;

@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(kPipeWarps * 32, 1)
         st_pairs += (unsigned long long)(nang * (nang - 1) / 2);
         __syncwarp();
         process_atom<KRT, KAT, EXACT, kFused, HB>(i_s, nnb, nang, B, net, s_par, s_tw, s_sh, W, lane, pos4, F4, eatom,
-                                                  rec_out, nullptr, e_acc, vir);
+                                                  rec_out, e_acc, vir);
         __syncwarp();
         if (lane == 0) {
             __threadfence_block();  // this atom's reads of the buffer are done
