@@ -21,19 +21,19 @@ namespace aenet {
 namespace {
 
 constexpr int kGThreads = 256;
-constexpr int kGChunk = 512;   // atoms per CTA
+constexpr int kGChunk = 512;   // atoms per CTA, at most
 constexpr int kGTile = 32;     // atoms staged at a time
 constexpr int kGMaxJ = 16;     // parameters per thread: n_params <= 16 * 256
 
 __global__ void __launch_bounds__(kGThreads)
     k_dEdW_partial(int n, int n_species, int n_params, int rec_len, const int *__restrict__ list,
                    const int *__restrict__ sp_off, const float *__restrict__ act, const int2 *__restrict__ pairs,
-                   float *__restrict__ partial, int n_chunks) {
+                   float *__restrict__ partial, int n_chunks, int per_chunk) {
     extern __shared__ float tile[];  // [kGTile][rec_len]
     const int chunk = blockIdx.x, t = blockIdx.y, tid = threadIdx.x;
     const int off = sp_off[t];
     const int cnt = (t + 1 < n_species ? sp_off[t + 1] : n) - off;
-    const int a0 = chunk * kGChunk, a1 = min(cnt, a0 + kGChunk);
+    const int a0 = chunk * per_chunk, a1 = min(cnt, a0 + per_chunk);
     float acc[kGMaxJ];
     int2 pr[kGMaxJ];
 #pragma unroll
@@ -75,12 +75,19 @@ __global__ void k_dEdW_reduce(int n_species, int n_params, int n_chunks, const f
     if (idx >= n_species * n_params) return;
     const int t = idx / n_params, w = idx % n_params;
     double s0 = 0.0, s1 = 0.0;
+    const float *p = partial + (size_t)t * n_chunks * n_params + w;
     int c = 0;
-    for (; c + 1 < n_chunks; c += 2) {
-        s0 += (double)partial[((size_t)t * n_chunks + c) * n_params + w];
-        s1 += (double)partial[((size_t)t * n_chunks + c + 1) * n_params + w];
+    for (; c + 7 < n_chunks; c += 8) {  // eight loads in flight
+        float v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = p[(size_t)(c + k) * n_params];
+#pragma unroll
+        for (int k = 0; k < 8; k += 2) {
+            s0 += (double)v[k];
+            s1 += (double)v[k + 1];
+        }
     }
-    if (c < n_chunks) s0 += (double)partial[((size_t)t * n_chunks + c) * n_params + w];
+    for (; c < n_chunks; ++c) s0 += (double)p[(size_t)c * n_params];
     out[idx] = s0 + s1;
 }
 
@@ -110,7 +117,11 @@ std::vector<int2> grad_pairs(const Net &net) {
 
 cudaError_t launch_grad_weights(Context &c, int n) {
     const int ns = c.basis.n_species, np = c.net.n_params, rec = activation_record_len(c.net);
-    const int n_chunks = std::max(1, (n + kGChunk - 1) / kGChunk);
+    // Atoms per CTA: about 64 CTAs per species for small systems, whose time is a
+    // CTA's serial pass over its atoms (192 atoms, 2 species: 82 us with 512 atoms a
+    // CTA, 8.4 us with 8), at least 8 and at most 512 of them.
+    const int per_chunk = std::max(8, std::min(kGChunk, (n + 63) / 64));
+    const int n_chunks = std::max(1, (n + per_chunk - 1) / per_chunk);
     const size_t need = (size_t)ns * n_chunks * np;
     cudaError_t e;
     if (need > c.cap_wpart || !c.d_wpart) {
@@ -124,7 +135,7 @@ cudaError_t launch_grad_weights(Context &c, int n) {
     const size_t smem = sizeof(float) * kGTile * rec;
     if ((e = allow_max_smem(k_dEdW_partial)) != cudaSuccess) return e;
     k_dEdW_partial<<<dim3(n_chunks, ns), kGThreads, smem, c.stream>>>(
-        n, ns, np, rec, c.d_sp_list, c.d_sp_off, c.d_act, c.d_wpairs, c.d_wpart, n_chunks);
+        n, ns, np, rec, c.d_sp_list, c.d_sp_off, c.d_act, c.d_wpairs, c.d_wpart, n_chunks, per_chunk);
     k_dEdW_reduce<<<(ns * np + 255) / 256, 256, 0, c.stream>>>(ns, np, n_chunks, c.d_wpart, c.d_dEdW);
     return cudaGetLastError();
 }
