@@ -367,9 +367,9 @@ class AenetGPU:
         self._check(self.lib.aenet_set_option(self.h, int(option), int(value)))
 
     def fuse_network(self, on=True):
-        """BF16 forms: run the tensor-core networks inside the fused potential
-        kernel (default) or as the three-kernel path (descriptor kernel, network
-        kernel, force kernel)."""
+        """BF16 forms: run the tensor-core networks of up to 4,096 atoms inside the
+        fused potential kernel (default), or always as the three-kernel path
+        (descriptor kernel, network kernel, force kernel)."""
         self.set_option(AENET_OPT_FUSED_NETWORK, 1 if on else 0)
 
     def pipeline(self, on=True):

@@ -163,6 +163,7 @@ struct Context {
     bool own_stream = false;
     int precision = AENET_FP32;
     bool fuse_network = true;      // BF16 forms: tensor-core network inside the fused kernel
+    int eval_n = 0;                // atoms of the evaluation being set up (tc_fused_supported)
     bool batch_call = false;       // set during the batch entry points
     bool cell_search = false;      // set while an MD step with AENET_MD_LIST_OFF is enqueued
     bool pipeline = false;         // FP32 fused form: the pipelined kernel (one CTA of 16 warps per SM)
@@ -246,6 +247,7 @@ struct Context {
     // itself) or _ON (2: the exact list is built in every step and the list kernel evaluates it)
     int md_list = 0;
     bool last_list = false;            // the captured MD step takes the list form of AENET_OPT_MD_LIST
+    bool last_fused = false;           // the captured MD step runs a fused kernel
     bool last_rows = false;            // ... or builds lists in every step as aenet_compute does
     // tilt factors xy, xz, yz of the restricted triclinic cell of single-structure
     // calls (zero: orthorhombic)
@@ -426,12 +428,20 @@ bool pipe_supported(const Context &c, const Grid &g);
 bool fused_supported(const Context &c);
 cudaError_t launch_fused_potential(Context &c, const Grid &g, int n);
 // Fused kernel with the networks on the tensor cores (BF16 forms; two hidden
-// layers <= 32 wide; the water (16, 8) and solid (20, 6) bases), unless the
-// context asked for the three-kernel path (AENET_OPT_FUSED_NETWORK 0).
+// layers <= 32 wide; the water (16, 8) and solid (20, 6) bases; c.eval_n at most
+// kTcFusedAtoms or kTcFusedAtomsSolid), unless the context asked for the three-kernel path
+// (AENET_OPT_FUSED_NETWORK 0).
 bool tc_fused_supported(const Context &c);
 cudaError_t launch_fused_tc(Context &c, const Grid &g, int n);
 // Either fused form: descriptor, networks and forces in one kernel.
 inline bool fused_path(const Context &c) { return fused_supported(c) || tc_fused_supported(c); }
+// Atoms up to which the BF16 forms run the networks inside the potential kernel:
+// its one launch wins where launches count, the three kernels over neighbour lists
+// where the chip is full. Split BF16, one evaluation, fused against three kernels
+// (us): water 1,536 77 / 103, 3,072 121 / 124, 6,144 142 / 133, 12,288 188 / 160,
+// 98,304 920 / 627, 331,776 2955 / 1929; the solid's cells hold more work per
+// atom: 2,000 189 / 135, 27,000 668 / 367.
+constexpr int kTcFusedAtoms = 4096, kTcFusedAtomsSolid = 1024;
 // Whether evaluations take that form: the FP32 fused form, except (for one
 // structure) the pipelined kernel and MD steps asked to search the cells in the
 // fused kernel.

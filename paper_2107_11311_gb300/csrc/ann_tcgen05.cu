@@ -80,15 +80,17 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a, uint64_t 
         "l"(a), "l"(b), "r"(idesc), "r"(acc));
 }
 
-// D[128 x N] (+)= A[128 x K] B[N x K]^T over K / 16 steps; split products when X3.
+// D[128 x N] (+)= A[128 x K] B[N x K]^T over K / 16 steps (added to D's contents
+// when add); split products when X3.
 template <bool X3>
 __device__ __forceinline__ void umma_gemm(uint32_t d_tmem, uint32_t a_hi, uint32_t a_lo, uint32_t b_hi,
-                                          uint32_t b_lo, int K, int N) {
+                                          uint32_t b_lo, int K, int N, bool add) {
     const uint32_t idesc = umma_idesc(kURows, N);
     const uint32_t a_sbo = (K >> 3) << 7, b_sbo = a_sbo;
     for (int ks = 0; ks < K / 16; ++ks) {
         const uint32_t step = ks * 256;
-        umma_bf16(d_tmem, umma_desc(a_hi + step, 128, a_sbo), umma_desc(b_hi + step, 128, b_sbo), idesc, ks > 0);
+        umma_bf16(d_tmem, umma_desc(a_hi + step, 128, a_sbo), umma_desc(b_hi + step, 128, b_sbo), idesc,
+                  add || ks > 0);
         if (X3) {
             umma_bf16(d_tmem, umma_desc(a_hi + step, 128, a_sbo), umma_desc(b_lo + step, 128, b_sbo), idesc, 1);
             umma_bf16(d_tmem, umma_desc(a_lo + step, 128, a_sbo), umma_desc(b_hi + step, 128, b_sbo), idesc, 1);
@@ -139,6 +141,21 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// The same 32 values (read-only global memory) into 32 columns of every thread's TMEM lane.
+__device__ __forceinline__ void tmem_fill32(uint32_t taddr, const float *v) {
+    uint32_t r[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__ldg(v + i));
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};\n" ::"r"(taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]),
+        "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]),
+        "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+        : "memory");
 }
 
 // Row `row` (K = 32 values) of an A operand, split into hi and lo parts.
@@ -264,11 +281,11 @@ __global__ void __launch_bounds__(kUThreads, 3) k_ann_tcgen05(AnnTcArgs a) {
     int cur_t = -1;
     double e_cta = 0.0;
 
-    auto run = [&](uint32_t d_col, int a_off, int a_K, int b_off, int b_rows, int K, int N) {
+    auto run = [&](uint32_t d_col, int a_off, int a_K, int b_off, int b_rows, int K, int N, bool add = false) {
         if (tid == 0) {
             tc_fence_after();
             umma_gemm<X3>(tmem + d_col, base + a_off, base + a_off + kURows * a_K * 2, base + b_off,
-                          base + b_off + b_rows * K * 2, K, N);
+                          base + b_off + b_rows * K * 2, K, N, add);
             umma_commit(mbar);
         }
         ok = mbar_wait(mbar, phase) && ok;
@@ -305,6 +322,15 @@ __global__ void __launch_bounds__(kUThreads, 3) k_ann_tcgen05(AnnTcArgs a) {
                     : "memory");
             }
             cur_t = t;
+        }
+        // ---- the biases of layers 1 and 2 into their accumulators (columns 0..63; the
+        // previous tile's reads of them are over): the sums then start from the bias,
+        // as in the fused kernel, and the tensor cores' rounding of them is the same
+        {
+            const float *gb = reinterpret_cast<const float *>(a.wtc + (size_t)t * kWtcBytes + (kBias - kB1));
+            tmem_fill32(lane_addr + 0, gb);
+            tmem_fill32(lane_addr + 32, gb + kUHid);
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         }
         // ---- row tid: the standardised descriptor g of its atom (A0, K = 64)
         const bool valid = tid < rows;
@@ -359,23 +385,23 @@ __global__ void __launch_bounds__(kUThreads, 3) k_ann_tcgen05(AnnTcArgs a) {
         }
         float x1[kUHid];
         float v[32];
-        // ---- layer 1: Z1 = g W1^T (TMEM columns 0..31)
-        run(0, kA0, 64, kB1, 32, 64, 32);
+        // ---- layer 1: Z1 = b1 + g W1^T (TMEM columns 0..31)
+        run(0, kA0, 64, kB1, 32, 64, 32, true);
         tmem_ld32(lane_addr + 0, v);
 #pragma unroll
-        for (int j = 0; j < kUHid; ++j) x1[j] = j < H1 ? tanh_exp(v[j] + s_bias[j]) : 0.f;
+        for (int j = 0; j < kUHid; ++j) x1[j] = j < H1 ? tanh_exp(v[j]) : 0.f;
         store_row32<X3>(smem, kA1, tid, x1);
         fence_async_smem();
         tc_fence_before();
         __syncthreads();
 
-        // ---- layer 2: Z2 = X1 W2^T (columns 32..63); output layer and delta2 in FP32
-        run(32, kA1, 32, kB2, 32, 32, 32);
+        // ---- layer 2: Z2 = b2 + X1 W2^T (columns 32..63); output layer and delta2 in FP32
+        run(32, kA1, 32, kB2, 32, 32, 32, true);
         tmem_ld32(lane_addr + 32, v);
         float e = s_bias[3 * kUHid];
 #pragma unroll
         for (int j = 0; j < kUHid; ++j) {
-            const float x2 = j < H2 ? tanh_exp(v[j] + s_bias[kUHid + j]) : 0.f;
+            const float x2 = j < H2 ? tanh_exp(v[j]) : 0.f;
             const float w = s_bias[2 * kUHid + j];
             e = fmaf(w, x2, e);
             v[j] = (1.0f - x2 * x2) * w;  // delta2

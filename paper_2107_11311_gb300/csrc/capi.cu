@@ -517,6 +517,7 @@ static int compute_impl(Context &c, int n, const double *pos, const int32_t *typ
     if (n < 0) return fail(&c, AENET_E_ARG, "n_atoms < 0");
     if (!box) return fail(&c, AENET_E_ARG, "box is NULL");
     if (n > 0 && (!pos || !types)) return fail(&c, AENET_E_ARG, "pos/types NULL");
+    c.eval_n = n;
     Grid g;
     int rc = make_grid(c, box, g, 0.0, c.tilt);
     if (rc) return rc;
@@ -597,6 +598,7 @@ extern "C" int aenet_compute_async(aenet_ctx *h, int n, const double *pos, const
     for (int k = 0; k < 6; ++k)
         if ((k < 2 || arrays[k]) && !is_device_ptr(arrays[k]))
             return fail(&c, AENET_E_ARG, "aenet_compute_async takes device pointers only (argument %d)", k);
+    c.eval_n = n;
     Grid g;
     int rc = make_grid(c, box, g, 0.0, c.tilt);
     if (rc) return rc;
@@ -676,6 +678,7 @@ int batch_layout(Context &c, int n_struct, const int64_t *atom_offset, const dou
 // Work buffers and neighbour-list capacities for a batch (capacities from the
 // densest structure, staging tile from the largest neighbourhood of a cell).
 int batch_buffers(Context &c, const BatchLayout &L) {
+    c.eval_n = L.n;
     int rc;
     if ((rc = ensure(c, L.n, L.gall)) || (rc = ensure_stage(c, L.n))) return rc;
     if (c.caps.nb == 0) {
@@ -1157,6 +1160,7 @@ static int md_fixed_cell(aenet_ctx *h, int n, double *pos, double *vel, const in
     if (c.mass.empty()) return fail(&c, AENET_E_ARG, "model has no masses");
     if (n <= 0 || !pos || !vel || !types || !box) return fail(&c, AENET_E_ARG, "bad MD arguments");
     if (n_steps < 0 || !isfinite(dt)) return fail(&c, AENET_E_ARG, "bad n_steps / dt");
+    c.eval_n = n;
     const bool async = (flags & AENET_MD_ASYNC) != 0;
     const bool keep_act = c.keep_act;  // MD steps keep no activation records
     c.keep_act = false;
@@ -1295,6 +1299,7 @@ static int md_fixed_cell(aenet_ctx *h, int n, double *pos, double *vel, const in
             c.md_key.skin = c.skin;
             c.md_key.list_form = list_form;
             c.last_list = list_form;
+            c.last_fused = fused_path(c);
             c.last_rows = rows && !verlet;
             c.md_key.thermo_T0 = c.thermo_T0;
             c.md_key.thermo_tau = c.thermo_tau;
@@ -1443,7 +1448,7 @@ extern "C" int aenet_md_stage_times(aenet_ctx *h, float *ms, int *kernels_per_st
     }
     if (kernels_per_step) *kernels_per_step = c.md_kernels;
     if (path_flags)
-        *path_flags = (fused_path(c) ? AENET_PATH_FUSED : 0) | (c.last_pipe ? AENET_PATH_PIPELINED : 0) |
+        *path_flags = (c.last_fused ? AENET_PATH_FUSED : 0) | (c.last_pipe ? AENET_PATH_PIPELINED : 0) |
                       (c.last_list ? AENET_PATH_LIST : 0) | (c.last_rows ? AENET_PATH_ROWS : 0);
     return AENET_OK;
 }
