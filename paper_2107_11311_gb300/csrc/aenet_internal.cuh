@@ -192,14 +192,22 @@ struct Context {
     int *d_slot = nullptr;         // input index -> rank inside its cell
     int *d_cell_count = nullptr;   // [ncell]
     int *d_cell_start = nullptr;   // [ncell + 1]
-    float *d_G = nullptr;          // [n * D] sorted order
-    float *d_dEdG = nullptr;       // [n * D] sorted order
+    float *d_G = nullptr;          // [n * D] sorted order (descriptor calls and the split path)
+    size_t cap_G = 0;
+    float *d_dEdG = nullptr;       // [n * D] sorted order (split path)
+    size_t cap_dEdG = 0;
     float *d_eatom = nullptr;      // [n] sorted order
     float4 *d_F4 = nullptr;        // [n] force accumulators, sorted order
     double *d_vir_part = nullptr;  // [cells * 9]
     double *d_e_part = nullptr;    // [blocks]
     double *d_ke_part = nullptr;   // [MD CTAs * 11] per-CTA energy, virial and kinetic-energy sums
     double *d_result = nullptr;    // [10]: energy, virial[9]
+    double *h_res = nullptr;       // mapped host memory [12]: energy, virial[9], -, error word
+    // mapped host memory for the arrays of small calls made with host pointers: the
+    // kernels read positions and species from it and write forces and E_i to it
+    unsigned char *h_stage = nullptr;
+    size_t cap_hstage = 0;
+    bool err_stale = false;        // the error word may hold an asynchronous call's error
     unsigned *d_err = nullptr;     // device error word
     unsigned long long *d_stats = nullptr;  // [4] radial entries, angular entries, angular pairs
     int *d_step = nullptr;         // MD record counter
@@ -221,6 +229,7 @@ struct Context {
     int *d_sp_off = nullptr;       // [kMaxSpecies]
     int *d_sp_rank = nullptr;      // [n]
     int *d_sp_list = nullptr;      // [n] sorted indices grouped by species
+    int cap_sp = 0;
 
     // staging of host arrays
     int cap_stage = 0;
@@ -396,8 +405,10 @@ cudaError_t launch_batch_reduce(Context &c, bool atoms, double *energies = nullp
 cudaError_t launch_ann(Context &c, int n);
 
 // Energy and virial reductions (E = sum_i E_i, Sec. II.A) over n_eparts energy partials and the
-// cells' virial partials, and outputs in input order.
-cudaError_t launch_finalize(Context &c, const Grid &g, int n, int n_eparts, double *forces, double *e_atom);
+// virial partials of the last evaluation, and outputs in input order (each or NULL); to_host:
+// energy, virial and the error word also to c.h_res.
+cudaError_t launch_finalize(Context &c, int n, int n_eparts, double *forces, double *e_atom, double *energy,
+                            double *virial, bool to_host);
 
 // BF16 tensor-core networks (precision forms; two hidden layers <= 32).
 bool bf16_supported(const Net &net);
@@ -453,7 +464,7 @@ int ann_blocks(int n);
 // Forces to input order (FP64) only.
 cudaError_t launch_finalize_forces(Context &c, int n, double *forces);
 
-// Descriptor rows to input order (float).
+// Descriptor rows to input order (float), and the error word to c.h_res[11].
 cudaError_t launch_unsort_G(Context &c, int n, float *G);
 
 // Velocity Verlet (the propagation step of the MD cycle, Fig. 1).

@@ -137,19 +137,14 @@ int ensure(Context &c, int n, const Grid &g) {
     if (n > c.cap_atoms || !c.d_pos4) {
         n = std::max(n, 1);
         size_t N = (size_t)n;
-        const int D = c.basis.D;
         CK(grow(c.d_pos4, 0, N), "cudaMalloc");
         CK(grow(c.d_tmp4, 0, N), "cudaMalloc");
         CK(grow(c.d_perm, 0, N), "cudaMalloc");
         CK(grow(c.d_cell_of, 0, N), "cudaMalloc");
         CK(grow(c.d_slot, 0, N), "cudaMalloc");
-        CK(grow(c.d_G, 0, N * D), "cudaMalloc");
-        CK(grow(c.d_dEdG, 0, N * D), "cudaMalloc");
         CK(grow(c.d_eatom, 0, N), "cudaMalloc");
         CK(grow(c.d_F4, 0, N), "cudaMalloc");
         CK(grow(c.d_ke_part, 0, 11 * ((N + 255) / 256 + 1)), "cudaMalloc");  // an 11-entry row per MD CTA
-        CK(grow(c.d_sp_rank, 0, N), "cudaMalloc");
-        CK(grow(c.d_sp_list, 0, N), "cudaMalloc");
         c.cap_atoms = n;
         ++c.buf_gen;
     }
@@ -173,6 +168,33 @@ int ensure(Context &c, int n, const Grid &g) {
     if (need_e > c.cap_blocks || !c.d_e_part) {
         CK(grow(c.d_e_part, 0, (size_t)need_e), "cudaMalloc");
         c.cap_blocks = need_e;
+        ++c.buf_gen;
+    }
+    return AENET_OK;
+}
+
+// G rows (the descriptor call and the split path); dE/dG rows too with grad.
+int ensure_G(Context &c, int n, bool grad) {
+    const size_t need = (size_t)std::max(n, 1) * c.basis.D;
+    if (need > c.cap_G || !c.d_G) {
+        CK(grow(c.d_G, 0, need), "cudaMalloc");
+        c.cap_G = need;
+        ++c.buf_gen;
+    }
+    if (grad && (need > c.cap_dEdG || !c.d_dEdG)) {
+        CK(grow(c.d_dEdG, 0, need), "cudaMalloc");
+        c.cap_dEdG = need;
+        ++c.buf_gen;
+    }
+    return AENET_OK;
+}
+
+// Species grouping (the BF16 network kernel and the weight gradient).
+int ensure_species(Context &c, int n) {
+    if (n > c.cap_sp || !c.d_sp_rank) {
+        CK(grow(c.d_sp_rank, 0, (size_t)std::max(n, 1)), "cudaMalloc");
+        CK(grow(c.d_sp_list, 0, (size_t)std::max(n, 1)), "cudaMalloc");
+        c.cap_sp = std::max(n, 1);
         ++c.buf_gen;
     }
     return AENET_OK;
@@ -226,6 +248,16 @@ int ensure_rows(Context &c, int n) {
         ++c.buf_gen;
     }
     return ensure_parts(c, (std::max(n, 1) + slice - 1) / slice);
+}
+
+// Every buffer that the evaluation of n atoms on the context's path allocates on
+// its own (before a capture, in which nothing can be allocated).
+int ensure_eval(Context &c, int n) {
+    int rc = AENET_OK;
+    if (rows_form(c) || !fused_path(c)) rc = ensure_rows(c, n);
+    if (!rc && !fused_path(c)) rc = ensure_G(c, n, true);
+    if (!rc && !fused_path(c) && c.precision != AENET_FP32) rc = ensure_species(c, n);
+    return rc;
 }
 
 int check_smem(Context &c, const Grid &g) {
@@ -291,7 +323,9 @@ int enqueue_potential(Context &c, const Grid &g, int n, int *n_eparts) {
         c.last_vpart = c.d_vir_part;
         c.last_vparts = c.pot_parts;
     } else {
-        int rc = enqueue_rows(c, g, n, RowsMode::descriptor);
+        int rc = ensure_G(c, n, true);
+        if (!rc && c.precision != AENET_FP32) rc = ensure_species(c, n);
+        if (!rc) rc = enqueue_rows(c, g, n, RowsMode::descriptor);
         if (rc) return rc;
         CK(mark(c, 3), "event");
         if (c.precision == AENET_FP32) {
@@ -313,23 +347,22 @@ int enqueue_potential(Context &c, const Grid &g, int n, int *n_eparts) {
 }
 
 // The whole path on device buffers, enqueued on c.stream (no synchronisation).
-// *n_eparts (optional) receives the number of energy partials.
+// forces, e_atom, energy, virial: where the results go (each or NULL); to_host: energy, virial
+// and the error word also to c.h_res.
 int enqueue_compute(Context &c, const Grid &g, int n, const double *pos, const int32_t *types, double *forces,
-                    double *e_atom, int *n_eparts_out = nullptr) {
+                    double *e_atom, double *energy = nullptr, double *virial = nullptr, bool to_host = false) {
     int rc = check_smem(c, g);
     if (rc) return rc;
     CK(launch_cells(c, g, n, pos, types), "cell list");
     int n_eparts = 0;
     if ((rc = enqueue_potential(c, g, n, &n_eparts))) return rc;
-    CK(launch_finalize(c, g, n, n_eparts, forces, e_atom), "reductions");
-    if (n_eparts_out) *n_eparts_out = n_eparts;
+    CK(launch_finalize(c, n, n_eparts, forces, e_atom, energy, virial, to_host), "reductions");
     return AENET_OK;
 }
 
-int read_error_word(Context &c) {
-    unsigned w = 0;
-    CK(cudaMemcpyAsync(&w, c.d_err, sizeof(unsigned), cudaMemcpyDeviceToHost, c.stream), "cudaMemcpyAsync");
-    CK(cudaStreamSynchronize(c.stream), "cudaStreamSynchronize");
+// The error word w that a call has read, as a status; a set word is cleared.
+int report_error_word(Context &c, unsigned w) {
+    c.err_stale = false;
     if (w) CK(cudaMemsetAsync(c.d_err, 0, sizeof(unsigned), c.stream), "cudaMemsetAsync");
     if (w & kErrType) return fail(&c, AENET_E_ARG, "species index out of range");
     if (w & kErrNonfinite) return fail(&c, AENET_E_NONFINITE, "non-finite coordinate");
@@ -337,6 +370,38 @@ int read_error_word(Context &c) {
     if (w & (kErrNbCap | kErrAngCap))
         return fail(&c, AENET_E_CAPACITY, "neighbour list overflow (capacity %d / %d)", c.caps.nb, c.caps.ang);
     if (w & kErrTimeout) return fail(&c, AENET_E_TIMEOUT, "a bounded wait inside the potential kernel gave up");
+    return AENET_OK;
+}
+
+int read_error_word(Context &c) {
+    unsigned *w = reinterpret_cast<unsigned *>(c.h_res + 11);
+    CK(cudaMemcpyAsync(w, c.d_err, sizeof(unsigned), cudaMemcpyDeviceToHost, c.stream), "cudaMemcpyAsync");
+    CK(cudaStreamSynchronize(c.stream), "cudaStreamSynchronize");
+    return report_error_word(c, *w);
+}
+
+// A synchronous call reports its own errors only: one that an asynchronous call
+// before it may have left is cleared.
+int clear_stale_error(Context &c) {
+    if (!c.err_stale) return AENET_OK;
+    CK(cudaMemsetAsync(c.d_err, 0, sizeof(unsigned), c.stream), "cudaMemsetAsync");
+    c.err_stale = false;
+    return AENET_OK;
+}
+
+// Calls with host arrays of at most this many atoms go through mapped host memory:
+// the binning reads positions and species from it, the closing kernel writes
+// forces and E_i to it, and the call needs no copy command at all.
+constexpr int kMappedAtoms = 4096;
+
+int ensure_mapped(Context &c, int n) {
+    const size_t need = (size_t)n * (7 * sizeof(double) + sizeof(int32_t));
+    if (need <= c.cap_hstage && c.h_stage) return AENET_OK;
+    if (c.h_stage) cudaFreeHost(c.h_stage);
+    c.h_stage = nullptr;
+    c.cap_hstage = 0;
+    CK(cudaHostAlloc(&c.h_stage, need, cudaHostAllocMapped | cudaHostAllocPortable), "cudaHostAlloc");
+    c.cap_hstage = need;
     return AENET_OK;
 }
 
@@ -465,6 +530,8 @@ extern "C" int aenet_setup(aenet_ctx **out, const aenet_model_desc *m, int preci
     if ((e = cudaMalloc(&c.d_sp_off, sizeof(int) * kMaxSpecies)) != cudaSuccess) return setup_fail(e, "cudaMalloc");
     if ((e = cudaMalloc(&c.d_result, sizeof(double) * 11)) != cudaSuccess) return setup_fail(e, "cudaMalloc");
     if ((e = cudaMalloc(&c.d_mass, sizeof(double) * kMaxSpecies)) != cudaSuccess) return setup_fail(e, "cudaMalloc");
+    if ((e = cudaHostAlloc(&c.h_res, 12 * sizeof(double), cudaHostAllocMapped | cudaHostAllocPortable)) != cudaSuccess)
+        return setup_fail(e, "cudaHostAlloc");
     if ((e = cudaMalloc(&c.d_work, 2 * sizeof(unsigned))) != cudaSuccess) return setup_fail(e, "cudaMalloc");
     if ((e = cudaMemset(c.d_work, 0, 2 * sizeof(unsigned))) != cudaSuccess) return setup_fail(e, "cudaMemset");
     if ((e = cudaDeviceGetAttribute(&c.n_sm, cudaDevAttrMultiProcessorCount, c.device)) != cudaSuccess)
@@ -522,25 +589,55 @@ static int compute_impl(Context &c, int n, const double *pos, const int32_t *typ
     int rc = make_grid(c, box, g, 0.0, c.tilt);
     if (rc) return rc;
     if ((rc = validate_types_host(c, n, types))) return rc;
-    if ((rc = ensure(c, n, g)) || (rc = ensure_stage(c, n))) return rc;
+    if ((rc = ensure(c, n, g)) || (n > kMappedAtoms && (rc = ensure_stage(c, n)))) return rc;
     if (c.caps.nb == 0) c.caps = estimate_caps(c, n, g);
-    const double *dpos;
-    const int32_t *dtypes;
-    if ((rc = stage_in(c, pos, c.d_pos, 3 * (size_t)n, &dpos))) return rc;
-    if ((rc = stage_in(c, types, c.d_types, (size_t)n, &dtypes))) return rc;
-    const bool f_dev = is_device_ptr(forces), ea_dev = is_device_ptr(e_atom), G_dev = is_device_ptr(G_out);
-    double *dF = forces ? (f_dev ? forces : c.d_forces) : nullptr;
-    double *dE = e_atom ? (ea_dev ? e_atom : c.d_eatom_out) : nullptr;
+    // a small call's host arrays through mapped memory, a large one's through device buffers
+    const bool pos_dev = is_device_ptr(pos), typ_dev = is_device_ptr(types);
+    const bool e_dev = is_device_ptr(energy), v_dev = is_device_ptr(virial);
+    const bool f_dev = is_device_ptr(forces), ea_dev = is_device_ptr(e_atom);
+    const bool mapped = n <= kMappedAtoms;
+    const size_t N = (size_t)n;
+    double *m_pos = nullptr, *m_f = nullptr, *m_e = nullptr;
+    int32_t *m_typ = nullptr;
+    if (mapped && n > 0 && !(pos_dev && typ_dev && (!forces || f_dev) && (!e_atom || ea_dev))) {
+        if ((rc = ensure_mapped(c, n))) return rc;
+        m_pos = reinterpret_cast<double *>(c.h_stage);
+        m_f = m_pos + 3 * N;
+        m_e = m_f + 3 * N;
+        m_typ = reinterpret_cast<int32_t *>(m_e + N);
+    }
+    const double *dpos = pos;
+    const int32_t *dtypes = types;
+    if (m_pos && !pos_dev) {
+        memcpy(m_pos, pos, 3 * sizeof(double) * N);
+        dpos = m_pos;
+    } else if ((rc = stage_in(c, pos, c.d_pos, 3 * N, &dpos))) {
+        return rc;
+    }
+    if (m_pos && !typ_dev) {
+        memcpy(m_typ, types, sizeof(int32_t) * N);
+        dtypes = m_typ;
+    } else if ((rc = stage_in(c, types, c.d_types, N, &dtypes))) {
+        return rc;
+    }
+    double *dF = !forces ? nullptr : f_dev ? forces : m_f ? m_f : c.d_forces;
+    double *dE = !e_atom ? nullptr : ea_dev ? e_atom : m_e ? m_e : c.d_eatom_out;
+    if ((rc = clear_stale_error(c))) return rc;
+    const bool G_dev = is_device_ptr(G_out);
     for (int attempt = 0; attempt < 2; ++attempt) {
-        CK(cudaMemsetAsync(c.d_err, 0, sizeof(unsigned), c.stream), "cudaMemsetAsync");
         if (G_out) {
             if ((rc = check_smem(c, g))) return rc;
+            if ((rc = ensure_G(c, n, !G_dev))) return rc;
             CK(launch_cells(c, g, n, dpos, dtypes), "cell list");
             if ((rc = enqueue_rows(c, g, n, RowsMode::descriptor))) return rc;
+            CK(launch_unsort_G(c, n, G_dev ? G_out : c.d_dEdG), "unsort");  // (host rows: the other row buffer first)
         } else {
-            if ((rc = enqueue_compute(c, g, n, dpos, dtypes, dF, dE))) return rc;
+            if ((rc = enqueue_compute(c, g, n, dpos, dtypes, dF, dE, e_dev ? energy : nullptr,
+                                      v_dev ? virial : nullptr, true)))
+                return rc;
         }
-        rc = read_error_word(c);
+        CK(cudaStreamSynchronize(c.stream), "cudaStreamSynchronize");
+        rc = report_error_word(c, (unsigned)c.h_res[11]);
         if (rc != AENET_E_CAPACITY || attempt == 1) break;
         c.caps.nb *= 2;  // regrow once and retry
         c.caps.ang *= 2;
@@ -549,35 +646,30 @@ static int compute_impl(Context &c, int n, const double *pos, const int32_t *typ
     }
     if (rc) return rc;
     if (G_out) {
-        if (G_dev) {
-            CK(launch_unsort_G(c, n, G_out), "unsort");
-        } else {
-            float *tmp = nullptr;
-            CK(cudaMalloc(&tmp, sizeof(float) * (size_t)n * c.basis.D + 4), "cudaMalloc");
-            cudaError_t e1 = launch_unsort_G(c, n, tmp);
-            cudaError_t e2 = e1 == cudaSuccess ? cudaMemcpyAsync(G_out, tmp, sizeof(float) * (size_t)n * c.basis.D,
-                                                                 cudaMemcpyDeviceToHost, c.stream)
-                                               : e1;
-            cudaError_t e3 = cudaStreamSynchronize(c.stream);
-            cudaFree(tmp);
-            if (e2 != cudaSuccess) return cuda_fail(&c, e2, "descriptor copy");
-            if (e3 != cudaSuccess) return cuda_fail(&c, e3, "cudaStreamSynchronize");
-        }
-        CK(cudaStreamSynchronize(c.stream), "cudaStreamSynchronize");
+        if (!G_dev && n > 0)
+            CK(cudaMemcpy(G_out, c.d_dEdG, sizeof(float) * N * c.basis.D, cudaMemcpyDeviceToHost), "descriptor copy");
         return AENET_OK;
     }
     c.act_valid = c.keep_act;
     c.act_atoms = n;
-    if (energy) CK(cudaMemcpyAsync(energy, c.d_result, sizeof(double), cudaMemcpyDefault, c.stream), "energy copy");
-    if (virial)
-        CK(cudaMemcpyAsync(virial, c.d_result + 1, 9 * sizeof(double), cudaMemcpyDefault, c.stream), "virial copy");
-    if (forces && !f_dev)
-        CK(cudaMemcpyAsync(forces, c.d_forces, 3 * sizeof(double) * (size_t)n, cudaMemcpyDeviceToHost, c.stream),
-           "forces copy");
-    if (e_atom && !ea_dev)
-        CK(cudaMemcpyAsync(e_atom, c.d_eatom_out, sizeof(double) * (size_t)n, cudaMemcpyDeviceToHost, c.stream),
-           "e_atom copy");
-    CK(cudaStreamSynchronize(c.stream), "cudaStreamSynchronize");
+    if (energy && !e_dev) *energy = c.h_res[0];
+    if (virial && !v_dev) memcpy(virial, c.h_res + 1, 9 * sizeof(double));
+    if (forces && !f_dev) {
+        if (m_f)
+            memcpy(forces, m_f, 3 * sizeof(double) * N);
+        else
+            CK(cudaMemcpyAsync(forces, c.d_forces, 3 * sizeof(double) * N, cudaMemcpyDeviceToHost, c.stream),
+               "forces copy");
+    }
+    if (e_atom && !ea_dev) {
+        if (m_e)
+            memcpy(e_atom, m_e, sizeof(double) * N);
+        else
+            CK(cudaMemcpyAsync(e_atom, c.d_eatom_out, sizeof(double) * N, cudaMemcpyDeviceToHost, c.stream),
+               "e_atom copy");
+    }
+    if (!mapped && ((forces && !f_dev) || (e_atom && !ea_dev)))
+        CK(cudaStreamSynchronize(c.stream), "cudaStreamSynchronize");
     return AENET_OK;
 }
 
@@ -604,12 +696,10 @@ extern "C" int aenet_compute_async(aenet_ctx *h, int n, const double *pos, const
     if (rc) return rc;
     if ((rc = ensure(c, n, g))) return rc;
     if (c.caps.nb == 0) c.caps = estimate_caps(c, n, g);
-    if ((rc = enqueue_compute(c, g, n, pos, types, forces, e_atom))) return rc;
+    c.err_stale = true;
+    if ((rc = enqueue_compute(c, g, n, pos, types, forces, e_atom, energy, virial))) return rc;
     c.act_valid = c.keep_act;
     c.act_atoms = n;
-    if (energy) CK(cudaMemcpyAsync(energy, c.d_result, sizeof(double), cudaMemcpyDeviceToDevice, c.stream), "energy");
-    if (virial)
-        CK(cudaMemcpyAsync(virial, c.d_result + 1, 9 * sizeof(double), cudaMemcpyDeviceToDevice, c.stream), "virial");
     return AENET_OK;
 }
 
@@ -695,7 +785,7 @@ int batch_buffers(Context &c, const BatchLayout &L) {
         c.caps.ang = std::max(32, cap(c.basis.rc_ang, 24.0));
         c.caps.tile = std::min(1024, std::max(128, (((int)(1.25 * L.max_neigh + 64.0)) + 31) / 32 * 32));
     }
-    return AENET_OK;
+    return ensure_eval(c, L.n);
 }
 
 // The batched evaluation on device buffers, enqueued on c.stream: binning,
@@ -770,8 +860,8 @@ extern "C" int aenet_compute_batch(aenet_ctx *h, int n_struct, const int64_t *at
         bool v;
         ~Restore() { c.persist = v; }
     } restore{c, persist};
+    if ((rc = clear_stale_error(c))) return rc;
     for (int attempt = 0; attempt < 2; ++attempt) {
-        CK(cudaMemsetAsync(c.d_err, 0, sizeof(unsigned), c.stream), "cudaMemsetAsync");
         if ((rc = batch_enqueue(c, L, c.d_sinfo, c.d_order, dpos, dtypes, dF, nullptr, nullptr))) break;
         rc = read_error_word(c);
         if (rc != AENET_E_CAPACITY || attempt == 1) break;
@@ -930,7 +1020,7 @@ extern "C" int aenet_batch_prepare(aenet_ctx *h, int n_struct, const int64_t *at
             continue;
         }
         for (int attempt = 0; attempt < 2; ++attempt) {  // warm-up run; regrow the lists once on overflow
-            CK(cudaMemsetAsync(c.d_err, 0, sizeof(unsigned), c.stream), "cudaMemsetAsync");
+            if ((rc = clear_stale_error(c))) break;
             if ((rc = batch_enqueue(c, L, c.d_psinfo, c.d_porder, pos, types, forces, energies, virials))) break;
             rc = read_error_word(c);
             if (rc != AENET_E_CAPACITY || attempt == 1) break;
@@ -994,6 +1084,7 @@ extern "C" int aenet_batch_run(aenet_ctx *h) {
         c.caps.tile = tile;
         if (rc) return rc;
     }
+    c.err_stale = true;
     CK(cudaGraphLaunch(c.batch_exec, c.stream), "graph launch");
     c.maps_n = c.plan.n_atoms;  // the replay rewrote the cell maps
     c.vl_valid = false;
@@ -1196,7 +1287,7 @@ static int md_fixed_cell(aenet_ctx *h, int n, double *pos, double *vel, const in
         if ((rc = ensure_verlet(c, n, g))) return rc;
     }
     const bool rows = fused_supported(c) && !c.pipeline && c.md_list != AENET_MD_LIST_OFF;
-    if (rows && !verlet && (rc = ensure_rows(c, n))) return rc;
+    if ((rc = ensure_eval(c, n))) return rc;
     double *dpos = pos_dev ? pos : c.d_pos;
     double *dvel = vel_dev ? vel : c.d_vel;
     const int32_t *dtypes = typ_dev ? types : c.d_types;
@@ -1215,7 +1306,10 @@ static int md_fixed_cell(aenet_ctx *h, int n, double *pos, double *vel, const in
         destroy_graph(c);
     }
     double *rec = want_rec ? c.d_rec : nullptr;
-    if (!async) CK(cudaMemsetAsync(c.d_err, 0, sizeof(unsigned), c.stream), "cudaMemsetAsync");
+    if (async)
+        c.err_stale = true;
+    else if ((rc = clear_stale_error(c)))
+        return rc;
     if (want_rec) CK(cudaMemsetAsync(c.d_step, 0, sizeof(int), c.stream), "cudaMemsetAsync");
     // frame 0: forces at the initial positions (unless continuing); a
     // neighbour-list overflow here regrows the capacities once before capture
@@ -1495,6 +1589,7 @@ extern "C" int aenet_grad_weights(aenet_ctx *h, double *dEdW) {
         return fail(&c, AENET_E_STATE, "no activation records: set AENET_OPT_KEEP_ACTIVATIONS and evaluate first");
     if (c.net.n_params > grad_max_params())
         return fail(&c, AENET_E_ARG, "network has more than %d parameters per species", grad_max_params());
+    if (const int rc = ensure_species(c, c.act_atoms)) return rc;
     CK(launch_grad_weights(c, c.act_atoms), "weight gradient");
     CK(cudaMemcpyAsync(dEdW, c.d_dEdW, sizeof(double) * c.basis.n_species * c.net.n_params, cudaMemcpyDefault,
                        c.stream),
@@ -1561,6 +1656,8 @@ extern "C" void aenet_destroy(aenet_ctx *h) {
                     c.d_vl_epart, c.d_vl_vpart, c.d_lambda, c.d_rows, c.d_list_count, c.d_pnet, c.d_vir_atom};
     for (void *p : ptrs)
         if (p) cudaFree(p);
+    if (c.h_res) cudaFreeHost(c.h_res);
+    if (c.h_stage) cudaFreeHost(c.h_stage);
     for (int k = 0; k <= Context::kStages; ++k)
         if (c.ev[k]) cudaEventDestroy(c.ev[k]);
     if (c.own_stream && c.stream) cudaStreamDestroy(c.stream);

@@ -99,26 +99,23 @@ cudaError_t launch_sort(Context &c, const Grid &g, int n) {
 }
 
 cudaError_t launch_cells(Context &c, const Grid &g, int n, const double *pos, const int32_t *types) {
-    cudaError_t e = cudaMemsetAsync(c.d_cell_count, 0, sizeof(int) * g.ncell, c.stream);
-    if (e != cudaSuccess) return e;
+    // (the cell counts are zero: a new array is cleared, and every scan clears what it reads)
     if (n > 0) {
         k_bin_count<<<(n + 255) / 256, 256, 0, c.stream>>>(n, c.basis.n_species, pos, types, g, c.d_tmp4,
                                                            c.d_cell_of, c.d_slot, c.d_cell_count, c.d_err);
     }
-    e = cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return launch_sort(c, g, n);
 }
 
 cudaError_t launch_cells_batch(Context &c, int n, int total_cells, const double *pos, const int32_t *types) {
-    cudaError_t e = cudaMemsetAsync(c.d_cell_count, 0, sizeof(int) * total_cells, c.stream);
-    if (e != cudaSuccess) return e;
     if (n > 0) {
         k_bin_count_batch<<<(n + 255) / 256, 256, 0, c.stream>>>(n, c.batch_n, c.basis.n_species, pos, types,
                                                                  c.batch_sinfo, c.d_tmp4, c.d_cell_of, c.d_slot,
                                                                  c.d_cell_count, c.d_err);
     }
-    e = cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     Grid g{};
     g.ncell = total_cells;

@@ -9,6 +9,8 @@
 // MD step runs in two kernels around the potential: kick + drift + binning, and
 // closing kick + all reductions (the last CTA to finish sums every partial in a
 // fixed order, so results are deterministic).
+#include <algorithm>
+
 #include "aenet_internal.cuh"
 #include "cell_scan.cuh"
 
@@ -18,6 +20,7 @@ namespace {
 
 constexpr double kEvPerAmu = 9648.533212;  // (A/ps)^2 per eV/amu
 constexpr int kRedThreads = 256;
+constexpr int kReduceCtas = 2;  // k_finalize: CTAs of the reductions (10 warps)
 constexpr int kMdThreads = 256;
 
 // Per-species kick factor dt/2 * c / m and kinetic factor m / (2 c).
@@ -63,35 +66,65 @@ __device__ inline double warp_reduce_strided(const double *x, int n, int stride,
     return warp_sum_d((a0 + a1) + (a2 + a3));
 }
 
-// result[q] for q = 0 (energy, n_e partials) and 1..9 (virial, n_v x 9 partials):
-// one warp per quantity.
-__global__ void k_reduce(int n_e, const double *__restrict__ e_part, int n_v, const double *__restrict__ vir_part,
-                         double *__restrict__ result) {
-    const int lane = threadIdx.x & 31;
-    const int q = blockIdx.x * (kRedThreads / 32) + (threadIdx.x >> 5);
-    if (q > 9) return;
-    const double v = q == 0 ? warp_reduce_strided(e_part, n_e, 1, lane)
-                            : warp_reduce_strided(vir_part + (q - 1), n_v, 9, lane);
-    if (lane == 0) result[q] = v;
+// Where an evaluation's results go: forces [n * 3] and E_i [n] in input order,
+// energy and virial[9], each or none; host_res (mapped host memory, 12 values):
+// energy, virial, and at 11 the error word, so that a synchronising call needs
+// no copy.
+struct FinalizeOut {
+    double *forces, *e_atom, *energy, *virial, *host_res;
+};
+
+// The closing kernel of an evaluation. CTAs 0 and 1: result[q] for q = 0 (energy,
+// n_e partials) and 1..9 (virial, n_v x 9 partials), one warp per quantity; the
+// others: forces and atomic energies in input order.
+__global__ void __launch_bounds__(kRedThreads)
+    k_finalize(int n, const int *__restrict__ perm, const float4 *__restrict__ F4, const float *__restrict__ eatom,
+               int n_e, const double *__restrict__ e_part, int n_v, const double *__restrict__ vir_part,
+               double *__restrict__ result, const unsigned *__restrict__ err, FinalizeOut o) {
+    if (blockIdx.x < kReduceCtas) {
+        const int lane = threadIdx.x & 31;
+        const int q = blockIdx.x * (kRedThreads / 32) + (threadIdx.x >> 5);
+        if (q > 9) {
+            if (q == 10 && lane == 0 && o.host_res) o.host_res[11] = (double)*err;
+            return;
+        }
+        const double v = q == 0 ? warp_reduce_strided(e_part, n_e, 1, lane)
+                                : warp_reduce_strided(vir_part + (q - 1), n_v, 9, lane);
+        if (lane == 0) {
+            result[q] = v;
+            if (o.host_res) o.host_res[q] = v;
+            if (q == 0 && o.energy) *o.energy = v;
+            if (q > 0 && o.virial) o.virial[q - 1] = v;
+        }
+        return;
+    }
+    const int s = (blockIdx.x - kReduceCtas) * blockDim.x + threadIdx.x;
+    if (s >= n) return;
+    const int i = perm[s];
+    if (o.forces) {
+        const float4 f = F4[s];
+        o.forces[3 * i + 0] = (double)f.x;
+        o.forces[3 * i + 1] = (double)f.y;
+        o.forces[3 * i + 2] = (double)f.z;
+    }
+    if (o.e_atom) o.e_atom[i] = (double)eatom[s];
 }
 
-__global__ void k_unsort_outputs(int n, const int *__restrict__ perm, const float4 *__restrict__ F4,
-                                 const float *__restrict__ eatom, double *__restrict__ forces,
-                                 double *__restrict__ e_atom_out) {
+__global__ void k_unsort_forces(int n, const int *__restrict__ perm, const float4 *__restrict__ F4,
+                                double *__restrict__ forces) {
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const int i = perm[s];
-    if (forces) {
-        const float4 f = F4[s];
-        forces[3 * i + 0] = (double)f.x;
-        forces[3 * i + 1] = (double)f.y;
-        forces[3 * i + 2] = (double)f.z;
-    }
-    if (e_atom_out) e_atom_out[i] = (double)eatom[s];
+    const float4 f = F4[s];
+    forces[3 * i + 0] = (double)f.x;
+    forces[3 * i + 1] = (double)f.y;
+    forces[3 * i + 2] = (double)f.z;
 }
 
+// (host_err: the error word into mapped host memory)
 __global__ void k_unsort_G(int n, int D, const int *__restrict__ perm, const float *__restrict__ Gs,
-                           float *__restrict__ G) {
+                           float *__restrict__ G, const unsigned *__restrict__ err, double *__restrict__ host_err) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *host_err = (double)*err;
     const size_t total = (size_t)n * D;
     for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < total; k += (size_t)gridDim.x * blockDim.x) {
         const int s = (int)(k / D), c = (int)(k % D);
@@ -449,23 +482,25 @@ __global__ void k_scale(double *__restrict__ x, long long count, double mu) {
 
 }  // namespace
 
-cudaError_t launch_finalize(Context &c, const Grid &g, int n, int n_eparts, double *forces, double *e_atom) {
-    k_reduce<<<(10 + kRedThreads / 32 - 1) / (kRedThreads / 32), kRedThreads, 0, c.stream>>>(
-        n_eparts, c.last_epart, c.last_vparts, c.last_vpart, c.d_result);
-    if ((forces || e_atom) && n > 0)
-        k_unsort_outputs<<<(n + 255) / 256, 256, 0, c.stream>>>(n, c.d_perm, c.d_F4, c.d_eatom, forces, e_atom);
+cudaError_t launch_finalize(Context &c, int n, int n_eparts, double *forces, double *e_atom, double *energy,
+                            double *virial, bool to_host) {
+    const int blocks = kReduceCtas + ((forces || e_atom) && n > 0 ? (n + kRedThreads - 1) / kRedThreads : 0);
+    k_finalize<<<blocks, kRedThreads, 0, c.stream>>>(
+        n, c.d_perm, c.d_F4, c.d_eatom, n_eparts, c.last_epart, c.last_vparts, c.last_vpart, c.d_result, c.d_err,
+        FinalizeOut{forces, e_atom, energy, virial, to_host ? c.h_res : nullptr});
     return cudaGetLastError();
 }
 
 cudaError_t launch_finalize_forces(Context &c, int n, double *forces) {
     if (!forces || n <= 0) return cudaSuccess;
-    k_unsort_outputs<<<(n + 255) / 256, 256, 0, c.stream>>>(n, c.d_perm, c.d_F4, c.d_eatom, forces, nullptr);
+    k_unsort_forces<<<(n + 255) / 256, 256, 0, c.stream>>>(n, c.d_perm, c.d_F4, forces);
     return cudaGetLastError();
 }
 
 cudaError_t launch_unsort_G(Context &c, int n, float *G) {
-    if (n <= 0) return cudaSuccess;
-    k_unsort_G<<<1024, 256, 0, c.stream>>>(n, c.basis.D, c.d_perm, c.d_G, G);
+    const long long blocks = ((long long)n * c.basis.D + 255) / 256;
+    k_unsort_G<<<(int)std::max(1LL, std::min(1024LL, blocks)), 256, 0, c.stream>>>(n, c.basis.D, c.d_perm, c.d_G, G,
+                                                                                  c.d_err, c.h_res + 11);
     return cudaGetLastError();
 }
 
@@ -530,8 +565,7 @@ cudaError_t launch_md_vl_kick_drift(Context &c, int n, double dt, double *pos, d
 }
 
 cudaError_t launch_md_vl_bin(Context &c, const Grid &g, int n, const double *pos, const int32_t *types) {
-    cudaError_t e = cudaMemsetAsync(c.d_cell_count, 0, sizeof(int) * g.ncell, c.stream);
-    if (e != cudaSuccess || n <= 0) return e;
+    if (n <= 0) return cudaSuccess;  // (the cell counts are zero: every scan clears them)
     k_md_vl_bin<<<(n + kMdThreads - 1) / kMdThreads, kMdThreads, 0, c.stream>>>(
         n, c.basis.n_species, pos, types, g, c.d_tmp4, c.d_cell_of, c.d_slot, c.d_cell_count, c.d_vl_origin,
         c.d_vl_ref, c.d_err);
