@@ -342,9 +342,10 @@ struct Context {
     std::vector<StructInfo> plan_layout;  // host copy of the prepared layout
     std::vector<int> plan_order;
 
-    // captured MD step
-    cudaGraphExec_t md_exec = nullptr;
-    struct {
+    // captured MD step (kick + drift + binning ... closing kick), and the part of a
+    // call between two drifts (sort, potential, k_md_turn), each with what it was
+    // captured for
+    struct MdKey {
         int n = -1;
         double *pos = nullptr, *vel = nullptr;
         const int32_t *types = nullptr;
@@ -352,14 +353,22 @@ struct Context {
         double dt = 0;
         double *rec = nullptr;
         cudaStream_t stream = nullptr;
-        Caps caps{};
-        bool timing = false;
+        int nb = 0, ang = 0, tile = 0, vl_cap = 0;
         unsigned gen = 0;
         double skin = 0.0;
         bool list_form = false;
         unsigned ev_mask = 0;
         double thermo_T0 = 0.0, thermo_tau = 0.0;
-    } md_key;
+        bool operator==(const MdKey &o) const {
+            return n == o.n && pos == o.pos && vel == o.vel && types == o.types && box[0] == o.box[0] &&
+                   box[1] == o.box[1] && box[2] == o.box[2] && dt == o.dt && rec == o.rec && stream == o.stream &&
+                   nb == o.nb && ang == o.ang && tile == o.tile && vl_cap == o.vl_cap && gen == o.gen &&
+                   skin == o.skin && list_form == o.list_form && ev_mask == o.ev_mask && thermo_T0 == o.thermo_T0 &&
+                   thermo_tau == o.thermo_tau;
+        }
+    };
+    cudaGraphExec_t md_exec = nullptr, turn_exec = nullptr;
+    MdKey md_key, turn_key;
     unsigned ev_mask = 0;              // stage events recorded while an MD step is captured
 
     // stage timing of the captured MD step (events recorded inside the graph)
@@ -479,6 +488,10 @@ cudaError_t launch_md_kick_drift_bin(Context &c, const Grid &g, int n, double dt
 // clear_vl, the last CTA also counts a list build and clears the rebuild flag.
 cudaError_t launch_md_kick_finish(Context &c, int n, double dt, double *vel, const int32_t *types,
                                   double *rec_pot, double *rec_kin, bool clear_vl = false);
+// The closing kick and reduction of one step and the opening kick, drift and
+// binning (with the scan) of the next in one kernel (NVE).
+cudaError_t launch_md_turn(Context &c, const Grid &g, int n, double dt, double *pos, double *vel,
+                           const int32_t *types, double *rec_pot, double *rec_kin);
 // x *= mu for count doubles (the barostat's isotropic scaling of positions).
 cudaError_t launch_scale(Context &c, double *x, long long count, double mu);
 

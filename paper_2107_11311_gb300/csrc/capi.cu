@@ -431,8 +431,9 @@ int validate_types_host(Context &c, int n, const int32_t *types) {
 
 void destroy_graph(Context &c) {
     if (c.md_exec) cudaGraphExecDestroy(c.md_exec);
-    c.md_exec = nullptr;
-    c.md_key.n = -1;
+    if (c.turn_exec) cudaGraphExecDestroy(c.turn_exec);
+    c.md_exec = c.turn_exec = nullptr;
+    c.md_key.n = c.turn_key.n = -1;
 }
 
 }  // namespace
@@ -1125,24 +1126,24 @@ static bool md_list_form(const Context &c) {
 // cell search), closing kick with the FP64 reductions (and the record of (E_pot,
 // E_kin) when rec != NULL). With timing, events bracket the 6 stages; the list
 // build is part of the cell sort's.
-static int enqueue_md_step(Context &c, const Grid &g, int n, double dt, double *pos, double *vel,
-                           const int32_t *types, double *rec, bool rows) {
-    c.cell_search = !rows;
-    int rc = check_smem(c, g);
-    c.cell_search = false;
-    if (rc) return rc;
-    CK(mark(c, 0), "event");
-    CK(launch_md_kick_drift_bin(c, g, n, dt, pos, vel, types), "kick + drift + binning + scan");
-    CK(mark(c, 1), "event");
+static int enqueue_md_forces(Context &c, const Grid &g, int n, bool rows) {
     CK(launch_scatter(c, n), "cell sort");
     c.cell_search = !rows;
     if (!rows_form(c)) CK(mark(c, 2), "event");
     int n_eparts = 0;
-    c.md_prezeroed = true;  // the kick + drift kernel cleared the forces and statistics
-    rc = enqueue_potential(c, g, n, &n_eparts);
+    c.md_prezeroed = true;  // the kernel with the drift cleared the forces and statistics
+    const int rc = enqueue_potential(c, g, n, &n_eparts);
     c.md_prezeroed = false;
     c.cell_search = false;
-    if (rc) return rc;
+    return rc;
+}
+
+static int enqueue_md_step(Context &c, const Grid &g, int n, double dt, double *pos, double *vel,
+                           const int32_t *types, double *rec, bool rows) {
+    CK(mark(c, 0), "event");
+    CK(launch_md_kick_drift_bin(c, g, n, dt, pos, vel, types), "kick + drift + binning + scan");
+    CK(mark(c, 1), "event");
+    if (const int rc = enqueue_md_forces(c, g, n, rows)) return rc;
     CK(launch_md_kick_finish(c, n, dt, vel, types, rec, rec ? rec + c.cap_rec : nullptr), "kick + reductions");
     CK(mark(c, 6), "event");
     return AENET_OK;
@@ -1337,22 +1338,54 @@ static int md_fixed_cell(aenet_ctx *h, int n, double *pos, double *vel, const in
     if (want_rec || (thermo && (!cont || !c.lambda_valid)))  // kinetic energy and record of frame 0
         CK(launch_md_kick_finish(c, n, 0.0, dvel, dtypes, rec, rec ? rec + c.cap_rec : nullptr), "frame 0");
     if (n_steps > 0) {
-        const bool same = c.md_exec && c.md_key.n == n && c.md_key.pos == dpos && c.md_key.vel == dvel &&
-                          c.md_key.types == dtypes && c.md_key.box[0] == box[0] && c.md_key.box[1] == box[1] &&
-                          c.md_key.box[2] == box[2] && c.md_key.dt == dt && c.md_key.rec == rec &&
-                          c.md_key.stream == c.stream && c.md_key.caps.nb == c.caps.nb &&
-                          c.md_key.caps.ang == c.caps.ang && c.md_key.caps.tile == c.caps.tile &&
-                          c.md_key.ev_mask == ev_mask && c.md_key.gen == c.buf_gen && c.md_key.skin == c.skin &&
-                          c.md_key.list_form == list_form && c.md_key.caps.vl_cap == c.caps.vl_cap &&
-                          c.md_key.thermo_T0 == c.thermo_T0 &&
-                          c.md_key.thermo_tau == c.thermo_tau;
-        if (!same) {
-            destroy_graph(c);
+        c.cell_search = !rows;
+        rc = check_smem(c, g);
+        c.cell_search = false;
+        if (rc) return rc;
+        // Two or more steps without stage events: the first drift, then per step the
+        // captured sort, potential and k_md_turn (closing kick, reductions, next drift),
+        // and after the last potential a closing kick alone. Otherwise, and where the
+        // opening kick needs the reductions (thermostat, Verlet list), one captured
+        // step per step.
+        const bool turn = n_steps >= 2 && !verlet && !thermo && !timing;
+        Context::MdKey key;
+        key.n = n;
+        key.pos = dpos;
+        key.vel = dvel;
+        key.types = dtypes;
+        for (int a = 0; a < 3; ++a) key.box[a] = box[a];
+        key.dt = dt;
+        key.rec = rec;
+        key.stream = c.stream;
+        key.nb = c.caps.nb;
+        key.ang = c.caps.ang;
+        key.tile = c.caps.tile;
+        key.vl_cap = c.caps.vl_cap;
+        key.gen = c.buf_gen;
+        key.skin = c.skin;
+        key.list_form = list_form;
+        key.ev_mask = ev_mask;
+        key.thermo_T0 = c.thermo_T0;
+        key.thermo_tau = c.thermo_tau;
+        cudaGraphExec_t &exec = turn ? c.turn_exec : c.md_exec;
+        Context::MdKey &have = turn ? c.turn_key : c.md_key;
+        if (!exec || !(have == key)) {
+            if (exec) cudaGraphExecDestroy(exec);
+            exec = nullptr;
+            have.n = -1;
             cudaGraph_t graph = nullptr;
             CK(cudaStreamBeginCapture(c.stream, cudaStreamCaptureModeThreadLocal), "begin capture");
             c.ev_mask = ev_mask;
-            int src = verlet ? enqueue_md_step_verlet(c, g, n, dt, dpos, dvel, dtypes, rec)
+            int src;
+            if (turn) {
+                src = enqueue_md_forces(c, g, n, rows);
+                cudaError_t te = cudaSuccess;
+                if (!src) te = launch_md_turn(c, g, n, dt, dpos, dvel, dtypes, rec, rec ? rec + c.cap_rec : nullptr);
+                if (te != cudaSuccess) src = cuda_fail(&c, te, "kick + reductions + drift");
+            } else {
+                src = verlet ? enqueue_md_step_verlet(c, g, n, dt, dpos, dvel, dtypes, rec)
                              : enqueue_md_step(c, g, n, dt, dpos, dvel, dtypes, rec, rows);
+            }
             c.ev_mask = 0u;
             cudaError_t ce = cudaStreamEndCapture(c.stream, &graph);
             if (src) {
@@ -1360,48 +1393,43 @@ static int md_fixed_cell(aenet_ctx *h, int n, double *pos, double *vel, const in
                 return src;
             }
             if (ce != cudaSuccess) return cuda_fail(&c, ce, "end capture");
-            size_t n_nodes = 0;
-            c.md_kernels = 0;
-            if (cudaGraphGetNodes(graph, nullptr, &n_nodes) == cudaSuccess && n_nodes > 0) {
-                std::vector<cudaGraphNode_t> nodes(n_nodes);
-                if (cudaGraphGetNodes(graph, nodes.data(), &n_nodes) == cudaSuccess) {
-                    for (size_t k = 0; k < n_nodes; ++k) {
-                        cudaGraphNodeType t;
-                        if (cudaGraphNodeGetType(nodes[k], &t) == cudaSuccess && t == cudaGraphNodeTypeKernel)
-                            ++c.md_kernels;
+            if (!turn) {
+                size_t n_nodes = 0;
+                c.md_kernels = 0;
+                if (cudaGraphGetNodes(graph, nullptr, &n_nodes) == cudaSuccess && n_nodes > 0) {
+                    std::vector<cudaGraphNode_t> nodes(n_nodes);
+                    if (cudaGraphGetNodes(graph, nodes.data(), &n_nodes) == cudaSuccess) {
+                        for (size_t k = 0; k < n_nodes; ++k) {
+                            cudaGraphNodeType t;
+                            if (cudaGraphNodeGetType(nodes[k], &t) == cudaSuccess && t == cudaGraphNodeTypeKernel)
+                                ++c.md_kernels;
+                        }
                     }
                 }
+                c.last_list = list_form;
+                c.last_fused = fused_path(c);
+                c.last_rows = rows && !verlet;
             }
-            ce = cudaGraphInstantiate(&c.md_exec, graph, 0);
+            ce = cudaGraphInstantiate(&exec, graph, 0);
             cudaGraphDestroy(graph);
             if (ce != cudaSuccess) {
-                c.md_exec = nullptr;
+                exec = nullptr;
                 return cuda_fail(&c, ce, "graph instantiate");
             }
-            c.md_key.n = n;
-            c.md_key.pos = dpos;
-            c.md_key.vel = dvel;
-            c.md_key.types = dtypes;
-            for (int a = 0; a < 3; ++a) c.md_key.box[a] = box[a];
-            c.md_key.dt = dt;
-            c.md_key.rec = rec;
-            c.md_key.stream = c.stream;
-            c.md_key.caps = c.caps;
-            c.md_key.timing = timing;
-            c.md_key.ev_mask = ev_mask;
-            c.md_key.gen = c.buf_gen;
-            c.md_key.skin = c.skin;
-            c.md_key.list_form = list_form;
-            c.last_list = list_form;
-            c.last_fused = fused_path(c);
-            c.last_rows = rows && !verlet;
-            c.md_key.thermo_T0 = c.thermo_T0;
-            c.md_key.thermo_tau = c.thermo_tau;
+            have = key;
         }
         // the first step after any other evaluation (or a new list shape) builds the list
         if (verlet && (!cont || !c.vl_valid))
             CK(cudaMemsetAsync(c.d_vl_flag, 0xff, sizeof(unsigned), c.stream), "cudaMemsetAsync");
-        for (int s = 0; s < n_steps; ++s) CK(cudaGraphLaunch(c.md_exec, c.stream), "graph launch");
+        if (turn) {
+            CK(launch_md_kick_drift_bin(c, g, n, dt, dpos, dvel, dtypes), "kick + drift + binning + scan");
+            for (int s = 1; s < n_steps; ++s) CK(cudaGraphLaunch(exec, c.stream), "graph launch");
+            if ((rc = enqueue_md_forces(c, g, n, rows))) return rc;
+            CK(launch_md_kick_finish(c, n, dt, dvel, dtypes, rec, rec ? rec + c.cap_rec : nullptr),
+               "kick + reductions");
+        } else {
+            for (int s = 0; s < n_steps; ++s) CK(cudaGraphLaunch(exec, c.stream), "graph launch");
+        }
         c.maps_n = n;
         c.vl_valid = verlet;
         c.lambda_valid = thermo;
@@ -1531,7 +1559,7 @@ extern "C" int aenet_neighbor_stats(aenet_ctx *h, int64_t *out) {
 extern "C" int aenet_md_stage_times(aenet_ctx *h, float *ms, int *kernels_per_step, int *path_flags) {
     if (!h || !ms) return fail(h ? &h->c : nullptr, AENET_E_ARG, "NULL argument");
     Context &c = h->c;
-    if (!c.md_exec || !c.md_key.timing) return fail(&c, AENET_E_STATE, "no MD step was run with AENET_MD_TIMING");
+    if (!c.md_exec || !c.md_key.ev_mask) return fail(&c, AENET_E_STATE, "no MD step was run with AENET_MD_TIMING");
     CK(cudaStreamSynchronize(c.stream), "cudaStreamSynchronize");
     for (int k = 0; k < Context::kStages; ++k) {
         const unsigned both = (1u << k) | (1u << (k + 1));

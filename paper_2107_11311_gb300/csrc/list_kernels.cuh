@@ -1057,9 +1057,20 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
     for (int t = 0; t < kMaxSpecies; ++t)
         if (tid == t) s_tw[t] = B.type_weight[t];
     if constexpr (kSh) load_sh_table(B.sh_b, s_sh, tid);
-    if constexpr (MODE == kFused)
+    // the parameters arrive while the first atoms' descriptors are computed
+    if constexpr (MODE == kFused) {
+        const unsigned dst = (unsigned)__cvta_generic_to_shared(s_par);
         for (int k = tid; k < B.n_species * net.stride / 4; k += blockDim.x)
-            reinterpret_cast<float4 *>(s_par)[k] = __ldg(reinterpret_cast<const float4 *>(pnet) + k);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * k), "l"(pnet + 4 * k) : "memory");
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    bool staged = MODE != kFused;
+    auto wait_params = [&]() {  // once per warp (a CTA barrier): every thread's copies are complete
+        if (staged) return;
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        staged = true;
+    };
     if constexpr (CODES) {
         const int wx = 2 * g.m[0] + 1, wy = 2 * g.m[1] + 1;
         for (int o = tid; o < g.n_off; o += blockDim.x) {  // image shift of every list code
@@ -1267,6 +1278,7 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
             // ---- 3. the network
             float c0, c1;
             if constexpr (MODE == kFused) {
+                wait_params();
                 const float E = list_network<KRT, KAT, HB>(net, s_par + type * net.stride, W.coef, lane, G0, G1,
                                                            G_out ? G_out + (size_t)a * net.rec_len : nullptr, Kr, Ka,
                                                            c0, c1);
@@ -1391,6 +1403,7 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
         a = next;
     }
 
+    wait_params();  // (a warp without atoms)
     // ---- the CTA's partial sums
     if constexpr (MODE != kDescriptor && !BATCH) {
 #pragma unroll

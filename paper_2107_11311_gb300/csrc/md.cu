@@ -6,9 +6,10 @@
 // FP64 arithmetic has a long latency on this part, so every FP64 reduction is a
 // wide tree (independent accumulators per thread, then shuffles) rather than a
 // serial chain, divisions are replaced by host-computed reciprocals, and the
-// MD step runs in two kernels around the potential: kick + drift + binning, and
-// closing kick + all reductions (the last CTA to finish sums every partial in a
-// fixed order, so results are deterministic).
+// MD step has one kernel between two potentials (closing kick, all reductions,
+// opening kick, drift and binning; the last CTA to finish sums every partial in a
+// fixed order, so results are deterministic), or two around each where the next
+// step needs the reductions first.
 #include <algorithm>
 
 #include "aenet_internal.cuh"
@@ -200,23 +201,79 @@ __global__ void k_md_kick_drift_bin(int n, int n_species, KickParams kp, double 
     if (threadIdx.x == 0) *done = 0u;  // left at zero for the next user of the counter
 }
 
-// v += dt/2 F/m c with F of the current evaluation. Every CTA also sums a fixed
-// slice of the potential's energy and virial partial rows and its atoms'
-// kinetic energy into an 11-entry row of cta_part; the last CTA reduces those
-// rows into result[0..10] (energy, virial, kinetic energy) and appends
-// (E_pot, E_kin) to the records. The partition is by CTA index, so the FP64 sums
-// do not depend on scheduling.
-__global__ void __launch_bounds__(kMdThreads)
-    k_md_kick_finish(int n, KickParams kp, double *__restrict__ vel, const int32_t *__restrict__ types,
-                     const float4 *__restrict__ F4, const int *__restrict__ slot, int n_e,
-                     const double *__restrict__ e_part, int n_v,
-                     const double *__restrict__ vir_part, double *__restrict__ cta_part, unsigned *__restrict__ done,
-                     double *__restrict__ result, int *__restrict__ step, double *__restrict__ rec_pot,
-                     double *__restrict__ rec_kin, unsigned *__restrict__ vl_flag,
-                     unsigned long long *__restrict__ vl_builds, Thermostat th) {
+// The partial sums an MD step's closing reduction starts from, and where it ends.
+struct MdSums {
+    int n_e, n_v;                    // energy and virial partial rows of the evaluation
+    const double *e_part, *vir_part;
+    double *cta_part;                // [CTAs * 11]
+    unsigned *done;
+    double *result;                  // [11]: energy, virial, kinetic energy
+    int *step;
+    double *rec_pot, *rec_kin;       // records (E_pot, E_kin), or NULL
+};
+
+// Every CTA sums a fixed slice of the potential's energy and virial partial rows
+// and its atoms' kinetic energy (ke: this thread's) into an 11-entry row of
+// cta_part; the last CTA reduces those rows into result[0..10] and appends (E_pot,
+// E_kin) to the records; true in its threads. The partition is by CTA index, so
+// the FP64 sums do not depend on scheduling. Writes of all threads before the
+// call are visible to the last CTA.
+__device__ inline bool md_close(const MdSums &m, double ke) {
     __shared__ double s_w[kMdThreads / 32];
     __shared__ bool s_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    ke = warp_sum_d(ke);
+    if (lane == 0) s_w[warp] = ke;
+    double *row = m.cta_part + (size_t)blockIdx.x * 11;
+    for (int q = warp; q < 10; q += kMdThreads / 32) {
+        const int rows = q == 0 ? m.n_e : m.n_v;
+        const int per = (rows + gridDim.x - 1) / gridDim.x;
+        const int r0 = min(rows, (int)blockIdx.x * per), r1 = min(rows, r0 + per);
+        double a = 0.0;
+        for (int r = r0 + lane; r < r1; r += 32)
+            a += q == 0 ? __ldcg(m.e_part + r) : __ldcg(m.vir_part + (size_t)r * 9 + (q - 1));
+        a = warp_sum_d(a);
+        if (lane == 0) row[q] = a;
+    }
+    __threadfence();
+    __syncthreads();
+    if (warp == 0) {
+        double v = lane < kMdThreads / 32 ? s_w[lane] : 0.0;
+        v = warp_sum_d(v);
+        if (lane == 0) {
+            row[10] = v;
+            __threadfence();
+            s_last = atomicAdd(m.done, 1u) == gridDim.x - 1;
+        }
+    }
+    __syncthreads();
+    if (!s_last) return false;
+    __threadfence();
+    // the 11 columns over the CTAs' rows, one warp each
+    for (int q = warp; q < 11; q += kMdThreads / 32) {
+        const double v = warp_reduce_strided(m.cta_part + q, gridDim.x, 11, lane);
+        if (lane == 0) m.result[q] = v;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        *m.done = 0u;
+        if (m.rec_pot) {
+            const int s = *m.step;
+            m.rec_pot[s] = m.result[0];
+            m.rec_kin[s] = m.result[10];
+            *m.step = s + 1;
+        }
+    }
+    return true;
+}
+
+// v += dt/2 F/m c with F of the current evaluation, and the closing reduction; the
+// last CTA also clears the Verlet rebuild flag and computes the thermostat's factor.
+__global__ void __launch_bounds__(kMdThreads)
+    k_md_kick_finish(int n, KickParams kp, double *__restrict__ vel, const int32_t *__restrict__ types,
+                     const float4 *__restrict__ F4, const int *__restrict__ slot, MdSums sums,
+                     unsigned *__restrict__ vl_flag, unsigned long long *__restrict__ vl_builds, Thermostat th) {
+    const int tid = threadIdx.x;
     const int i = blockIdx.x * blockDim.x + tid;
     double ke = 0.0;
     if (i < n) {
@@ -231,57 +288,65 @@ __global__ void __launch_bounds__(kMdThreads)
         vel[3 * i + 2] = vz;
         ke = select_species(kp.hm, t) * fma(vx, vx, fma(vy, vy, vz * vz));
     }
-    ke = warp_sum_d(ke);
-    if (lane == 0) s_w[warp] = ke;
-    // this CTA's slice of the energy (q = 0) and virial (q = 1..9) partial rows
-    double *row = cta_part + (size_t)blockIdx.x * 11;
-    for (int q = warp; q < 10; q += kMdThreads / 32) {
-        const int rows = q == 0 ? n_e : n_v;
-        const int per = (rows + gridDim.x - 1) / gridDim.x;
-        const int r0 = min(rows, (int)blockIdx.x * per), r1 = min(rows, r0 + per);
-        double a = 0.0;
-        for (int r = r0 + lane; r < r1; r += 32)
-            a += q == 0 ? __ldcg(e_part + r) : __ldcg(vir_part + (size_t)r * 9 + (q - 1));
-        a = warp_sum_d(a);
-        if (lane == 0) row[q] = a;
-    }
-    __syncthreads();
-    if (warp == 0) {
-        double v = lane < kMdThreads / 32 ? s_w[lane] : 0.0;
-        v = warp_sum_d(v);
-        if (lane == 0) {
-            row[10] = v;
-            __threadfence();
-            s_last = atomicAdd(done, 1u) == gridDim.x - 1;
-        }
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    // last CTA: the 11 columns over the CTAs' rows, one warp each
-    for (int q = warp; q < 11; q += kMdThreads / 32) {
-        const double v = warp_reduce_strided(cta_part + q, gridDim.x, 11, lane);
-        if (lane == 0) result[q] = v;
-    }
-    __syncthreads();
+    if (!md_close(sums, ke)) return;
     if (tid == 0) {
-        *done = 0u;
         if (vl_flag && vl_flag[0]) {  // this step rebuilt the Verlet list
             ++*vl_builds;
             vl_flag[0] = 0u;
         }
-        if (rec_pot) {
-            const int s = *step;
-            rec_pot[s] = result[0];
-            rec_kin[s] = result[10];
-            *step = s + 1;
-        }
         if (th.lambda) {  // Berendsen factor of the next step, from this frame's temperature
-            const double T = 2.0 * result[10] * th.inv_dof_kb;
+            const double T = 2.0 * sums.result[10] * th.inv_dof_kb;
             const double l2 = T > 0.0 ? 1.0 + th.dt_over_tau * (th.T0 / T - 1.0) : 1.0;
             *th.lambda = l2 > 0.0 ? sqrt(l2) : 0.0;
         }
     }
+}
+
+// Between two steps of a call: the closing kick and reduction of one step
+// (k_md_kick_finish) and the opening kick, drift and binning of the next
+// (k_md_kick_drift_bin) in one pass over the atoms: positions, velocities and
+// forces are read once, and a step has one launch less (about 10 us on 1,536
+// atoms, whose step is a chain of launch latencies). The last CTA also scans the
+// cell counts when fold. NVE only: a thermostat's factor needs the reduction first.
+__global__ void __launch_bounds__(kMdThreads)
+    k_md_turn(int n, int n_species, KickParams kp, double dt, double *__restrict__ pos, double *__restrict__ vel,
+              const int32_t *__restrict__ types, float4 *__restrict__ F4, Grid g, float4 *__restrict__ tmp4,
+              int *__restrict__ cell_of, int *__restrict__ slot, int *__restrict__ cell_count,
+              int *__restrict__ cell_start, bool fold, unsigned long long *__restrict__ stats,
+              unsigned *__restrict__ err, MdSums sums) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < 4) stats[i] = 0ull;
+    double ke = 0.0;
+    if (i < n) {
+        int t = types[i];
+        if (t < 0 || t >= n_species) {
+            atomicOr(err, kErrType);
+            t = 0;
+        }
+        const int s_old = slot[i];
+        const float4 f = F4[s_old];
+        F4[s_old] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const double k = select_species(kp.k, t);
+        const float fa[3] = {f.x, f.y, f.z};
+        double x[3], v[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            v[a] = fma(k, (double)fa[a], vel[3 * i + a]);          // closing kick
+            const double w = fma(k, (double)fa[a], v[a]);          // opening kick
+            x[a] = fma(dt, w, pos[3 * i + a]);
+            vel[3 * i + a] = w;
+            pos[3 * i + a] = x[a];
+        }
+        ke = select_species(kp.hm, t) * fma(v[0], v[0], fma(v[1], v[1], v[2] * v[2]));
+        float u[3];
+        bool finite = true;
+        const int cell = bin_position(x[0], x[1], x[2], g, u, finite);
+        if (!finite) atomicOr(err, kErrNonfinite);
+        tmp4[i] = make_float4(u[0], u[1], u[2], __int_as_float(t));
+        cell_of[i] = cell;
+        slot[i] = atomicAdd(&cell_count[cell], 1);
+    }
+    if (md_close(sums, ke) && fold) scan_cells_block(g.ncell, cell_count, cell_start);
 }
 
 // Verlet form of v += dt/2 F/m c; x += dt v (the list is kept, nothing is
@@ -517,6 +582,13 @@ cudaError_t launch_batch_reduce(Context &c, bool atoms, double *energies, double
     return cudaGetLastError();
 }
 
+static bool scan_folds(const Grid &g) { return g.ncell <= 4 * kMdThreads; }
+
+static MdSums md_sums(const Context &c, double *rec_pot, double *rec_kin) {
+    return MdSums{c.last_eparts, c.last_vparts, c.last_epart, c.last_vpart, c.d_ke_part, c.d_done,
+                  c.d_result,    c.d_step,      rec_pot,      rec_kin};
+}
+
 // Kick, drift, binning and the scan of the cell counts (the cell counts are
 // zero: every binning is followed by a scan, which clears them, and a newly
 // allocated count array is cleared once); k_scatter follows (launch_scatter).
@@ -526,7 +598,7 @@ cudaError_t launch_batch_reduce(Context &c, bool atoms, double *energies, double
 cudaError_t launch_md_kick_drift_bin(Context &c, const Grid &g, int n, double dt, double *pos, double *vel,
                                      const int32_t *types) {
     if (n <= 0) return launch_sort(c, g, n);  // no atoms: the (all-zero) cell starts still come from a scan
-    const bool fold = g.ncell <= 4 * kMdThreads;
+    const bool fold = scan_folds(g);
     k_md_kick_drift_bin<<<(n + kMdThreads - 1) / kMdThreads, kMdThreads, 0, c.stream>>>(
         n, c.basis.n_species, kick_params(c, dt), dt, pos, vel, types, c.d_F4, g, c.d_tmp4, c.d_cell_of, c.d_slot,
         c.d_cell_count, c.d_cell_start, fold ? c.d_done : nullptr, c.d_stats, c.d_err,
@@ -546,11 +618,22 @@ cudaError_t launch_scale(Context &c, double *x, long long count, double mu) {
 cudaError_t launch_md_kick_finish(Context &c, int n, double dt, double *vel, const int32_t *types,
                                   double *rec_pot, double *rec_kin, bool clear_vl) {
     const int blocks = n > 0 ? (n + kMdThreads - 1) / kMdThreads : 1;
-    k_md_kick_finish<<<blocks, kMdThreads, 0, c.stream>>>(
-        n, kick_params(c, dt), vel, types, c.d_F4, c.d_slot, c.last_eparts,
-        c.last_epart, c.last_vparts, c.last_vpart, c.d_ke_part, c.d_done, c.d_result, c.d_step, rec_pot, rec_kin,
-        clear_vl ? c.d_vl_flag : nullptr, c.d_vl_builds, thermostat(c, n));
+    k_md_kick_finish<<<blocks, kMdThreads, 0, c.stream>>>(n, kick_params(c, dt), vel, types, c.d_F4, c.d_slot,
+                                                          md_sums(c, rec_pot, rec_kin),
+                                                          clear_vl ? c.d_vl_flag : nullptr, c.d_vl_builds,
+                                                          thermostat(c, n));
     return cudaGetLastError();
+}
+
+cudaError_t launch_md_turn(Context &c, const Grid &g, int n, double dt, double *pos, double *vel,
+                           const int32_t *types, double *rec_pot, double *rec_kin) {
+    const bool fold = scan_folds(g);
+    k_md_turn<<<(n + kMdThreads - 1) / kMdThreads, kMdThreads, 0, c.stream>>>(
+        n, c.basis.n_species, kick_params(c, dt), dt, pos, vel, types, c.d_F4, g, c.d_tmp4, c.d_cell_of, c.d_slot,
+        c.d_cell_count, c.d_cell_start, fold, c.d_stats, c.d_err, md_sums(c, rec_pot, rec_kin));
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess || fold) return e;
+    return launch_scan(c, g);
 }
 
 cudaError_t launch_md_vl_kick_drift(Context &c, int n, double dt, double *pos, double *vel, const int32_t *types,
