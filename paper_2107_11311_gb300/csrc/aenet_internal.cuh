@@ -64,6 +64,7 @@ struct Grid {
     double inv_box[3];             // reciprocals: no FP64 division on the device
     double inv_h[3];
     float hf[3];
+    float inv_boxf[3];
     int tri;                       // any tilt != 0
     double tilt[3];                // xy, xz, yz
     double ht[3];                  // off-diagonal of the cell edges: B_x = xy / nc[1], C_x = xz / nc[2], C_y = yz / nc[2]
@@ -115,21 +116,36 @@ __device__ inline int bin_position(double x0, double x1, double x2, const Grid &
         }
         return (ci[2] * g.nc[1] + ci[1]) * g.nc[0] + ci[0];
     }
+    // FP64 instructions run at 1/64 of the FP32 rate here: the box an atom lies in is
+    // found in FP32 (off by one box at most, put right by the sign of w and the cell
+    // index), so that the usual atom costs five FP64 operations per axis.
     const double xs[3] = {x0, x1, x2};
     int ci[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         double x = xs[a];
-        if (!isfinite(x)) {
-            finite = false;
-            x = 0.0;
+        const float xf = (float)x;
+        float k = floorf(xf * g.inv_boxf[a]);
+        if (!(fabsf(k) < 4096.0f)) {  // far from the box (or not finite): the exact form
+            if (!isfinite(x)) {
+                finite = false;
+                x = 0.0;
+            }
+            const double L = g.box[a];
+            x = fma(-floor(x * g.inv_box[a]), L, x);
+            if (x >= L) x -= L;
+            k = 0.f;
         }
-        const double L = g.box[a];
-        double w = fma(-floor(x * g.inv_box[a]), L, x);
-        if (w >= L) w -= L;
-        if (w < 0.0) w = 0.0;
+        double w = k == 0.f ? x : fma(-(double)k, g.box[a], x);
+        if (__double2hiint(w) < 0) w += g.box[a];
         int c = (int)(w * g.inv_h[a]);
-        c = c >= g.nc[a] ? g.nc[a] - 1 : c;
+        if (c >= g.nc[a]) {
+            if (w >= g.box[a]) {
+                w -= g.box[a];
+                c = (int)(w * g.inv_h[a]);
+            }
+            c = c >= g.nc[a] ? g.nc[a] - 1 : c;
+        }
         ci[a] = c;
         const double ua = fma(-(double)c, g.h[a], w);
         u[a] = (float)ua;
@@ -163,6 +179,7 @@ struct Context {
     bool own_stream = false;
     int precision = AENET_FP32;
     bool fuse_network = true;      // BF16 forms: tensor-core network inside the fused kernel
+    bool pdl = false;              // set while a chain of kernels without event records is enqueued (pdl.cuh)
     int eval_n = 0;                // atoms of the evaluation being set up (tc_fused_supported)
     bool batch_call = false;       // set during the batch entry points
     bool cell_search = false;      // set while an MD step with AENET_MD_LIST_OFF is enqueued

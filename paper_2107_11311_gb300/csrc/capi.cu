@@ -99,6 +99,7 @@ int make_grid(Context &c, const double *box, Grid &g, double rc_cut = 0.0, const
         g.hf[a] = (float)g.h[a];
         g.inv_box[a] = 1.0 / g.box[a];
         g.inv_h[a] = 1.0 / g.h[a];
+        g.inv_boxf[a] = (float)g.inv_box[a];
         g.m[a] = g.tri ? (int)ceil(rc * nc / w[a]) : (int)ceil(rc / g.h[a]);
         g.ncell *= nc;
         g.n_off *= 2 * g.m[a] + 1;
@@ -301,6 +302,15 @@ int enqueue_rows(Context &c, const Grid &g, int n, RowsMode mode) {
     return AENET_OK;
 }
 
+// While it lives, launches of the context may overlap their predecessors' tails
+// (programmatic dependent launch), unless stage events lie between them.
+struct Overlap {
+    Context &c;
+    bool was;
+    explicit Overlap(Context &ctx) : c(ctx), was(ctx.pdl) { c.pdl = c.ev_mask == 0u; }
+    ~Overlap() { c.pdl = was; }
+};
+
 // Descriptor, networks and forces after the cell list (fused kernel or the
 // three split kernels), with stage events 3, 4 (after descriptor, network) and
 // 5 (after forces) when selected. *n_eparts = number of energy partials written.
@@ -351,6 +361,7 @@ int enqueue_potential(Context &c, const Grid &g, int n, int *n_eparts) {
 // and the error word also to c.h_res.
 int enqueue_compute(Context &c, const Grid &g, int n, const double *pos, const int32_t *types, double *forces,
                     double *e_atom, double *energy = nullptr, double *virial = nullptr, bool to_host = false) {
+    const Overlap overlap(c);
     int rc = check_smem(c, g);
     if (rc) return rc;
     CK(launch_cells(c, g, n, pos, types), "cell list");
@@ -629,6 +640,7 @@ static int compute_impl(Context &c, int n, const double *pos, const int32_t *typ
         if (G_out) {
             if ((rc = check_smem(c, g))) return rc;
             if ((rc = ensure_G(c, n, !G_dev))) return rc;
+            const Overlap overlap(c);
             CK(launch_cells(c, g, n, dpos, dtypes), "cell list");
             if ((rc = enqueue_rows(c, g, n, RowsMode::descriptor))) return rc;
             CK(launch_unsort_G(c, n, G_dev ? G_out : c.d_dEdG), "unsort");  // (host rows: the other row buffer first)
@@ -796,6 +808,7 @@ int batch_enqueue(Context &c, const BatchLayout &L, const StructInfo *sinfo, con
                   const int32_t *dtypes, double *dF, double *energies, double *virials) {
     int rc = check_smem(c, L.gall);
     if (rc) return rc;
+    const Overlap overlap(c);
     c.batch_sinfo = sinfo;
     c.batch_order = order;
     c.batch_n = (int)L.info.size();
@@ -1140,6 +1153,7 @@ static int enqueue_md_forces(Context &c, const Grid &g, int n, bool rows) {
 
 static int enqueue_md_step(Context &c, const Grid &g, int n, double dt, double *pos, double *vel,
                            const int32_t *types, double *rec, bool rows) {
+    const Overlap overlap(c);
     CK(mark(c, 0), "event");
     CK(launch_md_kick_drift_bin(c, g, n, dt, pos, vel, types), "kick + drift + binning + scan");
     CK(mark(c, 1), "event");
@@ -1378,6 +1392,7 @@ static int md_fixed_cell(aenet_ctx *h, int n, double *pos, double *vel, const in
             c.ev_mask = ev_mask;
             int src;
             if (turn) {
+                const Overlap overlap(c);
                 src = enqueue_md_forces(c, g, n, rows);
                 cudaError_t te = cudaSuccess;
                 if (!src) te = launch_md_turn(c, g, n, dt, dpos, dvel, dtypes, rec, rec ? rec + c.cap_rec : nullptr);
@@ -1422,6 +1437,7 @@ static int md_fixed_cell(aenet_ctx *h, int n, double *pos, double *vel, const in
         if (verlet && (!cont || !c.vl_valid))
             CK(cudaMemsetAsync(c.d_vl_flag, 0xff, sizeof(unsigned), c.stream), "cudaMemsetAsync");
         if (turn) {
+            const Overlap overlap(c);
             CK(launch_md_kick_drift_bin(c, g, n, dt, dpos, dvel, dtypes), "kick + drift + binning + scan");
             for (int s = 1; s < n_steps; ++s) CK(cudaGraphLaunch(exec, c.stream), "graph launch");
             if ((rc = enqueue_md_forces(c, g, n, rows))) return rc;

@@ -8,6 +8,7 @@
 // ~1e-5 A.
 #include "aenet_internal.cuh"
 #include "cell_scan.cuh"
+#include "pdl.cuh"
 
 namespace aenet {
 
@@ -61,6 +62,7 @@ __global__ void k_bin_count_batch(int n, int n_struct, int n_species, const doub
 
 // Exclusive scan of the cell counts by one CTA (scan_cells_block).
 __global__ void k_scan_cells(int ncell, int *__restrict__ count, int *__restrict__ start) {
+    pdl_wait();
     scan_cells_block(ncell, count, start);
 }
 
@@ -70,6 +72,7 @@ __global__ void k_scatter(int n, const float4 *__restrict__ tmp4, const int *__r
                           int *__restrict__ slot, const int *__restrict__ cell_start,
                           float4 *__restrict__ pos4, int *__restrict__ perm) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait();
     if (i >= n) return;
     int s = cell_start[cell_of[i]] + slot[i];
     pos4[s] = tmp4[i];
@@ -78,24 +81,18 @@ __global__ void k_scatter(int n, const float4 *__restrict__ tmp4, const int *__r
 }
 
 cudaError_t launch_scan(Context &c, const Grid &g) {
-    k_scan_cells<<<1, 1024, 0, c.stream>>>(g.ncell, c.d_cell_count, c.d_cell_start);
-    return cudaGetLastError();
+    return launch_after(c.pdl, k_scan_cells, 1, 1024, 0, c.stream, g.ncell, c.d_cell_count, c.d_cell_start);
 }
 
 cudaError_t launch_scatter(Context &c, int n) {
-    if (n > 0)
-        k_scatter<<<(n + 255) / 256, 256, 0, c.stream>>>(n, c.d_tmp4, c.d_cell_of, c.d_slot, c.d_cell_start,
-                                                         c.d_pos4, c.d_perm);
-    return cudaGetLastError();
+    if (n <= 0) return cudaSuccess;
+    return launch_after(c.pdl, k_scatter, (n + 255) / 256, 256, 0, c.stream, n, c.d_tmp4, c.d_cell_of, c.d_slot,
+                        c.d_cell_start, c.d_pos4, c.d_perm);
 }
 
 cudaError_t launch_sort(Context &c, const Grid &g, int n) {
-    k_scan_cells<<<1, 1024, 0, c.stream>>>(g.ncell, c.d_cell_count, c.d_cell_start);
-    if (n > 0) {
-        k_scatter<<<(n + 255) / 256, 256, 0, c.stream>>>(n, c.d_tmp4, c.d_cell_of, c.d_slot, c.d_cell_start,
-                                                         c.d_pos4, c.d_perm);
-    }
-    return cudaGetLastError();
+    const cudaError_t e = launch_scan(c, g);
+    return e != cudaSuccess ? e : launch_scatter(c, n);
 }
 
 cudaError_t launch_cells(Context &c, const Grid &g, int n, const double *pos, const int32_t *types) {

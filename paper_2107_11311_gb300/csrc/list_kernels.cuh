@@ -16,6 +16,9 @@
 // from step to step.
 #pragma once
 
+#include <type_traits>
+
+#include "pdl.cuh"
 #include "potential_kernels.cuh"
 
 namespace aenet {
@@ -73,6 +76,7 @@ __global__ void __launch_bounds__(kBuildThreads, 12)
     __shared__ int s_kept, s_next;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned lt_mask = (1u << lane) - 1u;
+    pdl_wait();
     if (stats && blockIdx.x == 0 && tid < 4) stats[tid] = 0ull;
     const int cell = blockIdx.x / parts, part = blockIdx.x - cell * parts;
     int first = cell_start[cell], n = cell_start[cell + 1] - first;
@@ -183,11 +187,11 @@ __global__ void __launch_bounds__(kBuildThreads, 12)
             if (a >= n) break;
             float mx[kBuildAtoms], my[kBuildAtoms], mz[kBuildAtoms], lim[kBuildAtoms];  // -2u; rc^2 - |u|^2
             int cnt[kBuildAtoms];
-            size_t row[kBuildAtoms];
+            typename std::conditional<CODES, size_t, unsigned>::type row[kBuildAtoms];  // (a slice: < 2^26 entries)
 #pragma unroll
             for (int b = 0; b < kBuildAtoms; ++b) {
                 const int i = first + min(a + b, n - 1);
-                row[b] = (size_t)(i - (CODES ? 0 : a_lo)) * cap;
+                row[b] = (decltype(row[b] + 0))(i - (CODES ? 0 : a_lo)) * cap;
                 const float4 u = pos4[i];
                 const float u2 = u.x * u.x + u.y * u.y + u.z * u.z, ur = sqrtf(u2) + rc;
                 mx[b] = -2.f * u.x;
@@ -1082,6 +1086,7 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
     if (lane < 4) s_sum.st[warp][lane] = 0ull;
     if (lane == 0) s_sum.e[warp] = 0.0;
     __syncthreads();
+    pdl_wait();  // (what is above reads only what the kernels of the evaluation leave alone)
 
     const float inv_rcr = 1.0f / B.rc_rad, inv_rca = 1.0f / B.rc_ang, rc2max = B.rc_max * B.rc_max;
     const int nb = caps.nb;

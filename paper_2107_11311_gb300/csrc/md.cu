@@ -14,6 +14,7 @@
 
 #include "aenet_internal.cuh"
 #include "cell_scan.cuh"
+#include "pdl.cuh"
 
 namespace aenet {
 
@@ -82,6 +83,7 @@ __global__ void __launch_bounds__(kRedThreads)
     k_finalize(int n, const int *__restrict__ perm, const float4 *__restrict__ F4, const float *__restrict__ eatom,
                int n_e, const double *__restrict__ e_part, int n_v, const double *__restrict__ vir_part,
                double *__restrict__ result, const unsigned *__restrict__ err, FinalizeOut o) {
+    pdl_wait();
     if (blockIdx.x < kReduceCtas) {
         const int lane = threadIdx.x & 31;
         const int q = blockIdx.x * (kRedThreads / 32) + (threadIdx.x >> 5);
@@ -230,9 +232,11 @@ __device__ inline bool md_close(const MdSums &m, double ke) {
         const int per = (rows + gridDim.x - 1) / gridDim.x;
         const int r0 = min(rows, (int)blockIdx.x * per), r1 = min(rows, r0 + per);
         double a = 0.0;
-        for (int r = r0 + lane; r < r1; r += 32)
-            a += q == 0 ? __ldcg(m.e_part + r) : __ldcg(m.vir_part + (size_t)r * 9 + (q - 1));
-        a = warp_sum_d(a);
+        if (r0 < r1) {  // (most CTAs of a large system have no row)
+            for (int r = r0 + lane; r < r1; r += 32)
+                a += q == 0 ? __ldcg(m.e_part + r) : __ldcg(m.vir_part + (size_t)r * 9 + (q - 1));
+            a = warp_sum_d(a);
+        }
         if (lane == 0) row[q] = a;
     }
     __threadfence();
@@ -275,6 +279,7 @@ __global__ void __launch_bounds__(kMdThreads)
                      unsigned *__restrict__ vl_flag, unsigned long long *__restrict__ vl_builds, Thermostat th) {
     const int tid = threadIdx.x;
     const int i = blockIdx.x * blockDim.x + tid;
+    pdl_wait();
     double ke = 0.0;
     if (i < n) {
         const int t = types[i];
@@ -315,6 +320,7 @@ __global__ void __launch_bounds__(kMdThreads)
               int *__restrict__ cell_start, bool fold, unsigned long long *__restrict__ stats,
               unsigned *__restrict__ err, MdSums sums) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait();
     if (i < 4) stats[i] = 0ull;
     double ke = 0.0;
     if (i < n) {
@@ -550,10 +556,9 @@ __global__ void k_scale(double *__restrict__ x, long long count, double mu) {
 cudaError_t launch_finalize(Context &c, int n, int n_eparts, double *forces, double *e_atom, double *energy,
                             double *virial, bool to_host) {
     const int blocks = kReduceCtas + ((forces || e_atom) && n > 0 ? (n + kRedThreads - 1) / kRedThreads : 0);
-    k_finalize<<<blocks, kRedThreads, 0, c.stream>>>(
-        n, c.d_perm, c.d_F4, c.d_eatom, n_eparts, c.last_epart, c.last_vparts, c.last_vpart, c.d_result, c.d_err,
-        FinalizeOut{forces, e_atom, energy, virial, to_host ? c.h_res : nullptr});
-    return cudaGetLastError();
+    return launch_after(c.pdl, k_finalize, blocks, kRedThreads, 0, c.stream, n, c.d_perm, c.d_F4, c.d_eatom, n_eparts,
+                        c.last_epart, c.last_vparts, c.last_vpart, c.d_result, c.d_err,
+                        FinalizeOut{forces, e_atom, energy, virial, to_host ? c.h_res : nullptr});
 }
 
 cudaError_t launch_finalize_forces(Context &c, int n, double *forces) {
@@ -618,20 +623,21 @@ cudaError_t launch_scale(Context &c, double *x, long long count, double mu) {
 cudaError_t launch_md_kick_finish(Context &c, int n, double dt, double *vel, const int32_t *types,
                                   double *rec_pot, double *rec_kin, bool clear_vl) {
     const int blocks = n > 0 ? (n + kMdThreads - 1) / kMdThreads : 1;
-    k_md_kick_finish<<<blocks, kMdThreads, 0, c.stream>>>(n, kick_params(c, dt), vel, types, c.d_F4, c.d_slot,
-                                                          md_sums(c, rec_pot, rec_kin),
-                                                          clear_vl ? c.d_vl_flag : nullptr, c.d_vl_builds,
-                                                          thermostat(c, n));
-    return cudaGetLastError();
+    return launch_after(false, k_md_kick_finish, blocks, kMdThreads, 0, c.stream, n, kick_params(c, dt), vel, types,
+                        c.d_F4, c.d_slot, md_sums(c, rec_pot, rec_kin), clear_vl ? c.d_vl_flag : nullptr,
+                        c.d_vl_builds, thermostat(c, n));
 }
 
 cudaError_t launch_md_turn(Context &c, const Grid &g, int n, double dt, double *pos, double *vel,
                            const int32_t *types, double *rec_pot, double *rec_kin) {
     const bool fold = scan_folds(g);
-    k_md_turn<<<(n + kMdThreads - 1) / kMdThreads, kMdThreads, 0, c.stream>>>(
-        n, c.basis.n_species, kick_params(c, dt), dt, pos, vel, types, c.d_F4, g, c.d_tmp4, c.d_cell_of, c.d_slot,
-        c.d_cell_count, c.d_cell_start, fold, c.d_stats, c.d_err, md_sums(c, rec_pot, rec_kin));
-    const cudaError_t e = cudaGetLastError();
+    // (an ordinary launch: placed early, its CTAs would crowd the first SMs that the
+    // list kernel leaves, and FP64 bounds it: MD of 12,288 atoms 124 us a step
+    // instead of 101)
+    const cudaError_t e = launch_after(false, k_md_turn, (n + kMdThreads - 1) / kMdThreads, kMdThreads, 0, c.stream, n,
+                                       c.basis.n_species, kick_params(c, dt), dt, pos, vel, types, c.d_F4, g, c.d_tmp4,
+                                       c.d_cell_of, c.d_slot, c.d_cell_count, c.d_cell_start, fold, c.d_stats, c.d_err,
+                                       md_sums(c, rec_pot, rec_kin));
     if (e != cudaSuccess || fold) return e;
     return launch_scan(c, g);
 }

@@ -286,6 +286,7 @@ extern "C" int aenet_descriptors_noalloc(int n, const double *pos, const int32_t
         g.hf[a] = (float)g.h[a];
         g.inv_box[a] = 1.0 / g.box[a];
         g.inv_h[a] = 1.0 / g.h[a];
+        g.inv_boxf[a] = (float)g.inv_box[a];
         g.m[a] = (int)ceil(B.rc_max / g.h[a]);
         g.ncell *= nc;
         g.n_off *= 2 * g.m[a] + 1;
