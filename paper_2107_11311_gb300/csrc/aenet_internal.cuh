@@ -160,6 +160,10 @@ __device__ inline int bin_position(double x0, double x1, double x2, const Grid &
 struct StructInfo {
     Grid g;
     int cell0, ncell, atom0, natoms;
+    // the list build's CTAs of the structure are item0 .. item0 + ncell parts - 1: a cell
+    // is divided into parts of about 24 atoms, since a small box is one cell of up to some
+    // hundred atoms that see thousands of image-atoms (a solid of 250 atoms: 6,750)
+    int item0, parts;
 };
 
 // Capacities of the per-warp neighbour lists of the potential kernel, and the
@@ -263,6 +267,7 @@ struct Context {
     double *d_bres = nullptr;          // [n_struct * 10]: energy, virial[9]
     const StructInfo *batch_sinfo = nullptr;  // non-NULL while a batch is enqueued
     int batch_n = 0;
+    int batch_items = 0;               // CTAs of its list build
 
     // Verlet neighbour list with a skin (MD steps of the fused FP32 form; skin 0 =
     // the cell list every step). Entries: sorted index | image-offset code << jbits,

@@ -78,7 +78,23 @@ __global__ void __launch_bounds__(kBuildThreads, 12)
     const unsigned lt_mask = (1u << lane) - 1u;
     pdl_wait();
     if (stats && blockIdx.x == 0 && tid < 4) stats[tid] = 0ull;
-    const int cell = blockIdx.x / parts, part = blockIdx.x - cell * parts;
+    int cell, part, sidx = 0;
+    if constexpr (BATCH) {  // the structure whose CTAs (cells x parts) this is one of
+        int lo = 0, hi = n_struct - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (sinfo[mid].item0 <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
+        }
+        sidx = lo;
+        parts = sinfo[sidx].parts;
+        const int k = (int)blockIdx.x - sinfo[sidx].item0;
+        cell = k / parts;
+        part = k - cell * parts;
+        cell += sinfo[sidx].cell0;
+    } else {
+        cell = blockIdx.x / parts;
+        part = blockIdx.x - cell * parts;
+    }
     int first = cell_start[cell], n = cell_start[cell + 1] - first;
     {
         const int lo = part * n / parts, hi = (part + 1) * n / parts;
@@ -93,15 +109,6 @@ __global__ void __launch_bounds__(kBuildThreads, 12)
     int *off_prefix = reinterpret_cast<int *>(smem + L.off_prefix);
     float4 *off_shift = reinterpret_cast<float4 *>(smem + L.off_shift);
     float4 *s_pos = reinterpret_cast<float4 *>(smem + L.s_pos);
-    int sidx = 0;
-    if constexpr (BATCH) {  // the structure that owns the cell
-        int lo = 0, hi = n_struct - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (sinfo[mid].cell0 <= cell) lo = mid; else hi = mid - 1;
-        }
-        sidx = lo;
-    }
     const Grid &g = BATCH ? sinfo[sidx].g : g_one;
     const int cell0 = BATCH ? sinfo[sidx].cell0 : 0;
     const int n_off = g.n_off;

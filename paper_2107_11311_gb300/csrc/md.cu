@@ -484,7 +484,7 @@ __global__ void k_batch_reduce(int n_struct, const StructInfo *__restrict__ sinf
 
 // The same from every atom's energy and virial (six sums, the list kernel): one
 // CTA per structure, a thread's atoms in FP64 and then a tree, in a fixed order.
-constexpr int kBatchThreads = 128;
+constexpr int kBatchThreads = 256;
 __global__ void __launch_bounds__(kBatchThreads)
     k_batch_reduce_atoms(const StructInfo *__restrict__ sinfo, const int *__restrict__ cell_start,
                          const float *__restrict__ eatom, const float *__restrict__ vir_atom,

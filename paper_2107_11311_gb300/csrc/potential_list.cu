@@ -28,14 +28,13 @@ cudaError_t launch_build(Context &c, const Grid &g, int n, int a_lo, int a_hi, b
     // idle (a part restages the neighbourhood); a part has at least 4 atoms
     const double per_cell = (double)n / std::max(1, g.ncell);
     const int parts =
-        c.batch_sinfo ? 1
-                      : std::max(1, std::min((4 * std::max(1, c.n_sm) + g.ncell - 1) / std::max(1, g.ncell),
-                                             (int)(per_cell / 4.0)));
+        std::max(1, std::min((4 * std::max(1, c.n_sm) + g.ncell - 1) / std::max(1, g.ncell), (int)(per_cell / 4.0)));
+    const int ctas = c.batch_sinfo ? c.batch_items : g.ncell * parts;  // (a batch: parts of each structure's own)
     auto kern = c.batch_sinfo ? k_list_build<true, false> : codes ? k_list_build<false, true> : k_list_build<false, false>;
     cudaError_t e = allow_max_smem(kern);
     if (e != cudaSuccess) return e;
     return launch_after(
-        c.pdl, kern, g.ncell * parts, kBuildThreads, smem, c.stream, g, c.batch_sinfo, c.batch_n,
+        c.pdl, kern, ctas, kBuildThreads, smem, c.stream, g, c.batch_sinfo, c.batch_n,
         codes ? c.caps.rc_list : c.basis.rc_max, tile, parts, a_lo, a_hi, c.d_pos4,
         c.d_cell_start, c.d_rows, c.d_vl, codes ? c.caps.vl_cap : c.caps.nb, c.caps.vl_jbits,
         codes ? c.d_vl_count : c.d_list_count, clear ? c.d_F4 : nullptr, clear ? c.d_stats : nullptr, c.d_err);
