@@ -32,7 +32,7 @@ constexpr int kEntryIndex = 0x0fffffff;  // sorted index of a list entry; the bi
 // ------------------------------------------------------------------ the build
 
 constexpr int kBuildThreads = 128;
-constexpr int kBuildAtoms = 2;  // atoms a warp tests every staged image-atom against
+constexpr int kBuildAtoms = 3;  // atoms a warp tests every staged image-atom against
 
 struct BuildLayout {
     size_t off_start, off_prefix, off_shift, s_pos, total;
@@ -59,15 +59,16 @@ __host__ __device__ inline BuildLayout make_build_layout(int n_off, int tile) {
 //     memory; in an orthorhombic box only those within the cutoff of the cell
 //     itself (about 72% of a 27-cell neighbourhood). More than `tile` of them
 //     are taken in chunks.
-//  2. Each warp tests the staged atoms against two atoms at a time (four: 40 more registers, 3% slower). With
-//     t = |p|^2 - 2 p.u the test is t <= rc^2 - |u|^2, three FMAs per pair;
+//  2. Each warp tests the staged atoms against three atoms at a time (whole
+//     evaluation: water 12,288 atoms, two at 12 CTAs per SM 94 us, three at 10
+//     91 us; water 98,304, four at 8 515 us, two at 12 507 us). With t = |p|^2 - 2 p.u the test is t <= rc^2 - |u|^2, three FMAs per pair;
 //     its rounding is covered by a margin (the potential kernel applies the
 //     exact cutoff to the displacement). The atom itself passes the test and
 //     is dropped there too.
 // It also clears the atoms' force accumulators and the neighbour statistics (F4
 // and stats, when given).
 template <bool BATCH, bool CODES>
-__global__ void __launch_bounds__(kBuildThreads, 12)
+__global__ void __launch_bounds__(kBuildThreads, 10)
     k_list_build(Grid g_one, const StructInfo *__restrict__ sinfo, int n_struct, float rc, int tile, int parts,
                  int a_lo, int a_hi, const float4 *__restrict__ pos4, const int *__restrict__ cell_start,
                  float4 *__restrict__ rows, int *__restrict__ codes, int cap, int jbits, int *__restrict__ count,
@@ -845,9 +846,91 @@ __device__ __forceinline__ void sh_fingerprints(const float *sh, const float *ta
     }
 }
 
-// (V, B) of every angular entry: with the coefficient pairs (D_c, D'_c) = 2 N_c^2
-// (A_c k_l, A'_c k'_l), k_l = sum_a g_a b_al, written over the component sums, V is
-// the contraction's gradient F and B = E - 2 w (sum_a g_a + s^2 sum_a g'_a).
+// Where the contraction's coefficients of component c lie in the warp's scratch:
+// m = 0: the pairs (D, D') of l = 0 .. 6 at [2l]; m > 0: the quad (D_cos, D_sin,
+// D'_cos, D'_sin) of (l, m) at [16 + 4 q], q counting the (l, m) column by column.
+constexpr int kShQuads = 16;
+
+// E = sum_c k_c v_c(u) and F = sum_c k_c grad_u v_c(u) of one entry, k_c = D_c + s
+// D'_c (sh_contract with cosine and sine parts packed: one 128-bit load and three
+// packed FMAs per (l, m)). Called by all 32 lanes together.
+__device__ __forceinline__ void sh_contract2(float x, float y, float z, float s, const float *D, float &E, float &Fx,
+                                             float &Fy, float &Fz) {
+    __syncwarp();  // (keeps the loads of one column from moving above the one before)
+    const float2 s2 = dup2(s), z2 = dup2(z);
+    float h0 = 0.f, d0 = 0.f;
+    {
+        float p2 = 0.f, p1 = 1.f, q2 = 0.f, q1 = 0.f;  // P_l and P_l'
+#pragma unroll
+        for (int l = 0; l <= kShL; ++l) {
+            float p = p1, d = 0.f;
+            if (l == 1) {
+                p = z;
+                d = 1.f;
+            } else if (l > 1) {
+                const float fa = (float)(2 * l - 1) / (float)l, fb = (float)(l - 1) / (float)l;
+                p = fmaf(fa * z, p1, -fb * p2);
+                d = fmaf(fa, fmaf(z, q1, p1), -fb * q2);
+            }
+            if (l > 0) {
+                p2 = p1;
+                p1 = p;
+                q2 = q1;
+                q1 = d;
+            }
+            const float2 kc = *reinterpret_cast<const float2 *>(D + 2 * l);
+            const float k = fmaf(s, kc.y, kc.x);
+            h0 = fmaf(k, p, h0);
+            d0 = fmaf(k, d, d0);
+        }
+    }
+    E = h0;
+    Fz = d0;
+    Fx = Fy = 0.f;
+    float cm = 1.f, sm = 0.f, pmm = 1.f;
+    int q = 0;
+#pragma unroll
+    for (int m = 1; m <= kShL; ++m) {
+        const float cp = cm, sp = sm;  // C_{m-1}, S_{m-1}
+        cm = x * cp - y * sp;
+        sm = fmaf(x, sp, y * cp);
+        pmm *= (float)(2 * m - 1);
+        __syncwarp();
+        float2 h = dup2(0.f), dh = h;              // cosine and sine sums of k Pbar and k Pbar'
+        float2 p2 = h, p1 = dup2(pmm), q2 = h, q1 = h;
+#pragma unroll
+        for (int l = m; l <= kShL; ++l, ++q) {
+            float2 p = p1, d = dup2(0.f);
+            if (l == m + 1) {
+                d = dup2((float)(2 * m + 1) * pmm);
+                p = __fmul2_rn(d, z2);
+            } else if (l > m + 1) {
+                const float fa = (float)(2 * l - 1) / (float)(l - m), fb = (float)(l + m - 1) / (float)(l - m);
+                const float2 nb = dup2(-fb);
+                p = ffma2(__fmul2_rn(dup2(fa), z2), p1, __fmul2_rn(nb, p2));
+                d = ffma2(dup2(fa), ffma2(z2, q1, p1), __fmul2_rn(nb, q2));
+            }
+            if (l > m) {
+                p2 = p1;
+                p1 = p;
+                q2 = q1;
+                q1 = d;
+            }
+            const float4 kq = *reinterpret_cast<const float4 *>(D + kShQuads + 4 * q);
+            const float2 k = ffma2(s2, make_float2(kq.z, kq.w), make_float2(kq.x, kq.y));
+            h = ffma2(k, p, h);
+            if (l > m) dh = ffma2(k, d, dh);
+        }
+        E = fmaf(h.x, cm, fmaf(h.y, sm, E));
+        Fz = fmaf(dh.x, cm, fmaf(dh.y, sm, Fz));
+        Fx = fmaf((float)m, fmaf(h.x, cp, h.y * sp), Fx);
+        Fy = fmaf((float)m, fmaf(h.y, cp, -h.x * sp), Fy);
+    }
+}
+
+// (V, B) of every angular entry: with the coefficients (D_c, D'_c) = 2 N_c^2 (A_c
+// k_l, A'_c k'_l), k_l = sum_a g_a b_al, written over the component sums, V is the
+// contraction's gradient F and B = E - 2 w (sum_a g_a + s^2 sum_a g'_a).
 template <int KRT, int KAT>
 __device__ __forceinline__ void sh_gradients(int nang, const ListWarp &W, const float2 *coef, const float *tab,
                                              int lane) {
@@ -880,15 +963,20 @@ __device__ __forceinline__ void sh_gradients(int nang, const ListWarp &W, const 
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int c = lane + 32 * h;
-        if (c < kShComps) *reinterpret_cast<float2 *>(W.sh + 2 * c) = make_float2(dv[h], dwv[h]);
+        // components 7, 8, 9, ...: cosine and sine of the (l, m) in turn (sh_comp)
+        const int at = c <= kShL ? 2 * c : kShQuads + 4 * ((c - kShL - 1) >> 1) + ((c - kShL - 1) & 1);
+        if (c < kShComps) {
+            W.sh[at] = dv[h];
+            W.sh[at + (c <= kShL ? 1 : 2)] = dwv[h];
+        }
     }
     __syncwarp();
-    for (int base = 0; base < nang; base += 32) {  // (sh_contract synchronises the warp)
+    for (int base = 0; base < nang; base += 32) {  // (sh_contract2 synchronises the warp)
         const int k = base + lane < nang ? base + lane : 0;
         const float4 u = W.a_u[k];
         const float s = W.a_s[k];
         float E, Fx, Fy, Fz;
-        sh_contract(u.x, u.y, u.z, s, W.sh, E, Fx, Fy, Fz);
+        sh_contract2(u.x, u.y, u.z, s, W.sh, E, Fx, Fy, Fz);
         if (base + lane < nang) W.a_g[k] = make_float4(Fx, Fy, Fz, E - 2.0f * u.w * fmaf(s * s, gwsum, gsum));
     }
 }
