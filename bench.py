@@ -71,18 +71,18 @@ def network_flops(widths, n_atoms):
 # DRAM bytes per launch of the dominant kernel (workload, form, kernel), from the ncu
 # captures summarised in profiles/; reported only while the kernel source is the
 # one the counters were taken on (first 16 hex digits of the SHA-256 of
-# potential_kernels.cuh followed by sh_angular.cuh).
-TRAFFIC_SOURCE_SHA256_16 = "9909f6a65756bb2a"
-TRAFFIC_CAPTURE = {("water_331776", "fp32", "k_potential_list"): 145725952,
-                   ("water_331776", "fp32_cell", "k_potential"): 10809600,
-                   ("water_12288", "fp32", "k_potential_list"): 5260288,
-                   ("amorphous_27000", "fp32", "k_potential"): 1104640}
+# potential_kernels.cuh, sh_angular.cuh and list_kernels.cuh, in that order).
+TRAFFIC_SOURCE_SHA256_16 = "88b930eacd75a635"
+TRAFFIC_CAPTURE = {("water_331776", "fp32", "k_potential_list"): 494584576,
+                   ("water_12288", "fp32", "k_potential_list"): 20122624,
+                   ("amorphous_27000", "fp32", "k_potential_list"): 69565696}
+
 
 
 def captured_traffic(workload_name, precision, kernel, skin=0.0):
     import hashlib
     h = hashlib.sha256()
-    for name in ("potential_kernels.cuh", "sh_angular.cuh"):
+    for name in ("potential_kernels.cuh", "sh_angular.cuh", "list_kernels.cuh"):
         with open(os.path.join(ROOT, "paper_2107_11311_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     sha = h.hexdigest()[:16]
@@ -504,8 +504,8 @@ def time_form(args, st, m, v0, precision, dev, stream, flush, world):
                                                       for s in ms}
         torch.cuda.synchronize()
         gpu.check()
-        from paper_2107_11311_gb300.aenet import AENET_PATH_LIST
-        list_form = bool(gpu.md_path_flags() & AENET_PATH_LIST)
+        from paper_2107_11311_gb300.aenet import AENET_PATH_LIST, AENET_PATH_ROWS
+        list_form = bool(gpu.md_path_flags() & (AENET_PATH_LIST | AENET_PATH_ROWS))
         builds = gpu.md_list_builds() - builds0
         step_ms = [a.elapsed_time(b) for a, b in zip(starts, ends)]
         # untimed: the full stage breakdown (every stage bracketed by events)

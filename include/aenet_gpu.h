@@ -237,9 +237,9 @@ int aenet_compute_batch(aenet_ctx *ctx, int n_struct, const int64_t *atom_offset
  * [N * 3], types [N]) and writes (energies [n_struct], forces [N * 3],
  * virials [n_struct * 9]; each output may be NULL). It evaluates the batch on
  * the current contents of pos, and with flags & AENET_BATCH_AUTOTUNE times
- * candidate launches of the potential kernel on them: one CTA per cell in
- * cell order, or one resident (persistent) CTA per SM slot taking cells from
- * a global counter heaviest first, each with staging tiles of 256, 512, 1024
+ * candidate launches on them: staging tiles (of the list build; of the fused
+ * kernel in the tensor-core forms, there also one CTA per cell in cell order or
+ * resident CTAs taking cells heaviest first from a counter) of 256, 512, 1024
  * and 2048 image-atoms. It keeps the fastest and captures the whole evaluation
  * (binning, cell sort, potential, per-structure reductions, forces) in one
  * CUDA graph. Without the flag it uses the persistent form and the current
