@@ -815,35 +815,27 @@ __device__ __forceinline__ void sh_sums(int nang, const ListWarp &W, int lane) {
     __syncwarp();
 }
 
-// S_a = sum_l b_al Q_l - sum w^2, Q_l = sum of N_c^2 A_c^2 over the components of
-// degree l: lanes 2l and 2l + 1 sum Q_l of the two copies, then the lane of
-// order a takes both copies' combination.
+// S_a = sum_c b_{a l(c)} N_c^2 A_c^2 - sum w^2 of both copies into the rows of orders
+// KRT .. KRT + KAT - 1 of dst (without the last term): each lane takes its two
+// components for every order, with the coefficients b N^2 of the table (rounded
+// once, as sh_fingerprint does), and the pairs are reduced across the warp.
+constexpr int kShTabList = kShTab + 7 * kShComps;  // the table with b_{a l(c)} N_c^2 at kShTab + 49 a + c
 template <int KRT, int KAT>
-__device__ __forceinline__ void sh_fingerprints(const float *sh, const float *tab, int lane, float &G0, float &G1) {
-    float Q = 0.f;
-    if (lane < 2 * (kShL + 1)) {
-        const int l = lane >> 1, cp = lane & 1;
-        const float a = sh[2 * l + cp];
-        Q = a * a;
-        for (int m = 1; m <= l; ++m) {
-            const int c = kShL + 1 + (m - 1) * (2 * (kShL + 1) - m) + 2 * (l - m);
-            const float a0 = sh[2 * c + cp], a1 = sh[2 * c + 2 + cp];
-            Q = fmaf(tab[kShTabN + c], fmaf(a0, a0, a1 * a1), Q);
+__device__ __forceinline__ void sh_fingerprints(const ListWarp &W, const float *tab, float *dst, int lane) {
+    float2 acc[KAT];
+#pragma unroll
+    for (int a = 0; a < KAT; ++a) acc[a] = dup2(0.f);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int c = lane + 32 * h;
+        if (c < kShComps) {
+            const float2 A = *reinterpret_cast<const float2 *>(W.sh + 2 * c);
+#pragma unroll
+            for (int a = 0; a < KAT; ++a)
+                acc[a] = ffma2(__fmul2_rn(dup2(tab[kShTab + kShComps * a + c]), A), A, acc[a]);
         }
     }
-    const int al = lane - KRT;
-    const bool on = al >= 0 && al < KAT;
-    const float *b = tab + kShTabB + (on ? al : 0) * (kShL + 1);
-    float g0 = -sh[2 * kShComps], g1 = -sh[2 * kShComps + 1];
-#pragma unroll
-    for (int l = 0; l <= kShL; ++l) {
-        g0 = fmaf(b[l], __shfl_sync(kFull, Q, 2 * l), g0);
-        g1 = fmaf(b[l], __shfl_sync(kFull, Q, 2 * l + 1), g1);
-    }
-    if (on) {
-        G0 = g0;
-        G1 = g1;
-    }
+    reduce_orders<KAT>(acc, W.red, dst, KRT, lane);
 }
 
 // Where the contraction's coefficients of component c lie in the warp's scratch:
@@ -1132,7 +1124,7 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
     constexpr int NW = list_max_warps<KRT, KAT, EXACT>();
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ float s_tw[kMaxSpecies];
-    __shared__ float s_sh[kSh ? kShTab : 1];
+    __shared__ float s_sh[kSh ? kShTabList : 1];
     __shared__ ListSums<NW> s_sum;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     const unsigned lt_mask = (1u << lane) - 1u;
@@ -1181,6 +1173,13 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
     if (lane < 4) s_sum.st[warp][lane] = 0ull;
     if (lane == 0) s_sum.e[warp] = 0.0;
     __syncthreads();
+    if constexpr (kSh) {
+        for (int k = tid; k < 7 * kShComps; k += blockDim.x) {
+            const int al = k / kShComps, c = k - al * kShComps;
+            s_sh[kShTab + k] = s_sh[kShTabB + al * (kShL + 1) + (int)s_sh[kShTabL + c]] * s_sh[kShTabN + c];
+        }
+        __syncthreads();
+    }
     pdl_wait();  // (what is above reads only what the kernels of the evaluation leave alone)
 
     const float inv_rcr = 1.0f / B.rc_rad, inv_rca = 1.0f / B.rc_ang, rc2max = B.rc_max * B.rc_max;
@@ -1359,11 +1358,12 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
                 G1 = lane < KRT + KAT ? two * G.y : 0.f;
             } else {
                 sh_sums(nang, W, lane);
+                sh_fingerprints<KRT, KAT>(W, s_sh, W.coef, lane);
                 __syncwarp();
                 const float2 G = *reinterpret_cast<const float2 *>(W.coef + 2 * lane);
-                G0 = lane < KRT ? G.x : 0.f;
-                G1 = lane < KRT ? G.y : 0.f;
-                sh_fingerprints<KRT, KAT>(W.sh, s_sh, lane, G0, G1);
+                const float2 w2 = *reinterpret_cast<const float2 *>(W.sh + 2 * kShComps);  // the j = k terms
+                G0 = lane < KRT ? G.x : lane < KRT + KAT ? G.x - w2.x : 0.f;
+                G1 = lane < KRT ? G.y : lane < KRT + KAT ? G.y - w2.y : 0.f;
             }
             __syncwarp();  // the row is written again
         }
