@@ -1096,8 +1096,8 @@ __device__ __forceinline__ float list_network(const FusedNet &net, const float *
 template <int NW>
 struct ListSums {
     double e[NW];
+    double vir[NW][6];
     unsigned long long st[NW][4];
-    float vir[NW][6];
 };
 
 // One warp per atom, atoms from a counter. For its atom the warp
@@ -1172,6 +1172,7 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
     }
     if (lane < 4) s_sum.st[warp][lane] = 0ull;
     if (lane == 0) s_sum.e[warp] = 0.0;
+    if (lane < 6) s_sum.vir[warp][lane] = 0.0;
     __syncthreads();
     if constexpr (kSh) {
         for (int k = tid; k < 7 * kShComps; k += blockDim.x) {
@@ -1184,9 +1185,6 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
 
     const float inv_rcr = 1.0f / B.rc_rad, inv_rca = 1.0f / B.rc_ang, rc2max = B.rc_max * B.rc_max;
     const int nb = caps.nb;
-    float vir[6];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) vir[k] = 0.f;
     // The first two rounds of an atom's row, its length and its species are loaded
     // while the atom before is in its last phase.
     struct Ahead {
@@ -1416,10 +1414,9 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
             // every entry: two rounds at a time, their Clenshaw sums packed
             float fix = 0.f, fiy = 0.f, fiz = 0.f;
             const float k2 = 2.0f * inv_rcr;
-            if constexpr (BATCH) {
+            float vir[6];
 #pragma unroll
-                for (int k = 0; k < 6; ++k) vir[k] = 0.f;
-            }
+            for (int k = 0; k < 6; ++k) vir[k] = 0.f;
             for (int r = 0; r < nrounds; r += 2) {
                 int ka, kb;
                 const bool va = rounds.at(r, ka), vb = rounds.at(r + 1, kb);  // (none past the last round)
@@ -1473,30 +1470,31 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
                 entry(va, ea, ja, S.x, dS.x, r, ka);
                 entry(vb, eb, jb, S.y, dS.y, r + 1, kb);
             }
-            // the atom's own force; in a batch its virial too
+            // the atom's own force and its virial. FP32 sums end with the atom: its virial is
+            // added up in FP64, per warp or (a batch) per structure, so that the rounding
+            // of the total does not grow with the atoms a warp takes.
             __syncwarp();
-            if constexpr (BATCH) {
-                const float2 sums[8] = {make_float2(fix, fiy), make_float2(fiz, 0.f), make_float2(vir[0], vir[1]),
-                                        make_float2(vir[2], vir[3]), make_float2(vir[4], vir[5]),
-                                        dup2(0.f), dup2(0.f), dup2(0.f)};
-                const float2 t = reduce8(sums, W.red, lane);
-                const int o = reduce8_order(lane);
-                float *f = reinterpret_cast<float *>(F4 + a);
-                if ((lane & 12) == 0) {
-                    if (o == 0) {
-                        atomicAdd(f, t.x);
-                        atomicAdd(f + 1, t.y);
-                    } else if (o == 1) {
-                        atomicAdd(f + 2, t.x);
-                    } else if (o < 5) {
+            const float2 sums[8] = {make_float2(fix, fiy), make_float2(fiz, 0.f), make_float2(vir[0], vir[1]),
+                                    make_float2(vir[2], vir[3]), make_float2(vir[4], vir[5]),
+                                    dup2(0.f), dup2(0.f), dup2(0.f)};
+            const float2 t = reduce8(sums, W.red, lane);
+            const int o = reduce8_order(lane);
+            float *f = reinterpret_cast<float *>(F4 + a);
+            if ((lane & 12) == 0) {
+                if (o == 0) {
+                    atomicAdd(f, t.x);
+                    atomicAdd(f + 1, t.y);
+                } else if (o == 1) {
+                    atomicAdd(f + 2, t.x);
+                } else if (o < 5) {
+                    if constexpr (BATCH) {
                         *reinterpret_cast<float2 *>(vir_atom + (size_t)a * 6 + 2 * (o - 2)) = t;
+                    } else {
+                        double *v = s_sum.vir[warp] + 2 * (o - 2);
+                        v[0] += (double)t.x;
+                        v[1] += (double)t.y;
                     }
                 }
-            } else {
-                fix = warp_sum(fix);
-                fiy = warp_sum(fiy);
-                fiz = warp_sum(fiz);
-                if (lane == 0) atomicAdd(&F4[a], make_float4(fix, fiy, fiz, 0.f));
             }
         }
         __syncwarp();
@@ -1505,13 +1503,6 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
 
     wait_params();  // (a warp without atoms)
     // ---- the CTA's partial sums
-    if constexpr (MODE != kDescriptor && !BATCH) {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            const float v = warp_sum(vir[k]);
-            if (lane == 0) s_sum.vir[warp][k] = v;
-        }
-    }
     __syncthreads();  // every warp has left the loop
     if (tid == 0) release_work_counter(work);
     if (MODE != kForces && tid < 3) {
@@ -1523,9 +1514,9 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
         if (tid < 9) {  // the virial of an atom is symmetric: six sums
             const int ra = tid / 3, rb = tid - 3 * ra, lo = min(ra, rb), hi = max(ra, rb);
             const int k = lo == 0 ? hi : lo == 1 ? 2 + hi : 5;
-            float t = 0.f;
+            double t = 0.0;
             for (int w = 0; w < nw; ++w) t += s_sum.vir[w][k];
-            vir_part[(size_t)blockIdx.x * 9 + tid] = (double)t;
+            vir_part[(size_t)blockIdx.x * 9 + tid] = t;
         }
     }
     if constexpr (MODE == kFused) {
