@@ -363,9 +363,11 @@ bool pipe_supported(const Context &c, const Grid &g);
 bool fused_supported(const Context &c);
 cudaError_t launch_fused_potential(Context &c, const Grid &g, int n);
 // Fused kernel with the networks on the tensor cores (BF16 forms; two hidden
-// layers <= 32 wide; the water (16, 8) and solid (20, 6) bases; c.eval_n at most
-// kTcFusedAtoms or kTcFusedAtomsSolid), unless the context asked for the three-kernel path
-// (AENET_OPT_FUSED_NETWORK 0).
+// layers <= 32 wide; the water (16, 8) and solid (20, 6) bases), unless the context
+// asked for the three-kernel path (AENET_OPT_FUSED_NETWORK 0): the form, and
+// whether the evaluation of c.eval_n atoms takes it (at most kTcFusedAtoms or
+// kTcFusedAtomsSolid; more take the three kernels).
+bool tc_fused_form(const Context &c);
 bool tc_fused_supported(const Context &c);
 cudaError_t launch_fused_tc(Context &c, const Grid &g, int n);
 // Either fused form: descriptor, networks and forces in one kernel.

@@ -177,6 +177,7 @@ __device__ __forceinline__ void store_row32(unsigned char *smem, int a_off, int 
 
 struct AnnTcArgs {
     int n, D, n_species, H1, H2, rec_len, n_tiles;
+    bool bias_first;             // layers 1 and 2: accumulate onto the biases, or add them in FP32 afterwards
     const float *G;              // [n, D] sorted order
     const unsigned char *wtc;    // [species][kWtcBytes] packed weights (k_pack_tcgen05)
     const float *shift, *scale;
@@ -324,9 +325,11 @@ __global__ void __launch_bounds__(kUThreads, 3) k_ann_tcgen05(AnnTcArgs a) {
             cur_t = t;
         }
         // ---- the biases of layers 1 and 2 into their accumulators (columns 0..63; the
-        // previous tile's reads of them are over): the sums then start from the bias,
-        // as in the fused kernel, and the tensor cores' rounding of them is the same
-        {
+        // previous tile's reads of them are over): where this kernel stands in for the
+        // fused one (bias_first) the sums start from the bias as there, and the tensor
+        // cores' rounding of them is the same. Otherwise the products are summed alone
+        // and the bias is added in FP32, to nearest.
+        if (a.bias_first) {
             const float *gb = reinterpret_cast<const float *>(a.wtc + (size_t)t * kWtcBytes + (kBias - kB1));
             tmem_fill32(lane_addr + 0, gb);
             tmem_fill32(lane_addr + 32, gb + kUHid);
@@ -386,22 +389,22 @@ __global__ void __launch_bounds__(kUThreads, 3) k_ann_tcgen05(AnnTcArgs a) {
         float x1[kUHid];
         float v[32];
         // ---- layer 1: Z1 = b1 + g W1^T (TMEM columns 0..31)
-        run(0, kA0, 64, kB1, 32, 64, 32, true);
+        run(0, kA0, 64, kB1, 32, 64, 32, a.bias_first);
         tmem_ld32(lane_addr + 0, v);
 #pragma unroll
-        for (int j = 0; j < kUHid; ++j) x1[j] = j < H1 ? tanh_exp(v[j]) : 0.f;
+        for (int j = 0; j < kUHid; ++j) x1[j] = j < H1 ? tanh_exp(v[j] + (a.bias_first ? 0.f : s_bias[j])) : 0.f;
         store_row32<X3>(smem, kA1, tid, x1);
         fence_async_smem();
         tc_fence_before();
         __syncthreads();
 
         // ---- layer 2: Z2 = b2 + X1 W2^T (columns 32..63); output layer and delta2 in FP32
-        run(32, kA1, 32, kB2, 32, 32, 32, true);
+        run(32, kA1, 32, kB2, 32, 32, 32, a.bias_first);
         tmem_ld32(lane_addr + 32, v);
         float e = s_bias[3 * kUHid];
 #pragma unroll
         for (int j = 0; j < kUHid; ++j) {
-            const float x2 = j < H2 ? tanh_exp(v[j]) : 0.f;
+            const float x2 = j < H2 ? tanh_exp(v[j] + (a.bias_first ? 0.f : s_bias[kUHid + j])) : 0.f;
             const float w = s_bias[2 * kUHid + j];
             e = fmaf(w, x2, e);
             v[j] = (1.0f - x2 * x2) * w;  // delta2
@@ -498,6 +501,7 @@ cudaError_t launch_ann_tcgen05(Context &c, int n) {
     a.H2 = c.net.widths[2];
     a.rec_len = activation_record_len(c.net);
     a.n_tiles = tcgen05_tiles(c, n);
+    a.bias_first = tc_fused_form(c);
     a.G = c.d_G;
     a.wtc = c.d_wtc;
     a.shift = c.d_shift;

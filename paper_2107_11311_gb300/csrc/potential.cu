@@ -46,10 +46,13 @@ bool fused_supported(const Context &c) {
     return true;
 }
 
-bool tc_fused_supported(const Context &c) {
+bool tc_fused_form(const Context &c) {
     if (c.precision == AENET_FP32 || !c.fuse_network || !bf16_supported(c.net) || !c.d_wbf) return false;
-    if (c.eval_n > (c.basis.Ka == 7 ? kTcFusedAtomsSolid : kTcFusedAtoms)) return false;
     return (c.basis.Kr == 17 && c.basis.Ka == 9) || (c.basis.Kr == 21 && c.basis.Ka == 7);
+}
+
+bool tc_fused_supported(const Context &c) {
+    return tc_fused_form(c) && c.eval_n <= (c.basis.Ka == 7 ? kTcFusedAtomsSolid : kTcFusedAtoms);
 }
 
 // The pipelined form (k_potential_pipe): FP32 fused evaluation of one

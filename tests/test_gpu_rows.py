@@ -38,3 +38,31 @@ def test_virial_is_summed_in_fp64(gpu_mod, precision):
     total, one = g.compute(pos, types, box), g.compute(pos[:2], types[:2], box)
     assert np.abs(one["virial"]).min() > 1e-4
     assert np.array_equal(total["virial"], k ** 3 * one["virial"])
+
+
+def _one_path_params(m, w2, b2):
+    """Parameters whose only path is x1[0] = tanh(20) = 1, z2[0] = w2 x1[0] + b2, E = 2^20 tanh(z2[0])."""
+    D, H1, H2, _ = m.widths
+    W1, b1, W2, B2, w3 = np.zeros((H1, D)), np.zeros(H1), np.zeros((H2, H1)), np.zeros(H2), np.zeros(H2)
+    b1[0], W2[0, 0], B2[0], w3[0] = 20.0, w2, b2, 2.0 ** 20
+    p = np.concatenate([W1.ravel(), b1, W2.ravel(), B2, w3, [0.0]])
+    return np.tile(p, (m.n_species, 1))
+
+
+@pytest.mark.parametrize("precision", ["bf16", "bf16x3"])
+@pytest.mark.parametrize("orders,fused", [(None, False), ((7, 5), True)])
+def test_three_kernel_bias_is_added_in_fp32(gpu_mod, precision, orders, fused):
+    """The three-kernel path, by the option or by the basis: 0.5 plus 3/4 of its last
+    place rounds up. Summed by the tensor cores, which cut off, it would stay 0.5."""
+    st = inputs.water(32, None, 3)
+    m = inputs.make_model("water", hidden=(15, 15), orders=orders)
+    g = gpu_mod.AenetGPU(m, precision)
+    g.fuse_network(fused)
+
+    def e_atom(w2, b2):
+        g.set_params(_one_path_params(m, w2, b2))
+        return g.compute(st.pos, st.types, st.box)["e_atom"]
+
+    up = e_atom(0.0, 0.5 + 2.0 ** -24)
+    assert not np.array_equal(up, e_atom(0.0, 0.5))
+    assert np.array_equal(e_atom(0.75 * 2.0 ** -24, 0.5), up)
