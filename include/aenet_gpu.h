@@ -454,7 +454,8 @@ int aenet_grad_weights(aenet_ctx *ctx, double *dEdW);
 /*
  * Replace the network parameters ([n_species * n_params] double, same layout as
  * at set-up; Sec. II.C trains exactly these). HOST params: converted on the host,
- * copied after a synchronisation of the context's stream. DEVICE params: the
+ * copied after a synchronisation of the context's stream, and in place on return
+ * (also for a stream given with aenet_set_stream next). DEVICE params: the
  * conversion to FP32 and, in the BF16 forms, the packing of the tensor-core
  * operands run as kernels on the context's stream, after the work already
  * enqueued there and without any host round trip; the caller keeps params

@@ -572,6 +572,8 @@ extern "C" int aenet_setup(aenet_ctx **out, const aenet_model_desc *m, int preci
             (e = cudaMalloc(&c.d_dEdW, sizeof(double) * NP)) != cudaSuccess)
             return setup_fail(e, "gradient tables");
     }
+    // (the packing above runs on the stream; the context may be given another one next)
+    if ((e = cudaStreamSynchronize(c.stream)) != cudaSuccess) return setup_fail(e, "cudaStreamSynchronize");
     *out = h;
     return AENET_OK;
 }
@@ -1663,7 +1665,8 @@ extern "C" int aenet_set_params(aenet_ctx *h, const double *params) {
     Context &c = h->c;
     cudaGetLastError();
     const size_t NP = (size_t)c.basis.n_species * c.net.n_params;
-    if (is_device_ptr(params)) {
+    const bool on_device = is_device_ptr(params);
+    if (on_device) {
         // on the context's stream, after the work already enqueued: no host round trip
         k_params_to_f32<<<(int)std::min<size_t>((NP + 255) / 256, 1024), 256, 0, c.stream>>>(NP, params, c.d_params);
         CK(cudaGetLastError(), "parameter conversion");
@@ -1675,6 +1678,9 @@ extern "C" int aenet_set_params(aenet_ctx *h, const double *params) {
     }
     if (c.precision != AENET_FP32) CK(prepare_bf16_weights(c), "BF16 weights");
     if (c.d_pnet) CK(pack_list_net(c), "network parameters");
+    // host parameters are in place on return, the packed forms too: whatever stream
+    // the context is given next finds them
+    if (!on_device) CK(cudaStreamSynchronize(c.stream), "cudaStreamSynchronize");
     c.act_valid = false;
     return AENET_OK;
 }

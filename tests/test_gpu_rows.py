@@ -66,3 +66,18 @@ def test_three_kernel_bias_is_added_in_fp32(gpu_mod, precision, orders, fused):
     up = e_atom(0.0, 0.5 + 2.0 ** -24)
     assert not np.array_equal(up, e_atom(0.0, 0.5))
     assert np.array_equal(e_atom(0.75 * 2.0 ** -24, 0.5), up)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "bf16x3"])
+def test_host_parameters_are_in_place_on_return(gpu_mod, precision):
+    """set_params from a host array, then another stream: nothing may be left running
+    on the stream before."""
+    m = inputs.make_model("water", hidden=(32, 32))
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    with torch.cuda.stream(a):
+        g = gpu_mod.AenetGPU(m, precision)
+    assert a.query()
+    for k in range(100):
+        g.set_stream(a.cuda_stream if k % 2 else b.cuda_stream)
+        g.set_params(m.params)
+        assert (a if k % 2 else b).query()
