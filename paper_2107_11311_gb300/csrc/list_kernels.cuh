@@ -1147,7 +1147,9 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
 #pragma unroll
     for (int t = 0; t < kMaxSpecies; ++t)
         if (tid == t) s_tw[t] = B.type_weight[t];
-    if constexpr (kSh) load_sh_table(B.sh_b, s_sh, tid);
+    if constexpr (kSh) {  // (the table's loader takes thread indices up to 64, a CTA may be one or two warps)
+        for (int t = tid; t <= 64; t += blockDim.x) load_sh_table(B.sh_b, s_sh, t);
+    }
     // the parameters arrive while the first atoms' descriptors are computed
     if constexpr (MODE == kFused) {
         const unsigned dst = (unsigned)__cvta_generic_to_shared(s_par);

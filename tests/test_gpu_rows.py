@@ -81,3 +81,38 @@ def test_host_parameters_are_in_place_on_return(gpu_mod, precision):
         g.set_stream(a.cuda_stream if k % 2 else b.cuda_stream)
         g.set_params(m.params)
         assert (a if k % 2 else b).query()
+
+
+@pytest.mark.parametrize("n", [60, 120, 162])
+def test_lists_that_leave_room_for_few_warps(gpu_mod, n):
+    """The solid's basis in a 6 A box: lists so long that a CTA of the list kernel holds
+    five, two and one of them (descriptors: six, three, two); its tables are then filled
+    by as few warps.
+
+    Coefficients: sums of N products in FP32, N / 32 + 8 roundings deep at most, and
+    |b| of T_a's Legendre series sums up to less than 3, twice (A^2) that in the angular
+    ones: 6 (N / 32 + 8) units of the a = 0 coefficient. Forces: from coefficients good to
+    some 300 units, and sums that cancel to the root of their N terms: 1e-3."""
+    rng = np.random.default_rng(n)
+    box = np.full(3, 6.0)
+    pts = []
+    while len(pts) < n:
+        p = rng.uniform(0, 6.0, 3)
+        if all((((p - q + 3.0) % 6.0 - 3.0) ** 2).sum() > 0.3 ** 2 for q in pts):
+            pts.append(p)
+    pos, types = np.array(pts), rng.integers(0, 4, n).astype(np.int32)
+    m = inputs.make_model("amorphous")
+    G = O.compute(m, pos, types, box, want_G=True)["G"]
+    m.in_shift[:], m.in_scale[:] = G.mean(0), 1.0 / np.maximum(G.std(0), 1e-2 * np.abs(G).max(0))
+    ref = O.compute(m, pos, types, box)
+    g = gpu_mod.AenetGPU(m, "fp32")
+    Kr, Ka, smax = m.order_rad + 1, m.order_ang + 1, float(np.abs(m.type_weights).max())
+    unit = np.concatenate([np.full((n, Kr), 1.0) * G[:, [0]], np.full((n, Ka), 1.0) * G[:, [Kr]]], 1)
+    unit = np.concatenate([unit, np.concatenate([smax * unit[:, :Kr], smax ** 2 * unit[:, Kr:]], 1)], 1)
+    N = n / 216.0 * 4.18879 * 8.0 ** 3
+    assert (np.abs(g.descriptors(pos, types, box) - G) <= 6 * (N / 32 + 8) * 2.0 ** -24 * unit + 1e-6).all()
+    out = g.compute(pos, types, box)
+    rms = np.sqrt((ref["forces"] ** 2).mean())
+    assert rms > 1e-4
+    assert np.sqrt(((out["forces"] - ref["forces"]) ** 2).mean()) <= 1e-3 * rms
+    assert np.abs(out["e_atom"] - ref["e_atom"]).max() <= 1e-3 * max(1.0, np.abs(ref["e_atom"]).max())
