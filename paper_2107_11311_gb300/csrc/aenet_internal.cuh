@@ -429,10 +429,10 @@ cudaError_t launch_potential_list(Context &c, const Grid &g, int n);
 int potential_list_max_ctas(const Context &c);
 // Evaluation over lists built for it, for the sorted atoms [a_lo, a_hi) (slices
 // of list_slice(c, n) atoms): the list build (direct rows) and the list kernel.
-// The first build also clears the forces and statistics unless c.md_prezeroed;
+// The first build also clears the forces and statistics when clear;
 // the kernel appends its partial rows after *parts and sets c.last_*.
 int list_slice(const Context &c, int n);
-cudaError_t launch_rows_build(Context &c, const Grid &g, int n, int a_lo, int a_hi);
+cudaError_t launch_rows_build(Context &c, const Grid &g, int n, int a_lo, int a_hi, bool clear);
 // What the list kernel evaluates: everything, the G rows (c.d_G) only, or forces
 // and virial from given dE/dG rows (c.d_dEdG).
 enum class RowsMode { fused, descriptor, forces };

@@ -288,10 +288,13 @@ int enqueue_rows(Context &c, const Grid &g, int n, RowsMode mode) {
     int rc = ensure_rows(c, n);
     if (rc) return rc;
     const int slice = list_slice(c, n);
+    // (the forces of the split path add to what its descriptor pass has cleared and, in the statistics, counted)
+    const bool clear = !c.md_prezeroed && mode != RowsMode::forces;
     int parts = 0;
     for (int a0 = 0; a0 < std::max(n, 1); a0 += slice) {
         const int a1 = std::min(n, a0 + slice);
-        if (mode != RowsMode::forces || slice < n) CK(launch_rows_build(c, g, n, a0, a1), "neighbour list");
+        if (mode != RowsMode::forces || slice < n)
+            CK(launch_rows_build(c, g, n, a0, a1, clear), "neighbour list");
         if (a0 == 0 && mode == RowsMode::fused) {
             CK(mark(c, 2), "event");
             CK(mark(c, 3), "event");

@@ -156,13 +156,13 @@ int potential_list_max_ctas(const Context &c) { return std::max(1, c.n_sm); }
 
 cudaError_t pack_list_net(Context &c) { return AENET_BY_BASIS(c, pack_net, c); }
 
-cudaError_t launch_rows_build(Context &c, const Grid &g, int n, int a_lo, int a_hi) {
+cudaError_t launch_rows_build(Context &c, const Grid &g, int n, int a_lo, int a_hi, bool clear) {
     // with one slice the build clears what the list kernel accumulates into; with
     // more, an earlier slice's forces already lie on a later slice's atoms
     const bool one = a_lo == 0 && a_hi >= n;
     cudaError_t e;
-    if (!c.md_prezeroed && !one && a_lo == 0 && (e = clear_sums(c, n)) != cudaSuccess) return e;
-    return launch_build(c, g, n, a_lo, a_hi, false, !c.md_prezeroed && one);
+    if (clear && !one && a_lo == 0 && (e = clear_sums(c, n)) != cudaSuccess) return e;
+    return launch_build(c, g, n, a_lo, a_hi, false, clear && one);
 }
 
 cudaError_t launch_rows_potential(Context &c, const Grid &g, RowsMode mode, int a_lo, int a_hi, int *parts) {

@@ -116,3 +116,39 @@ def test_lists_that_leave_room_for_few_warps(gpu_mod, n):
     assert rms > 1e-4
     assert np.sqrt(((out["forces"] - ref["forces"]) ** 2).mean()) <= 1e-3 * rms
     assert np.abs(out["e_atom"] - ref["e_atom"]).max() <= 1e-3 * max(1.0, np.abs(ref["e_atom"]).max())
+
+
+@pytest.mark.parametrize("precision,hidden", [("fp32", (15, 15)), ("bf16x3", (15, 15)), ("fp32", (48, 48))])
+def test_slices_of_rows_give_what_one_slice_gives(gpu_mod, precision, hidden):
+    """24,000 atoms after a structure so dense (two atoms in 0.73 A^3) that the lists it
+    sizes fill a slice of rows with 20,560 atoms, against a context that never saw it:
+    the fused, the three-kernel and the wide FP32 path, descriptors and a batch. Sums in
+    another order, in FP32: a few units of 2^-24 of an atom's terms, 5e-6 of the RMS;
+    through the split-BF16 network, whose products drop 2^-16 of a factor, 1e-4."""
+    m = inputs.make_model("water", hidden=hidden)
+    st, half = inputs.water(8000, None, 5), inputs.water(4000, None, 6)
+    dense = np.array([[0.1, 0.2, 0.3], [0.55, 0.65, 0.75]]), np.array([0, 1], np.int32), np.full(3, 0.9)
+    off = np.array([0, 12000, 24000])
+    both = np.concatenate([half.pos, half.pos + 0.3]), np.tile(half.types, 2), np.stack([half.box] * 2)
+
+    def results(after):
+        g = gpu_mod.AenetGPU(m, precision)
+        if after:
+            g.fuse_network(False)  # (few atoms otherwise take the fused kernel, which has no room for such lists)
+            g.compute(*dense)
+            g.fuse_network(True)
+        r = dict(g.compute(st.pos, st.types, st.box), stats=np.array(g.neighbor_stats()))
+        r["G"] = g.descriptors(st.pos, st.types, st.box)
+        r["G_stats"] = np.array(g.neighbor_stats())
+        b = g.compute_batch(off, both[0], both[1], both[2])
+        r.update({"b_" + k: v for k, v in b.items()}, b_stats=np.array(g.neighbor_stats()))
+        return r
+
+    one, many = results(False), results(True)
+    tol = 5e-6 if precision == "fp32" else 1e-4
+    for k, x in one.items():
+        if k.endswith("stats"):
+            assert x.min() > 0 and np.array_equal(x, many[k]), k
+        else:
+            x, y = np.asarray(x, dtype=np.float64), np.asarray(many[k], dtype=np.float64)
+            assert np.sqrt(((x - y) ** 2).mean()) <= (5e-6 if k == "G" else tol) * np.sqrt((x ** 2).mean()), k
