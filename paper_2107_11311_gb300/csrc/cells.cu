@@ -61,15 +61,14 @@ __global__ void k_bin_count_batch(int n, int n_struct, int n_species, const doub
 }
 
 // Exclusive scan of the cell counts by one CTA (scan_cells_block).
-__global__ void k_scan_cells(int ncell, int *__restrict__ count, int *__restrict__ start) {
+__global__ void k_scan_cells(int ncell, int *count, int *__restrict__ start) {
     pdl_wait();
     scan_cells_block(ncell, count, start);
 }
 
 // Atom i to its sorted position s = cell_start[cell] + rank; slot[i] then holds
 // s itself (the MD kernels read the forces of atom i at F4[slot[i]]).
-__global__ void k_scatter(int n, const float4 *__restrict__ tmp4, const int *__restrict__ cell_of,
-                          int *__restrict__ slot, const int *__restrict__ cell_start,
+__global__ void k_scatter(int n, const float4 *tmp4, const int *cell_of, int *slot, const int *cell_start,
                           float4 *__restrict__ pos4, int *__restrict__ perm) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     pdl_wait();

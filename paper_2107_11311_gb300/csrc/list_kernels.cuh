@@ -70,9 +70,9 @@ __host__ __device__ inline BuildLayout make_build_layout(int n_off, int tile) {
 template <bool BATCH, bool CODES>
 __global__ void __launch_bounds__(kBuildThreads, 10)
     k_list_build(Grid g_one, const StructInfo *__restrict__ sinfo, int n_struct, float rc, int tile, int parts,
-                 int a_lo, int a_hi, const float4 *__restrict__ pos4, const int *__restrict__ cell_start,
-                 float4 *__restrict__ rows, int *__restrict__ codes, int cap, int jbits, int *__restrict__ count,
-                 float4 *__restrict__ F4, unsigned long long *__restrict__ stats, unsigned *__restrict__ err) {
+                 int a_lo, int a_hi, const float4 *pos4, const int *cell_start, float4 *__restrict__ rows,
+                 int *__restrict__ codes, int cap, int jbits, int *__restrict__ count, float4 *__restrict__ F4,
+                 unsigned long long *__restrict__ stats, unsigned *__restrict__ err) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_kept, s_next;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1113,10 +1113,9 @@ struct ListSums {
 // structure afterwards) instead of the CTA's partial row.
 template <int KRT, int KAT, bool EXACT, int MODE, int HB, bool CODES, bool BATCH>
 __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
-    k_potential_list(Basis B, FusedNet net, Grid g, Caps caps, int a_lo, int a_hi, const float4 *__restrict__ pos4,
-                     const float4 *__restrict__ rows, const int *__restrict__ codes, const int *__restrict__ count,
-                     const float *__restrict__ pnet, float4 *__restrict__ F4, float *__restrict__ eatom,
-                     float *__restrict__ G_out, const float *__restrict__ dEdG_in, double *__restrict__ e_part,
+    k_potential_list(Basis B, FusedNet net, Grid g, Caps caps, int a_lo, int a_hi, const float4 *pos4,
+                     const float4 *rows, const int *codes, const int *count, const float *__restrict__ pnet, float4 *__restrict__ F4, float *__restrict__ eatom,
+                     float *__restrict__ G_out, const float *dEdG_in, double *__restrict__ e_part,
                      double *__restrict__ vir_part, float *__restrict__ vir_atom,
                      unsigned long long *__restrict__ stats, unsigned *__restrict__ err,
                      unsigned *__restrict__ work) {
@@ -1183,7 +1182,8 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
         }
         __syncthreads();
     }
-    pdl_wait();  // (what is above reads only what the kernels of the evaluation leave alone)
+    // (what is above reads only what the kernels of the evaluation leave alone)
+    pdl_wait();
 
     const float inv_rcr = 1.0f / B.rc_rad, inv_rca = 1.0f / B.rc_ang, rc2max = B.rc_max * B.rc_max;
     const int nb = caps.nb;
@@ -1200,8 +1200,8 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
         nx.type = __float_as_int(pos4[i].w);
         if constexpr (CODES) {
             const int *row = codes + (size_t)i * caps.vl_cap;
-            nx.c0 = __ldg(row + lane);  // (rows hold at least 64 entries; those past the count are not used)
-            nx.c1 = __ldg(row + 32 + lane);
+            nx.c0 = __ldcg(row + lane);  // (rows hold at least 64 entries; those past the count are not used)
+            nx.c1 = __ldcg(row + 32 + lane);
         } else {
             const float4 *row = rows + (size_t)(i - a_lo) * caps.vl_cap;
             nx.e0 = __ldcs(row + lane);
@@ -1218,6 +1218,13 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
         // ---- 1. the list, and the radial sums of the descriptor as it is read (in
         // row order: sorted by distance the FP32 sums would be biased)
         const int cnt = nx.cnt, type = nx.type;
+        float c0, c1;  // dE/dG of this lane's order and its weighted copy
+        if constexpr (MODE == kForces) {
+            const int D = 2 * (Kr + Ka);
+            const int k0 = lane_col<KRT, KAT>(lane, 0, Kr, Ka), k1 = lane_col<KRT, KAT>(lane, 1, Kr, Ka);
+            c0 = k0 >= 0 ? dEdG_in[(size_t)a * D + k0] : 0.f;
+            c1 = k1 >= 0 ? dEdG_in[(size_t)a * D + k1] : 0.f;
+        }
         int nang = 0, nrest = 0;
         bool over = false;
         constexpr bool kDesc = MODE != kForces;
@@ -1282,7 +1289,7 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
             const int jmask = (1 << caps.vl_jbits) - 1;
             const float4 ui = pos4[a];
             const int *row = codes + (size_t)a * caps.vl_cap;
-            auto code = [&](int base) { return base + lane < cnt ? __ldg(row + base + lane) : -1; };  // (entries >= 0)
+            auto code = [&](int base) { return base + lane < cnt ? __ldcg(row + base + lane) : -1; };  // (entries >= 0)
             auto gather = [&](int e) { return e >= 0 ? pos4[e & jmask] : make_float4(0.f, 0.f, 0.f, 0.f); };
             int e0 = lane < cnt ? nx.c0 : -1, e1 = 32 + lane < cnt ? nx.c1 : -1;
             float4 p0 = gather(e0);
@@ -1376,7 +1383,6 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
             fetch(next);
         } else {
             // ---- 3. the network
-            float c0, c1;
             if constexpr (MODE == kFused) {
                 wait_params();
                 const float E = list_network<KRT, KAT, HB>(net, s_par + type * net.stride, W.coef, lane, G0, G1,
@@ -1387,10 +1393,6 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
                     eatom[a] = E;
                 }
             } else {  // dE/dG given
-                const int D = 2 * (Kr + Ka);
-                const int k0 = lane_col<KRT, KAT>(lane, 0, Kr, Ka), k1 = lane_col<KRT, KAT>(lane, 1, Kr, Ka);
-                c0 = k0 >= 0 ? dEdG_in[(size_t)a * D + k0] : 0.f;
-                c1 = k1 >= 0 ? dEdG_in[(size_t)a * D + k1] : 0.f;
                 if constexpr (kSh) sh_sums(nang, W, lane);
             }
             if (!kSh && lane >= KRT) {  // the ordered-pair sum's factor

@@ -80,9 +80,8 @@ struct FinalizeOut {
 // n_e partials) and 1..9 (virial, n_v x 9 partials), one warp per quantity; the
 // others: forces and atomic energies in input order.
 __global__ void __launch_bounds__(kRedThreads)
-    k_finalize(int n, const int *__restrict__ perm, const float4 *__restrict__ F4, const float *__restrict__ eatom,
-               int n_e, const double *__restrict__ e_part, int n_v, const double *__restrict__ vir_part,
-               double *__restrict__ result, const unsigned *__restrict__ err, FinalizeOut o) {
+    k_finalize(int n, const int *perm, const float4 *F4, const float *eatom, int n_e, const double *e_part, int n_v,
+               const double *vir_part, double *__restrict__ result, const unsigned *err, FinalizeOut o) {
     pdl_wait();
     if (blockIdx.x < kReduceCtas) {
         const int lane = threadIdx.x & 31;
@@ -274,8 +273,8 @@ __device__ inline bool md_close(const MdSums &m, double ke) {
 // v += dt/2 F/m c with F of the current evaluation, and the closing reduction; the
 // last CTA also clears the Verlet rebuild flag and computes the thermostat's factor.
 __global__ void __launch_bounds__(kMdThreads)
-    k_md_kick_finish(int n, KickParams kp, double *__restrict__ vel, const int32_t *__restrict__ types,
-                     const float4 *__restrict__ F4, const int *__restrict__ slot, MdSums sums,
+    k_md_kick_finish(int n, KickParams kp, double *vel, const int32_t *__restrict__ types, const float4 *F4,
+                     const int *slot, MdSums sums,
                      unsigned *__restrict__ vl_flag, unsigned long long *__restrict__ vl_builds, Thermostat th) {
     const int tid = threadIdx.x;
     const int i = blockIdx.x * blockDim.x + tid;
@@ -314,11 +313,10 @@ __global__ void __launch_bounds__(kMdThreads)
 // atoms, whose step is a chain of launch latencies). The last CTA also scans the
 // cell counts when fold. NVE only: a thermostat's factor needs the reduction first.
 __global__ void __launch_bounds__(kMdThreads)
-    k_md_turn(int n, int n_species, KickParams kp, double dt, double *__restrict__ pos, double *__restrict__ vel,
-              const int32_t *__restrict__ types, float4 *__restrict__ F4, Grid g, float4 *__restrict__ tmp4,
-              int *__restrict__ cell_of, int *__restrict__ slot, int *__restrict__ cell_count,
-              int *__restrict__ cell_start, bool fold, unsigned long long *__restrict__ stats,
-              unsigned *__restrict__ err, MdSums sums) {
+    k_md_turn(int n, int n_species, KickParams kp, double dt, double *pos, double *vel,
+              const int32_t *__restrict__ types, float4 *F4, Grid g, float4 *__restrict__ tmp4,
+              int *__restrict__ cell_of, int *slot, int *cell_count, int *__restrict__ cell_start, bool fold,
+              unsigned long long *__restrict__ stats, unsigned *__restrict__ err, MdSums sums) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     pdl_wait();
     if (i < 4) stats[i] = 0ull;

@@ -9,6 +9,16 @@
 // that another kernel of the chain reads or writes (launched without the
 // attribute the call does nothing), and lets its own successor start after that:
 // whatever came before its predecessor is then complete for the successor too.
+//
+// The kernel runs while its predecessor still writes, so what it reads of it is not
+// read-only memory. Loads through a __restrict__ parameter are not bound by the wait's
+// memory clobber (nothing else may alias them), and those through a `const
+// __restrict__` one may become non-coherent loads besides: either could be moved above
+// the wait. Pointers to memory that an earlier kernel of the chain writes are therefore
+// declared without __restrict__; plain loads through them, and the volatile load
+// intrinsics, stay below the wait. Never __ldg: it reads through the non-coherent path.
+// What no kernel of an evaluation writes (network parameters, batch layouts, species)
+// needs none of this.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -144,9 +144,8 @@ __global__ void k_bin_count(int n, int n_species, const double *__restrict__ pos
                             const int32_t *__restrict__ types, Grid g, float4 *__restrict__ tmp4,
                             int *__restrict__ cell_of, int *__restrict__ slot, int *__restrict__ cell_count,
                             unsigned *__restrict__ err);
-__global__ void k_scan_cells(int ncell, int *__restrict__ count, int *__restrict__ start);
-__global__ void k_scatter(int n, const float4 *__restrict__ tmp4, const int *__restrict__ cell_of,
-                          int *__restrict__ slot, const int *__restrict__ cell_start,
+__global__ void k_scan_cells(int ncell, int *count, int *__restrict__ start);
+__global__ void k_scatter(int n, const float4 *tmp4, const int *cell_of, int *slot, const int *cell_start,
                           float4 *__restrict__ pos4, int *__restrict__ perm);
 
 namespace {
