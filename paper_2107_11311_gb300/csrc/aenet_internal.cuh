@@ -59,6 +59,12 @@ struct StructInfo {
     int item0, parts;
 };
 
+// Energy and virial partial rows of one evaluation (read by the MD reductions).
+struct Partials {
+    const double *epart = nullptr, *vpart = nullptr;
+    int eparts = 0, vparts = 0;
+};
+
 // Capacities of the per-warp neighbour lists of the potential kernel, and the
 // shape of the Verlet list (MD with a skin).
 struct Caps {
@@ -198,9 +204,9 @@ struct Context {
     bool vl_valid = false;             // list, origins and cell maps describe the MD state
     cudaStream_t aux_stream = nullptr; // captures the body of the rebuild conditional
     int maps_n = -1;                   // atoms of the evaluation that last wrote the cell maps
-    // partials of the last potential evaluation (read by the MD reductions)
-    const double *last_epart = nullptr, *last_vpart = nullptr;
-    int last_eparts = 0, last_vparts = 0;
+    // partials of the last potential evaluation, and those that the captured MD step writes: a
+    // replay makes them the last again (frame 0 of its call may have taken another form)
+    Partials last, md_last;
 
     // Berendsen thermostat of the MD path (tau <= 0: NVE). d_lambda holds the
     // velocity scale of the next step, written by the closing kick.

@@ -331,10 +331,10 @@ int enqueue_potential(Context &c, const Grid &g, int n, int *n_eparts) {
         else
             CK(launch_fused_tc(c, g, n), "potential kernel (tensor-core network)");
         *n_eparts = c.pot_parts;
-        c.last_epart = c.d_e_part;
-        c.last_eparts = c.pot_parts;
-        c.last_vpart = c.d_vir_part;
-        c.last_vparts = c.pot_parts;
+        c.last.epart = c.d_e_part;
+        c.last.eparts = c.pot_parts;
+        c.last.vpart = c.d_vir_part;
+        c.last.vparts = c.pot_parts;
     } else {
         int rc = ensure_G(c, n, true);
         if (!rc && c.precision != AENET_FP32) rc = ensure_species(c, n);
@@ -350,8 +350,8 @@ int enqueue_potential(Context &c, const Grid &g, int n, int *n_eparts) {
         }
         CK(mark(c, 4), "event");
         if ((rc = enqueue_rows(c, g, n, RowsMode::forces))) return rc;
-        c.last_epart = c.d_e_part;
-        c.last_eparts = *n_eparts;
+        c.last.epart = c.d_e_part;
+        c.last.eparts = *n_eparts;
     }
     c.maps_n = n;          // the cell maps now describe this evaluation
     c.vl_valid = false;    // and no Verlet list matches them
@@ -1432,6 +1432,7 @@ static int md_fixed_cell(aenet_ctx *h, int n, double *pos, double *vel, const in
                         }
                     }
                 }
+                c.md_last = c.last;
                 c.last_list = list_form;
                 c.last_fused = fused_path(c);
                 c.last_rows = rows && !verlet;
@@ -1456,6 +1457,7 @@ static int md_fixed_cell(aenet_ctx *h, int n, double *pos, double *vel, const in
                "kick + reductions");
         } else {
             for (int s = 0; s < n_steps; ++s) CK(cudaGraphLaunch(exec, c.stream), "graph launch");
+            c.last = c.md_last;
         }
         c.maps_n = n;
         c.vl_valid = verlet;

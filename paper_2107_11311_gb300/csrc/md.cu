@@ -555,7 +555,7 @@ cudaError_t launch_finalize(Context &c, int n, int n_eparts, double *forces, dou
                             double *virial, bool to_host) {
     const int blocks = kReduceCtas + ((forces || e_atom) && n > 0 ? (n + kRedThreads - 1) / kRedThreads : 0);
     return launch_after(c.pdl, k_finalize, blocks, kRedThreads, 0, c.stream, n, c.d_perm, c.d_F4, c.d_eatom, n_eparts,
-                        c.last_epart, c.last_vparts, c.last_vpart, c.d_result, c.d_err,
+                        c.last.epart, c.last.vparts, c.last.vpart, c.d_result, c.d_err,
                         FinalizeOut{forces, e_atom, energy, virial, to_host ? c.h_res : nullptr});
 }
 
@@ -588,7 +588,7 @@ cudaError_t launch_batch_reduce(Context &c, bool atoms, double *energies, double
 static bool scan_folds(const Grid &g) { return g.ncell <= 4 * kMdThreads; }
 
 static MdSums md_sums(const Context &c, double *rec_pot, double *rec_kin) {
-    return MdSums{c.last_eparts, c.last_vparts, c.last_epart, c.last_vpart, c.d_ke_part, c.d_done,
+    return MdSums{c.last.eparts, c.last.vparts, c.last.epart, c.last.vpart, c.d_ke_part, c.d_done,
                   c.d_result,    c.d_step,      rec_pot,      rec_kin};
 }
 

@@ -174,9 +174,9 @@ cudaError_t launch_rows_potential(Context &c, const Grid &g, RowsMode mode, int 
     int got = 0;
     const cudaError_t e = AENET_BY_BASIS(c, launch_list, c, g, q, &got);
     *parts += got;
-    c.last_epart = c.d_vl_epart;
-    c.last_vpart = c.d_vl_vpart;
-    c.last_eparts = c.last_vparts = c.pot_parts = *parts;
+    c.last.epart = c.d_vl_epart;
+    c.last.vpart = c.d_vl_vpart;
+    c.last.eparts = c.last.vparts = c.pot_parts = *parts;
     c.last_grid = got;
     return e;
 }
@@ -191,9 +191,9 @@ cudaError_t launch_potential_list(Context &c, const Grid &g, int n) {
     q.a_hi = n;
     int parts = 0;
     if ((e = AENET_BY_BASIS(c, launch_list, c, g, q, &parts)) != cudaSuccess) return e;
-    c.last_epart = c.d_vl_epart;
-    c.last_vpart = c.d_vl_vpart;
-    c.last_eparts = c.last_vparts = parts;
+    c.last.epart = c.d_vl_epart;
+    c.last.vpart = c.d_vl_vpart;
+    c.last.eparts = c.last.vparts = parts;
     return cudaSuccess;
 }
 

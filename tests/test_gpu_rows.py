@@ -152,3 +152,23 @@ def test_slices_of_rows_give_what_one_slice_gives(gpu_mod, precision, hidden):
         else:
             x, y = np.asarray(x, dtype=np.float64), np.asarray(many[k], dtype=np.float64)
             assert np.sqrt(((x - y) ** 2).mean()) <= (5e-6 if k == "G" else tol) * np.sqrt((x ** 2).mean()), k
+
+
+@pytest.mark.parametrize("mode", ["off", "on", "auto"])
+@pytest.mark.parametrize("steps", [1, 3])
+def test_continued_md_records_the_frame_it_starts_from(gpu_mod, mode, steps):
+    """The third of three MD calls of the same shape (the second replays the first's
+    captured step) continues the second: its frame 0 is the second's last one. Two
+    reductions of the same FP32 numbers, so equal in every bit."""
+    st = inputs.water(64, None, 4)
+    m = inputs.make_model("water")
+    g = gpu_mod.AenetGPU(m, "fp32")
+    g.md_list(mode)
+    pos = torch.as_tensor(st.pos, device="cuda")
+    vel = torch.as_tensor(inputs.maxwell_boltzmann(m.masses[st.types], 300.0, seed=2), device="cuda")
+    types = torch.as_tensor(st.types, device="cuda")
+    e = [np.zeros(steps + 1) for _ in range(3)]
+    for k in range(3):
+        g.md_nve(pos, vel, types, st.box, 2.5e-4, steps, e[k], None, gpu_mod.AENET_MD_CONTINUE if k == 2 else 0)
+    assert abs(e[1][0] - e[1][-1]) > 1e-6
+    assert e[2][0] == e[1][-1]
