@@ -646,6 +646,9 @@ static int compute_impl(Context &c, int n, const double *pos, const int32_t *typ
             if ((rc = check_smem(c, g))) return rc;
             if ((rc = ensure_G(c, n, !G_dev))) return rc;
             const Overlap overlap(c);
+            // the sort and the cleared forces take the MD state with them
+            c.maps_n = -1;
+            c.vl_valid = false;
             CK(launch_cells(c, g, n, dpos, dtypes), "cell list");
             if ((rc = enqueue_rows(c, g, n, RowsMode::descriptor))) return rc;
             CK(launch_unsort_G(c, n, G_dev ? G_out : c.d_dEdG), "unsort");  // (host rows: the other row buffer first)

@@ -172,3 +172,25 @@ def test_continued_md_records_the_frame_it_starts_from(gpu_mod, mode, steps):
         g.md_nve(pos, vel, types, st.box, 2.5e-4, steps, e[k], None, gpu_mod.AENET_MD_CONTINUE if k == 2 else 0)
     assert abs(e[1][0] - e[1][-1]) > 1e-6
     assert e[2][0] == e[1][-1]
+
+
+@pytest.mark.parametrize("skin", [0.0, 0.5])
+def test_md_after_descriptors_starts_from_its_forces(gpu_mod, skin):
+    """Descriptors between two MD calls, the second, of one step, with AENET_MD_CONTINUE:
+    x1 = x0 + dt v0 + dt^2 / 2 F(x0) c / m, so the step shows the forces it started from.
+    They are those of a separate evaluation up to the order of FP32 sums: 5e-6 of the RMS."""
+    st = inputs.water(64, None, 4)
+    m = inputs.make_model("water")
+    g = gpu_mod.AenetGPU(m, "fp32")
+    g.set_skin(skin)
+    dt, mass = 2.5e-4, m.masses[st.types][:, None]
+    pos, vel = st.pos.copy(), inputs.maxwell_boltzmann(m.masses[st.types], 300.0, seed=2)
+    g.md_nve(pos, vel, st.types, st.box, dt, 4)
+    x0, v0 = pos.copy(), vel.copy()
+    g.descriptors(st.pos[::-1].copy(), st.types[::-1].copy(), st.box)
+    g.md_nve(pos, vel, st.types, st.box, dt, 1, flags=gpu_mod.AENET_MD_CONTINUE)
+    F = 2.0 * (pos - x0 - dt * v0) / dt ** 2 * mass / inputs.EV_PER_AMU
+    ref = gpu_mod.AenetGPU(m, "fp32").compute(x0, st.types, st.box)["forces"]
+    rms = np.sqrt((ref ** 2).mean())
+    assert rms > 0.1
+    assert np.sqrt(((F - ref) ** 2).mean()) <= 5e-6 * rms
