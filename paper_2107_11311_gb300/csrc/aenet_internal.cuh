@@ -176,9 +176,7 @@ struct Context {
     // MD steps without a skin: AENET_MD_LIST_AUTO (0), _OFF (1: the fused kernel searches the cells
     // itself) or _ON (2: the exact list is built in every step and the list kernel evaluates it)
     int md_list = 0;
-    bool last_list = false;            // the captured MD step takes the list form of AENET_OPT_MD_LIST
-    bool last_fused = false;           // the captured MD step runs a fused kernel
-    bool last_rows = false;            // ... or builds lists in every step as aenet_compute does
+    int md_path = 0;                   // AENET_PATH_* flags of the captured MD step
     // tilt factors xy, xz, yz of the restricted triclinic cell of single-structure
     // calls (zero: orthorhombic)
     double tilt[3] = {0.0, 0.0, 0.0};
@@ -277,14 +275,13 @@ struct Context {
         int nb = 0, ang = 0, tile = 0, vl_cap = 0;
         unsigned gen = 0;
         double skin = 0.0;
-        bool list_form = false;
         unsigned ev_mask = 0;
         double thermo_T0 = 0.0, thermo_tau = 0.0;
         bool operator==(const MdKey &o) const {
             return n == o.n && pos == o.pos && vel == o.vel && types == o.types && box[0] == o.box[0] &&
                    box[1] == o.box[1] && box[2] == o.box[2] && dt == o.dt && rec == o.rec && stream == o.stream &&
                    nb == o.nb && ang == o.ang && tile == o.tile && vl_cap == o.vl_cap && gen == o.gen &&
-                   skin == o.skin && list_form == o.list_form && ev_mask == o.ev_mask && thermo_T0 == o.thermo_T0 &&
+                   skin == o.skin && ev_mask == o.ev_mask && thermo_T0 == o.thermo_T0 &&
                    thermo_tau == o.thermo_tau;
         }
     };

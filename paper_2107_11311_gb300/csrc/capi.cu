@@ -1138,10 +1138,10 @@ extern "C" int aenet_descriptors(aenet_ctx *h, int n, const double *pos, const i
     return compute_impl(h->c, n, pos, types, box, nullptr, nullptr, nullptr, nullptr, G);
 }
 
-// Whether an MD step without a skin builds the exact neighbour list in every
-// step (AENET_OPT_MD_LIST): the FP32 fused form only, not the pipelined form;
-// automatic: every basis but the spherical-harmonic one (radial / angular
-// coefficient counts 21 / 7), whose fused kernel is the faster there.
+// Whether MD steps without a skin report AENET_PATH_LIST: the list form that
+// AENET_OPT_MD_LIST names (FP32 fused form, not pipelined). AUTO names it for every
+// basis but the spherical-harmonic one (radial / angular coefficient counts 21 / 7);
+// the steps of AUTO and ON run the same kernels for all of them (AENET_PATH_ROWS).
 static bool md_list_form(const Context &c) {
     if (c.skin > 0.0 || !fused_supported(c) || c.pipeline || c.md_list == AENET_MD_LIST_OFF) return false;
     if (c.md_list == AENET_MD_LIST_ON) return true;
@@ -1391,7 +1391,6 @@ static int md_fixed_cell(aenet_ctx *h, int n, double *pos, double *vel, const in
         key.vl_cap = c.caps.vl_cap;
         key.gen = c.buf_gen;
         key.skin = c.skin;
-        key.list_form = list_form;
         key.ev_mask = ev_mask;
         key.thermo_T0 = c.thermo_T0;
         key.thermo_tau = c.thermo_tau;
@@ -1404,6 +1403,7 @@ static int md_fixed_cell(aenet_ctx *h, int n, double *pos, double *vel, const in
             cudaGraph_t graph = nullptr;
             CK(cudaStreamBeginCapture(c.stream, cudaStreamCaptureModeThreadLocal), "begin capture");
             c.ev_mask = ev_mask;
+            c.last_pipe = false;
             int src;
             if (turn) {
                 const Overlap overlap(c);
@@ -1436,9 +1436,8 @@ static int md_fixed_cell(aenet_ctx *h, int n, double *pos, double *vel, const in
                     }
                 }
                 c.md_last = c.last;
-                c.last_list = list_form;
-                c.last_fused = fused_path(c);
-                c.last_rows = rows && !verlet;
+                c.md_path = (fused_path(c) ? AENET_PATH_FUSED : 0) | (c.last_pipe ? AENET_PATH_PIPELINED : 0) |
+                            (list_form ? AENET_PATH_LIST : 0) | (rows && !verlet ? AENET_PATH_ROWS : 0);
             }
             ce = cudaGraphInstantiate(&exec, graph, 0);
             cudaGraphDestroy(graph);
@@ -1601,9 +1600,7 @@ extern "C" int aenet_md_stage_times(aenet_ctx *h, float *ms, int *kernels_per_st
             ms[k] = nanf("");  // stage not recorded in the light timing mode
     }
     if (kernels_per_step) *kernels_per_step = c.md_kernels;
-    if (path_flags)
-        *path_flags = (c.last_fused ? AENET_PATH_FUSED : 0) | (c.last_pipe ? AENET_PATH_PIPELINED : 0) |
-                      (c.last_list ? AENET_PATH_LIST : 0) | (c.last_rows ? AENET_PATH_ROWS : 0);
+    if (path_flags) *path_flags = c.md_path;
     return AENET_OK;
 }
 

@@ -194,3 +194,17 @@ def test_md_after_descriptors_starts_from_its_forces(gpu_mod, skin):
     rms = np.sqrt((ref ** 2).mean())
     assert rms > 0.1
     assert np.sqrt(((F - ref) ** 2).mean()) <= 5e-6 * rms
+
+
+def test_path_flags_follow_the_last_captured_step(gpu_mod):
+    """Pipelined, then not, then over a Verlet list with the pipelined frame 0."""
+    st, m = inputs.water_192(), inputs.make_model("water")
+    vel = inputs.maxwell_boltzmann(m.masses[st.types], 300.0, seed=2)
+    g = gpu_mod.AenetGPU(m, "fp32")
+    got = []
+    for pipeline, skin in ((True, 0.0), (False, 0.0), (True, 0.5), (True, 0.5)):
+        g.pipeline(pipeline)
+        g.set_skin(skin)
+        g.md_nve(st.pos.copy(), vel.copy(), st.types, st.box, 5e-4, 2, flags=gpu_mod.AENET_MD_TIMING)
+        got.append(g.md_path_flags() & (gpu_mod.AENET_PATH_PIPELINED | gpu_mod.AENET_PATH_ROWS))
+    assert got == [gpu_mod.AENET_PATH_PIPELINED, gpu_mod.AENET_PATH_ROWS, 0, 0]
