@@ -71,10 +71,16 @@ struct Caps {
     int nb;     // entries with r <= rc_max
     int ang;    // entries with r <= rc_ang
     int tile;   // staged neighbour-cell atoms per chunk (fused kernel)
-    int vl_cap = 0;        // Verlet-list entries per atom (r <= rc_max + skin at the build)
+    int vl_cap = 0;        // Verlet-list entries per atom (r <= rc_max + skin at the build, and kRowSlack)
     int vl_jbits = 0;      // bits of the sorted atom index in an entry; the rest: image-offset code
     float rc_list = 0.f;   // rc_max + skin
 };
+
+// Entries of a list row beyond those an atom may have: the list build keeps the atom
+// itself and, by its rounding margin, now and then a pair just outside the cutoff. The
+// kernel that reads the row drops both, so an atom with exactly caps.nb neighbours fits.
+constexpr int kRowSlack = 8;
+inline int row_cap(const Caps &k) { return k.nb + kRowSlack; }
 
 struct Context {
     int device = 0;
@@ -189,7 +195,7 @@ struct Context {
     unsigned *d_vl_flag = nullptr;     // [2]: rebuild flag, last-CTA counter
     unsigned long long *d_vl_builds = nullptr;  // list builds so far
     // neighbour lists built for every evaluation (direct rows: displacement, index and species)
-    float4 *d_rows = nullptr;          // [atoms of a slice * caps.nb]
+    float4 *d_rows = nullptr;          // [atoms of a slice * row_cap(caps)]
     size_t cap_rows = 0;
     int *d_list_count = nullptr;       // [atoms]
     int cap_list = 0;

@@ -231,7 +231,7 @@ int ensure_parts(Context &c, int launches) {
 // Buffers of the evaluation over direct rows for n atoms with the capacities c.caps.
 int ensure_rows(Context &c, int n) {
     const int slice = list_slice(c, n);
-    const size_t need = (size_t)slice * c.caps.nb;
+    const size_t need = (size_t)slice * row_cap(c.caps);
     if (need > c.cap_rows || !c.d_rows) {
         c.cap_rows = 0;
         CK(grow(c.d_rows, 0, need), "cudaMalloc");
@@ -1248,7 +1248,7 @@ static int ensure_verlet(Context &c, int n, const Grid &g) {
     const double V = g.box[0] * g.box[1] * g.box[2];
     const double rl = c.caps.rc_list;
     const int need_cap =
-        std::max(64, (((int)(1.3 * (n / V) * 4.18879020478639 * rl * rl * rl + 32.0)) + 15) / 16 * 16);
+        std::max(64, (((int)(1.3 * (n / V) * 4.18879020478639 * rl * rl * rl + 32.0)) + 15) / 16 * 16) + kRowSlack;
     if (c.caps.vl_cap < need_cap) c.caps.vl_cap = need_cap;
     c.caps.vl_jbits = jbits;
     const size_t N = (size_t)std::max(n, 1);

@@ -10,7 +10,7 @@ namespace {
 using namespace detail;
 
 // Direct rows of one slice of atoms are limited to this many bytes; more atoms are
-// evaluated in slices (water: 466,000 atoms a slice; a slice's last atoms leave a
+// evaluated in slices (water: 441,000 atoms a slice; a slice's last atoms leave a
 // few warps busy for about 10 us of its 1.5 ms).
 constexpr size_t kMaxRowBytes = size_t(1) << 30;
 
@@ -36,7 +36,7 @@ cudaError_t launch_build(Context &c, const Grid &g, int n, int a_lo, int a_hi, b
     return launch_after(
         c.pdl, kern, ctas, kBuildThreads, smem, c.stream, g, c.batch_sinfo, c.batch_n,
         codes ? c.caps.rc_list : c.basis.rc_max, tile, parts, a_lo, a_hi, c.d_pos4,
-        c.d_cell_start, c.d_rows, c.d_vl, codes ? c.caps.vl_cap : c.caps.nb, c.caps.vl_jbits,
+        c.d_cell_start, c.d_rows, c.d_vl, codes ? c.caps.vl_cap : row_cap(c.caps), c.caps.vl_jbits,
         codes ? c.d_vl_count : c.d_list_count, clear ? c.d_F4 : nullptr, clear ? c.d_stats : nullptr, c.d_err);
 }
 
@@ -76,7 +76,7 @@ cudaError_t launch_list(Context &c, const Grid &g, const ListLaunch &q, int *par
     constexpr int most = list_max_warps<KRT, KAT, EXACT>();
     constexpr bool sh = sh_angular<KRT, KAT, EXACT>();
     Caps caps = c.caps;
-    if (!q.codes) caps.vl_cap = caps.nb;
+    if (!q.codes) caps.vl_cap = row_cap(caps);
     const ListLayout L = make_list_layout(q.codes ? g.n_off : 0, caps.nb, caps.ang, fused ? c.basis.n_species : 0,
                                           net.stride, sh, 1);
     const int n = q.a_hi - q.a_lo;
@@ -148,7 +148,7 @@ size_t list_smem_bytes(const Context &c) { return AENET_BY_BASIS(c, list_smem, c
 
 // Atoms of one slice of direct rows.
 int list_slice(const Context &c, int n) {
-    const size_t most = std::max<size_t>(1, kMaxRowBytes / (sizeof(float4) * (size_t)std::max(1, c.caps.nb)));
+    const size_t most = std::max<size_t>(1, kMaxRowBytes / (sizeof(float4) * (size_t)std::max(1, row_cap(c.caps))));
     return (int)std::min<size_t>((size_t)std::max(1, n), most);
 }
 

@@ -121,7 +121,7 @@ def test_lists_that_leave_room_for_few_warps(gpu_mod, n):
 @pytest.mark.parametrize("precision,hidden", [("fp32", (15, 15)), ("bf16x3", (15, 15)), ("fp32", (48, 48))])
 def test_slices_of_rows_give_what_one_slice_gives(gpu_mod, precision, hidden):
     """24,000 atoms after a structure so dense (two atoms in 0.73 A^3) that the lists it
-    sizes fill a slice of rows with 20,560 atoms, against a context that never saw it:
+    sizes fill a slice of rows with some 20,500 atoms, against a context that never saw it:
     the fused, the three-kernel and the wide FP32 path, descriptors and a batch. Sums in
     another order, in FP32: a few units of 2^-24 of an atom's terms, 5e-6 of the RMS;
     through the split-BF16 network, whose products drop 2^-16 of a factor, 1e-4."""
@@ -208,3 +208,33 @@ def test_path_flags_follow_the_last_captured_step(gpu_mod):
         g.md_nve(st.pos.copy(), vel.copy(), st.types, st.box, 5e-4, 2, flags=gpu_mod.AENET_MD_TIMING)
         got.append(g.md_path_flags() & (gpu_mod.AENET_PATH_PIPELINED | gpu_mod.AENET_PATH_ROWS))
     assert got == [gpu_mod.AENET_PATH_PIPELINED, gpu_mod.AENET_PATH_ROWS, 0, 0]
+
+
+def _shell(n, radius):
+    """n atoms spread over a sphere (a golden spiral): all within its diameter of one another."""
+    k = np.arange(n) + 0.5
+    z, a = 1.0 - 2.0 * k / n, np.pi * (1.0 + 5.0 ** 0.5) * k
+    s = np.sqrt(1.0 - z * z)
+    return radius * np.stack([s * np.cos(a), s * np.sin(a), z], 1)
+
+
+@pytest.mark.parametrize("skin", [0.0, 0.5])
+def test_an_atom_may_have_as_many_neighbours_as_its_list(gpu_mod, skin):
+    """65 atoms with exactly 64 neighbours each, the capacity that a sparse system's first
+    call sets: an asynchronous evaluation, which cannot regrow it, and MD."""
+    pos, box = _shell(65, 2.98) + 20.0, np.full(3, 40.0)
+    r = np.linalg.norm(pos[:, None] - pos[None], axis=2)
+    assert r.max() < 6.0 and ((r < 4.0).sum(1) - 1).max() <= 32
+    types = (np.arange(65) % 3 > 0).astype(np.int32)
+    m = inputs.make_model("water")
+    ref = O.compute(m, pos, types, box)
+    g = gpu_mod.AenetGPU(m, "fp32")
+    g.compute(pos[:2], types[:2], box)
+    p, t = torch.as_tensor(pos, device="cuda"), torch.as_tensor(types, device="cuda")
+    F = torch.zeros((65, 3), dtype=torch.float64, device="cuda")
+    g.compute_async(p, t, box, forces=F)
+    g.check()
+    rms = np.sqrt((ref["forces"] ** 2).mean())
+    assert np.sqrt(((F.cpu().numpy() - ref["forces"]) ** 2).mean()) <= max(1e-4, 2e-5 * rms)
+    g.set_skin(skin)
+    g.md_nve(p, torch.zeros_like(p), t, box, 1e-6, 2)
