@@ -238,3 +238,72 @@ def test_an_atom_may_have_as_many_neighbours_as_its_list(gpu_mod, skin):
     assert np.sqrt(((F.cpu().numpy() - ref["forces"]) ** 2).mean()) <= max(1e-4, 2e-5 * rms)
     g.set_skin(skin)
     g.md_nve(p, torch.zeros_like(p), t, box, 1e-6, 2)
+
+
+@pytest.mark.parametrize("n", [4096, 4097])
+def test_host_and_device_arrays_mixed(gpu_mod, n):
+    """Both sides of the size up to which host arrays go through mapped memory, every
+    array in turn on the host and on the device, against the call with all of them on the
+    device: the same sums in FP32 in another order, 5e-6 of the RMS."""
+    st = inputs.amorphous(n, seed=11)
+    g = gpu_mod.AenetGPU(inputs.make_model("amorphous"), "fp32")
+    shapes = {"energy": (1,), "forces": (n, 3), "virial": (3, 3), "e_atom": (n,)}
+
+    def arrays(host):
+        given = [torch.as_tensor(st.pos), torch.as_tensor(st.types)]
+        given = [x.numpy() if k in host else x.cuda() for k, x in zip(("pos", "types"), given)]
+        out = {k: np.zeros(s) if k in host else torch.zeros(s, dtype=torch.float64, device="cuda")
+               for k, s in shapes.items()}
+        g.compute(*given, st.box, **out)
+        return {k: np.array(v) if k in host else v.cpu().numpy() for k, v in out.items()}
+
+    ref = arrays(())
+    for host in (("pos",), ("types",), ("forces",), ("e_atom", "energy"), ("virial",), ("pos", "types", "e_atom"),
+                 ("pos", "types", "energy", "forces", "virial", "e_atom")):
+        for k, x in arrays(host).items():
+            assert np.sqrt(((x - ref[k]) ** 2).mean()) <= 5e-6 * np.sqrt((ref[k] ** 2).mean()), (host, k)
+
+
+@pytest.mark.parametrize("family,n", [("water", 4095), ("water", 4098), ("amorphous", 1024), ("amorphous", 1025)])
+def test_split_bf16_on_both_sides_of_the_fused_sizes(gpu_mod, family, n):
+    """Energies, forces and the weight gradient where the fused tensor-core kernel gives way
+    to the three kernels, against the FP32 form. The split drops 2^-16 of a factor: 1e-4
+    of the RMS (E_i, forces); 1e-3 of the largest gradient, a sum over all atoms whose
+    terms partly cancel."""
+    st = inputs.water(n // 3, None, 7) if family == "water" else inputs.amorphous(n, seed=7)
+    m = inputs.make_model(family)
+    res = {}
+    for precision in ("fp32", "bf16x3"):
+        g = gpu_mod.AenetGPU(m, precision)
+        g.keep_activations(True)
+        res[precision] = dict(g.compute(st.pos, st.types, st.box), dEdW=g.grad_weights())
+    a, b = res["fp32"], res["bf16x3"]
+    for k in ("e_atom", "forces"):
+        assert np.sqrt(((a[k] - b[k]) ** 2).mean()) <= 1e-4 * np.sqrt((a[k] ** 2).mean()), k
+    assert np.abs(a["dEdW"] - b["dEdW"]).max() <= 1e-3 * np.abs(a["dEdW"]).max()
+
+
+@pytest.mark.parametrize("box", [None, 70.0])
+def test_md_turn_equals_single_steps(gpu_mod, box):
+    """Four steps in one call (one kernel between two potentials) against four calls of one
+    step, on a grid that the turn scans itself and on one of 1,331 cells that it leaves to
+    the scan kernel. The FP64 steps are the same; the forces differ by the order of their
+    FP32 sums, 5e-6 of the largest: positions by that acceleration over four steps."""
+    st = inputs.water(512, box, 8)
+    m = inputs.make_model("water")
+    dt, mass = 2.5e-4, m.masses[st.types][:, None]
+    v0 = inputs.maxwell_boltzmann(m.masses[st.types], 300.0, seed=2)
+    g = gpu_mod.AenetGPU(m, "fp32")
+    a = np.abs(g.compute(st.pos, st.types, st.box)["forces"] / mass).max() * inputs.EV_PER_AMU
+    many, e = (st.pos.copy(), v0.copy()), (np.zeros(5), np.zeros(5))
+    g.md_nve(*many, st.types, st.box, dt, 4, *e)
+    one, e_pot, e_kin = (st.pos.copy(), v0.copy()), [], []
+    for k in range(4):
+        ep, ek = np.zeros(2), np.zeros(2)
+        g.md_nve(*one, st.types, st.box, dt, 1, ep, ek, gpu_mod.AENET_MD_CONTINUE if k else 0)
+        e_pot += list(ep if k == 0 else ep[1:])
+        e_kin += list(ek if k == 0 else ek[1:])
+    assert np.abs(many[0] - one[0]).max() <= 5e-6 * a * (4 * dt) ** 2
+    assert np.abs(many[1] - one[1]).max() <= 5e-6 * a * 4 * dt
+    np.testing.assert_allclose(e[0], e_pot, atol=2e-6 * st.n)
+    np.testing.assert_allclose(e[1], e_kin, rtol=1e-5)
