@@ -739,7 +739,7 @@ struct BatchCall {
 
 struct BatchLayout {
     std::vector<StructInfo> info;  // per structure
-    std::vector<int> order;        // cells, heaviest first
+    std::vector<int> order;        // cells, heaviest first (BF16 forms: the fused tensor-core kernel)
     Grid gall{};                   // ncell = all cells, n_off = largest image table
     int n = 0;                     // atoms
     double max_rho = 0.0, max_neigh = 0.0;
@@ -781,6 +781,8 @@ int batch_layout(Context &c, int n_struct, const int64_t *atom_offset, const dou
     L.gall = Grid{};
     L.gall.ncell = total_cells;
     L.gall.n_off = max_off;
+    // (FP32 batches go over lists, whose kernel takes atoms from a counter: they need no order)
+    if (c.precision == AENET_FP32) return AENET_OK;
     L.order.resize((size_t)total_cells);
     std::vector<int> sorder((size_t)n_struct);
     for (int s = 0; s < n_struct; ++s) sorder[s] = s;
@@ -870,15 +872,16 @@ extern "C" int aenet_compute_batch(aenet_ctx *h, int n_struct, const int64_t *at
         c.cap_struct = n_struct;
         ++c.buf_gen;
     }
-    if ((rc = grow_order(c, L.gall.ncell))) return rc;
+    if (!L.order.empty() && (rc = grow_order(c, L.gall.ncell))) return rc;
     const double *dpos;
     const int32_t *dtypes;
     if ((rc = stage_in(c, pos, c.d_pos, 3 * (size_t)n, &dpos))) return rc;
     if ((rc = stage_in(c, types, c.d_types, (size_t)n, &dtypes))) return rc;
     CK(cudaMemcpyAsync(c.d_sinfo, L.info.data(), sizeof(StructInfo) * n_struct, cudaMemcpyHostToDevice, c.stream),
        "cudaMemcpyAsync");
-    CK(cudaMemcpyAsync(c.d_order, L.order.data(), sizeof(int) * L.order.size(), cudaMemcpyHostToDevice, c.stream),
-       "cudaMemcpyAsync");
+    if (!L.order.empty())
+        CK(cudaMemcpyAsync(c.d_order, L.order.data(), sizeof(int) * L.order.size(), cudaMemcpyHostToDevice, c.stream),
+           "cudaMemcpyAsync");
     const bool f_dev = is_device_ptr(forces);
     double *dF = forces ? (f_dev ? forces : c.d_forces) : nullptr;
     const bool persist = c.persist;
@@ -994,11 +997,12 @@ extern "C" int aenet_batch_prepare(aenet_ctx *h, int n_struct, const int64_t *at
     c.d_psinfo = nullptr;
     c.d_porder = nullptr;
     CK(cudaMalloc(&c.d_psinfo, sizeof(StructInfo) * (size_t)n_struct), "cudaMalloc");
-    CK(cudaMalloc(&c.d_porder, sizeof(int) * std::max<size_t>(1, L.order.size())), "cudaMalloc");
+    if (!L.order.empty()) CK(cudaMalloc(&c.d_porder, sizeof(int) * L.order.size()), "cudaMalloc");
     CK(cudaMemcpyAsync(c.d_psinfo, L.info.data(), sizeof(StructInfo) * n_struct, cudaMemcpyHostToDevice, c.stream),
        "cudaMemcpyAsync");
-    CK(cudaMemcpyAsync(c.d_porder, L.order.data(), sizeof(int) * L.order.size(), cudaMemcpyHostToDevice, c.stream),
-       "cudaMemcpyAsync");
+    if (!L.order.empty())
+        CK(cudaMemcpyAsync(c.d_porder, L.order.data(), sizeof(int) * L.order.size(), cudaMemcpyHostToDevice, c.stream),
+           "cudaMemcpyAsync");
     CK(cudaStreamSynchronize(c.stream), "cudaStreamSynchronize");
     c.plan.n_struct = n_struct;
     c.plan.n_atoms = n;
