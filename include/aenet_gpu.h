@@ -266,7 +266,9 @@ int aenet_batch_run(aenet_ctx *ctx);
 /*
  * The launch aenet_batch_prepare chose: persistent (1) or one CTA per cell
  * (0), staging tile, CTAs of the potential launch, kernel nodes in the
- * captured graph, and the measured time of one evaluation (ms). Any output
+ * captured graph (over lists, that is for FP32 and the three-kernel BF16 path,
+ * the list kernel is always persistent and the tile is the list build's),
+ * and the measured time of one evaluation (ms). Any output
  * may be NULL. AENET_E_STATE without a prepared batch.
  */
 int aenet_batch_tuning(aenet_ctx *ctx, int *persistent, int *tile, int *ctas, int *kernels, float *ms);
@@ -426,11 +428,11 @@ int aenet_descriptors_noalloc(int n_atoms, const double *pos, const int32_t *typ
  * fused potential kernel itself from the staged cells (OFF) or by a list
  * kernel that writes each atom's exact list after the binning, which the
  * list-driven potential kernel then reads (ON). The same pairs enter the same
- * sums, so the two agree to FP32 rounding order. AUTO takes ON for every basis
- * except angular order 6 with radial order 20, whose steps evaluate as
- * aenet_compute does: over lists as well (AENET_PATH_ROWS). aenet_compute
- * builds its lists in every call, whatever this option says. A change
- * re-captures the MD step. Other values give AENET_E_ARG.
+ * sums, so the two agree to FP32 rounding order. AUTO runs the same kernels as
+ * ON (AENET_PATH_ROWS); for angular order 6 with radial order 20 it does not
+ * report AENET_PATH_LIST, the name of an earlier list form. aenet_compute and
+ * the frame that an MD call starts from build their lists whatever this option
+ * says. A change re-captures the MD step. Other values give AENET_E_ARG.
  */
 #define AENET_OPT_MD_LIST 4
 #define AENET_MD_LIST_AUTO 0

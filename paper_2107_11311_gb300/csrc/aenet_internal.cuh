@@ -176,7 +176,7 @@ struct Context {
 
     // Verlet neighbour list with a skin (MD steps of the fused FP32 form; skin 0 =
     // the cell list every step). Entries: sorted index | image-offset code << jbits,
-    // built by k_potential's list mode, rebuilt inside the captured step (a graph
+    // built by k_list_build (code rows), rebuilt inside the captured step (a graph
     // conditional node) whenever an atom moved more than skin/2 since the build.
     double skin = 0.0;
     // MD steps without a skin: AENET_MD_LIST_AUTO (0), _OFF (1: the fused kernel searches the cells
@@ -385,10 +385,15 @@ inline bool fused_path(const Context &c) { return fused_supported(c) || tc_fused
 // its one launch wins where launches count, the three kernels over neighbour lists
 // where the chip is full. Split BF16, one evaluation, fused against three kernels
 // (us): water 1,536 77 / 103, 3,072 121 / 124, 6,144 142 / 133, 12,288 188 / 160,
-// 98,304 920 / 627, 331,776 2955 / 1929; the solid's cells hold more work per
-// atom: 2,000 189 / 135, 27,000 668 / 367.
+// 98,304 920 / 627, 331,776 2955 / 1929; device calls in a row, water 192 42 / 66,
+// 384 82 / 75, 768 76 / 77, 1,536 55 / 75, 3,072 89 / 91, 4,095 105 / 102.
+// The solid's cells hold more work per atom, and its fused time goes by how the
+// cells fill the chip: 32 82 / 93, 64 97 / 85, 128 186 / 94, 256 481 / 116, 512 123 /
+// 91, 700 162 / 99, 1,024 80 / 95, 2,000 189 / 135, 27,000 668 / 367. So its line is
+// the largest size at which the fused form is known to win, not a crossover: between
+// 64 and 1,000 atoms the three kernels (AENET_OPT_FUSED_NETWORK 0) are the faster.
 constexpr int kTcFusedAtoms = 4096, kTcFusedAtomsSolid = 1024;
-// Whether evaluations take that form: the FP32 fused form, except (for one
+// Whether evaluations go over neighbour rows: the FP32 fused form, except (for one
 // structure) the pipelined kernel and MD steps asked to search the cells in the
 // fused kernel.
 inline bool rows_form(const Context &c) {

@@ -61,10 +61,11 @@ __host__ __device__ inline BuildLayout make_build_layout(int n_off, int tile) {
 //     are taken in chunks.
 //  2. Each warp tests the staged atoms against three atoms at a time (whole
 //     evaluation: water 12,288 atoms, two at 12 CTAs per SM 94 us, three at 10
-//     91 us; water 98,304, four at 8 515 us, two at 12 507 us). With t = |p|^2 - 2 p.u the test is t <= rc^2 - |u|^2, three FMAs per pair;
-//     its rounding is covered by a margin (the potential kernel applies the
-//     exact cutoff to the displacement). The atom itself passes the test and
-//     is dropped there too.
+//     91 us; water 98,304, four at 8 515 us, two at 12 507 us). With
+//     t = |p|^2 - 2 p.u the test is t <= rc^2 - |u|^2, three FMAs per pair; its
+//     rounding is covered by a margin (the potential kernel applies the exact
+//     cutoff to the displacement). The atom itself passes the test and is
+//     dropped there too (kRowSlack).
 // It also clears the atoms' force accumulators and the neighbour statistics (F4
 // and stats, when given).
 template <bool BATCH, bool CODES>
@@ -1114,11 +1115,11 @@ struct ListSums {
 template <int KRT, int KAT, bool EXACT, int MODE, int HB, bool CODES, bool BATCH>
 __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
     k_potential_list(Basis B, FusedNet net, Grid g, Caps caps, int a_lo, int a_hi, const float4 *pos4,
-                     const float4 *rows, const int *codes, const int *count, const float *__restrict__ pnet, float4 *__restrict__ F4, float *__restrict__ eatom,
-                     float *__restrict__ G_out, const float *dEdG_in, double *__restrict__ e_part,
-                     double *__restrict__ vir_part, float *__restrict__ vir_atom,
-                     unsigned long long *__restrict__ stats, unsigned *__restrict__ err,
-                     unsigned *__restrict__ work) {
+                     const float4 *rows, const int *codes, const int *count, const float *__restrict__ pnet,
+                     float4 *__restrict__ F4, float *__restrict__ eatom, float *__restrict__ G_out,
+                     const float *dEdG_in, double *__restrict__ e_part, double *__restrict__ vir_part,
+                     float *__restrict__ vir_atom, unsigned long long *__restrict__ stats,
+                     unsigned *__restrict__ err, unsigned *__restrict__ work) {
     constexpr bool kSh = sh_angular<KRT, KAT, EXACT>();
     constexpr int NW = list_max_warps<KRT, KAT, EXACT>();
     extern __shared__ __align__(16) unsigned char smem[];

@@ -1268,8 +1268,8 @@ __global__ void __launch_bounds__(NW * 32, NW == kPWarps ? 2 : 1)
     const int tile = caps.tile;
     // one layout for every cell: sized for the largest image-offset table
     // (g_one.n_off is that maximum in a batch)
-    const PLayout L = make_playout(g_one.n_off, tile, caps.nb, caps.ang, (MODE == kFused || kTC) ? B.n_species : 0, kTC ? kTcParStride : net.stride, NW,
-                                   kTC);
+    const PLayout L = make_playout(g_one.n_off, tile, caps.nb, caps.ang, (MODE == kFused || kTC) ? B.n_species : 0,
+                                   kTC ? kTcParStride : net.stride, NW, kTC);
     int *off_start = reinterpret_cast<int *>(smem + L.off_start);
     int *off_count = reinterpret_cast<int *>(smem + L.off_count);
     int *off_prefix = reinterpret_cast<int *>(smem + L.off_prefix);

@@ -103,9 +103,10 @@ cudaError_t launch_list(Context &c, const Grid &g, const ListLaunch &q, int *par
     float *out = fused ? (c.keep_act ? c.d_act : nullptr) : c.d_G;  // activation records or G rows
     *parts = grid;
     return launch_after(
-        c.pdl, kern, grid, nw * 32, L.warp_base + L.warp_bytes * nw, c.stream, c.basis, net, g, caps, q.a_lo, q.a_hi, c.d_pos4, c.d_rows, c.d_vl, q.codes ? c.d_vl_count : c.d_list_count,
-        c.d_pnet, c.d_F4, c.d_eatom, out, c.d_dEdG, c.d_vl_epart + q.part0, c.d_vl_vpart + 9 * (size_t)q.part0,
-        c.d_vir_atom, c.d_stats, c.d_err, c.d_work);
+        c.pdl, kern, grid, nw * 32, L.warp_base + L.warp_bytes * nw, c.stream, c.basis, net, g, caps, q.a_lo, q.a_hi,
+        c.d_pos4, c.d_rows, c.d_vl, q.codes ? c.d_vl_count : c.d_list_count, c.d_pnet, c.d_F4, c.d_eatom, out,
+        c.d_dEdG, c.d_vl_epart + q.part0, c.d_vl_vpart + 9 * (size_t)q.part0, c.d_vir_atom, c.d_stats, c.d_err,
+        c.d_work);
 }
 
 template <int KRT, int KAT, bool EXACT>
