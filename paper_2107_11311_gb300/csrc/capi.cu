@@ -261,13 +261,15 @@ int ensure_eval(Context &c, int n) {
     return rc;
 }
 
-int check_smem(Context &c, const Grid &g) {
+// (codes: the list kernel over a Verlet list, which also holds its image table)
+int check_smem(Context &c, const Grid &g, bool codes = false) {
     int dev = 0, optin = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     // + the kernel's static shared memory
     const bool rows = rows_form(c) || !fused_path(c);
-    const size_t need = rows ? list_smem_bytes(c) + 4096 : potential_smem_bytes(c, g) + 1024;
+    const size_t need = (rows ? list_smem_bytes(c) + 4096 : potential_smem_bytes(c, g) + 1024) +
+                        (codes ? sizeof(float4) * (size_t)g.n_off : 0);
     if (optin > 0 && need > (size_t)optin)
         return fail(&c, AENET_E_CAPACITY, "neighbour lists need %zu B of shared memory (limit %d B)", need, optin);
     return AENET_OK;
@@ -1188,7 +1190,7 @@ static int enqueue_md_step(Context &c, const Grid &g, int n, double dt, double *
 // list, and the closing kick with the reductions. Events bracket the stages.
 static int enqueue_md_step_verlet(Context &c, const Grid &g, int n, double dt, double *pos, double *vel,
                                   const int32_t *types, double *rec) {
-    int rc = check_smem(c, g);
+    int rc = check_smem(c, g, true);
     if (rc) return rc;
     cudaStreamCaptureStatus status;
     cudaGraph_t graph = nullptr;

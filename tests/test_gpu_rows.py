@@ -307,3 +307,18 @@ def test_md_turn_equals_single_steps(gpu_mod, box):
     assert np.abs(many[1] - one[1]).max() <= 5e-6 * a * 4 * dt
     np.testing.assert_allclose(e[0], e_pot, atol=2e-6 * st.n)
     np.testing.assert_allclose(e[1], e_kin, rtol=1e-5)
+
+
+def test_verlet_lists_without_room_are_a_capacity_error(gpu_mod):
+    """Five atoms in 1 A^3: one warp's lists fit a CTA, with the 3,375 image offsets of the
+    Verlet list's grid beside them they do not."""
+    m = inputs.make_model("water")
+    g = gpu_mod.AenetGPU(m, "fp32")
+    pos = np.array([[0.1, 0.1, 0.1], [0.6, 0.6, 0.1], [0.6, 0.1, 0.6], [0.1, 0.6, 0.6], [0.35, 0.35, 0.35]])
+    types, box = np.array([0, 1, 1, 0, 1], np.int32), np.full(3, 1.0)
+    g.set_skin(0.5)
+    with pytest.raises(gpu_mod.AenetError) as e:
+        g.md_nve(pos.copy(), np.zeros((5, 3)), types, box, 1e-6, 2)
+    assert e.value.code == -3
+    g.set_skin(0.0)
+    g.md_nve(pos.copy(), np.zeros((5, 3)), types, box, 1e-6, 2)
