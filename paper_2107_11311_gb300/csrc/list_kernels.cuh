@@ -1484,21 +1484,16 @@ __global__ void __launch_bounds__(32 * list_max_warps<KRT, KAT, EXACT>(), 1)
                                     dup2(0.f), dup2(0.f), dup2(0.f)};
             const float2 t = reduce8(sums, W.red, lane);
             const int o = reduce8_order(lane);
-            float *f = reinterpret_cast<float *>(F4 + a);
-            if ((lane & 12) == 0) {
-                if (o == 0) {
-                    atomicAdd(f, t.x);
-                    atomicAdd(f + 1, t.y);
-                } else if (o == 1) {
-                    atomicAdd(f + 2, t.x);
-                } else if (o < 5) {
-                    if constexpr (BATCH) {
-                        *reinterpret_cast<float2 *>(vir_atom + (size_t)a * 6 + 2 * (o - 2)) = t;
-                    } else {
-                        double *v = s_sum.vir[warp] + 2 * (o - 2);
-                        v[0] += (double)t.x;
-                        v[1] += (double)t.y;
-                    }
+            // (one vector atomic; three scalar ones: water 331,776 1% slower)
+            const float tz = __shfl_sync(kFull, t.x, 16);  // order 1
+            if (lane == 0) atomicAdd(&F4[a], make_float4(t.x, t.y, tz, 0.f));
+            if ((lane & 12) == 0 && o > 1 && o < 5) {
+                if constexpr (BATCH) {
+                    *reinterpret_cast<float2 *>(vir_atom + (size_t)a * 6 + 2 * (o - 2)) = t;
+                } else {
+                    double *v = s_sum.vir[warp] + 2 * (o - 2);
+                    v[0] += (double)t.x;
+                    v[1] += (double)t.y;
                 }
             }
         }
